@@ -33,6 +33,7 @@ struct gt_ctx {
     int cam_valid = 0;
     int cam_flags = -1;
     double cam_rsw = -2.0;
+    gt::PairSpacetime cam_pair = {}; // the camera's double-float constants as set up on the device
     // batch descriptors (device)
     CamDesc *d_batch = nullptr;
     int batch_cap = 0;
@@ -170,6 +171,7 @@ int prepare_camera(gt_ctx *c)
     if (err == cudaSuccess) err = cudaStreamSynchronize(c->stream);
     if (err != cudaSuccess) return cuda_code(err);
     c->cam_valid = d.valid;
+    c->cam_pair = d.pair;
     c->cam_dirty = false;
     c->cam_flags = e.flags;
     c->cam_rsw = e.r_switch;
@@ -218,8 +220,9 @@ int build_mixed_graph(gt_ctx *c, const gt::TraceArgs &base, int kind_hint, const
     gt::ParkItem *listA = c->d_park, *listB = c->d_park + c->park_cap;
     unsigned long long *w = c->d_scratch;
     int grid32 = 0, grid64 = 0;
+    const int zone = base.zone_df ? gt::KMODE_ZONE_PAIR : gt::KMODE_ZONE_FP64;
     rc = grid_for(c, e, gt::KMODE_MIXED_FP32, kind_hint, base.n_rays, false, &grid32);
-    if (rc == GT_OK) rc = grid_for(c, e, gt::KMODE_ZONE_FP64, kind_hint, base.n_rays, false, &grid64);
+    if (rc == GT_OK) rc = grid_for(c, e, zone, kind_hint, base.n_rays, false, &grid64);
     if (rc != GT_OK) return rc;
     cudaGraph_t g = nullptr;
     cudaGraphConditionalHandle h;
@@ -281,7 +284,7 @@ int build_mixed_graph(gt_ctx *c, const gt::TraceArgs &base, int kind_hint, const
         a.out_items = listB;
         a.out_count = w + gt::SCR_TO32;
         if (e1 == cudaSuccess)
-            e1 = gt::launch_trace(a, gt::KMODE_ZONE_FP64, kind_hint, e.block_size, grid64, false, cs);
+            e1 = gt::launch_trace(a, zone, kind_hint, e.block_size, grid64, false, cs);
         if (e1 == cudaSuccess) e1 = cudaMemsetAsync(w + gt::SCR_NEXT_RAY, 0, W8, cs);
         if (e1 == cudaSuccess) e1 = cudaMemsetAsync(w + gt::SCR_TO64, 0, W8, cs);
         a.in_items = listB;
@@ -341,10 +344,10 @@ int run_mixed_rounds(gt_ctx *c, gt::TraceArgs &a, int kind_hint, const gt_option
         if (err == cudaSuccess)
             err = cudaMemsetAsync(w + gt::SCR_TO32, 0, sizeof(unsigned long long), c->stream);
         if (err != cudaSuccess) return cuda_code(err);
-        rc = grid_for(c, e, gt::KMODE_ZONE_FP64, kind_hint, (int64_t)parked, one_shot, &grid);
+        const int zone = a.zone_df ? gt::KMODE_ZONE_PAIR : gt::KMODE_ZONE_FP64;
+        rc = grid_for(c, e, zone, kind_hint, (int64_t)parked, one_shot, &grid);
         if (rc != GT_OK) return rc;
-        err = gt::launch_trace(a, gt::KMODE_ZONE_FP64, kind_hint, e.block_size, grid, one_shot,
-                               c->stream);
+        err = gt::launch_trace(a, zone, kind_hint, e.block_size, grid, one_shot, c->stream);
         if (err != cudaSuccess) return cuda_code(err);
         // FP32 continuation: B -> (A, finished)
         a.in_items = listB;
@@ -367,7 +370,8 @@ int run_trace(gt_ctx *c, const CamDesc *d_cams, int n_cams, int kind_hint, int64
               int64_t n_rays, int64_t n_steps, double sp, int mode, double *t, double *r,
               double *th, double *ph, uint8_t *status, uint32_t *nsteps,
               const int64_t *fresh_ids = nullptr, const gt::RayParams *d_rays = nullptr,
-              bool compact_out = false, const Extra &x = Extra())
+              bool compact_out = false, const Extra &x = Extra(), bool range_ok = true,
+              const gt::PairSpacetime *pair = nullptr)
 {
     const gt_options e = effective(c->opts);
     if ((e.flags & PAPER_FLAGS) && mode != GT_MODE_FP64) return GT_ERR_INVALID_ARG;
@@ -402,16 +406,21 @@ int run_trace(gt_ctx *c, const CamDesc *d_cams, int n_cams, int kind_hint, int64
     a.disk = x.disk;
     a.z = x.z;
     a.states = x.states;
+    if (pair) {
+        a.pair = *pair;
+        a.pair_single = 1;
+    }
     cudaError_t err =
         cudaMemsetAsync(c->d_scratch, 0, gt::SCR_WORDS * sizeof(unsigned long long), c->stream);
     if (err != cudaSuccess) return cuda_code(err);
     const bool one_shot = (e.flags & GT_FLAG_ONE_SHOT) != 0;
+    const int kmode64 = gt::fp64_kmode(a, kind_hint, range_ok);
     int rc;
     if (e.flags & GT_FLAG_GRAPH) {
         // the launch replayed from a CUDA graph, captured once per distinct launch and
         // cached: FP64 is one persistent launch; FP32-mixed is its rounds under a WHILE
         // node whose condition the device sets from the park count
-        const int kmode = mode == GT_MODE_FP64 ? gt::KMODE_FP64 : gt::KMODE_MIXED_FP32;
+        const int kmode = mode == GT_MODE_FP64 ? kmode64 : gt::KMODE_MIXED_FP32;
         if (one_shot) return GT_ERR_INVALID_ARG; // graphs replay the persistent launch
         int grid;
         rc = grid_for(c, e, kmode, kind_hint, n_rays, one_shot, &grid);
@@ -429,7 +438,7 @@ int run_trace(gt_ctx *c, const CamDesc *d_cams, int n_cams, int kind_hint, int64
                 cudaGraphExecDestroy(c->graph_exec);
                 c->graph_exec = nullptr;
             }
-            if (kmode == gt::KMODE_FP64) {
+            if (mode == GT_MODE_FP64) {
                 cudaGraph_t graph = nullptr;
                 err = cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal);
                 if (err != cudaSuccess) return cuda_code(err);
@@ -466,9 +475,9 @@ int run_trace(gt_ctx *c, const CamDesc *d_cams, int n_cams, int kind_hint, int64
         rc = cuda_code(cudaGraphLaunch(c->graph_exec, c->stream));
     } else if (mode == GT_MODE_FP64) {
         int grid;
-        rc = grid_for(c, e, gt::KMODE_FP64, kind_hint, n_rays, one_shot, &grid);
+        rc = grid_for(c, e, kmode64, kind_hint, n_rays, one_shot, &grid);
         if (rc != GT_OK) return rc;
-        err = gt::launch_trace(a, gt::KMODE_FP64, kind_hint, e.block_size, grid, one_shot,
+        err = gt::launch_trace(a, kmode64, kind_hint, e.block_size, grid, one_shot,
                                c->stream);
         rc = cuda_code(err);
     } else {
@@ -643,7 +652,8 @@ int gt_trace_range(gt_ctx *c, int64_t first, int64_t count, int64_t n_steps, dou
         return GT_ERR_INVALID_ARG;
     const int kind = (c->Q != 0.0) ? gt::KIND_MN : gt::KIND_KERR;
     return run_trace(c, c->d_cam, 1, kind, first, count, n_steps, sp, mode, t, r, th, ph, status,
-                     nsteps);
+                     nsteps, nullptr, nullptr, false, Extra(), gt::pair_range(c->M, c->r0),
+                     &c->cam_pair);
 }
 
 int gt_trace_pixels(gt_ctx *c, const int64_t *pixels, int64_t n, int64_t n_steps, double sp,
@@ -663,7 +673,8 @@ int gt_trace_pixels(gt_ctx *c, const int64_t *pixels, int64_t n, int64_t n_steps
     if (!c->cam_valid) return GT_ERR_INVALID_ARG;
     const int kind = (c->Q != 0.0) ? gt::KIND_MN : gt::KIND_KERR;
     return run_trace(c, c->d_cam, 1, kind, 0, n, n_steps, sp, mode, t, r, th, ph, status, nsteps,
-                     pixels, nullptr, true);
+                     pixels, nullptr, true, Extra(), gt::pair_range(c->M, c->r0),
+                     &c->cam_pair);
 }
 
 int gt_trace_disk(gt_ctx *c, double r_in, double r_out, double half_thickness, int64_t n_steps,
@@ -691,7 +702,7 @@ int gt_trace_disk(gt_ctx *c, double r_in, double r_out, double half_thickness, i
     x.z = z;
     const int kind = (c->Q != 0.0) ? gt::KIND_MN : gt::KIND_KERR;
     return run_trace(c, c->d_cam, 1, kind, 0, (int64_t)c->res_x * c->res_y, n_steps, sp, mode, t,
-                     r, th, ph, status, nsteps, nullptr, nullptr, false, x);
+                     r, th, ph, status, nsteps, nullptr, nullptr, false, x, true, &c->cam_pair);
 }
 
 int gt_trace_states(gt_ctx *c, int64_t n, double *t, double *r, double *th, double *ph,
@@ -784,9 +795,10 @@ int gt_trace_batch(gt_ctx *c, const gt_camera_desc *cams, int n_cams, int64_t n_
         return GT_ERR_INVALID_ARG;
     std::vector<CamDesc> h(n_cams);
     int64_t off = 0;
-    bool any_mn = false, any_kerr = false;
+    bool any_mn = false, any_kerr = false, range_ok = true;
     for (int i = 0; i < n_cams; i++) {
         const gt_camera_desc &d = cams[i];
+        range_ok = range_ok && gt::pair_range(d.M, d.r0);
         if (!valid_spacetime(d.M, d.S, d.Q) ||
             !valid_camera(d.r0, d.theta0, d.fov_deg, d.res_x, d.res_y))
             return GT_ERR_INVALID_ARG;
@@ -823,7 +835,7 @@ int gt_trace_batch(gt_ctx *c, const gt_camera_desc *cams, int n_cams, int64_t n_
         if (!h[i].valid) return GT_ERR_INVALID_ARG;
     const int kind = any_mn && any_kerr ? 2 : (any_mn ? gt::KIND_MN : gt::KIND_KERR);
     return run_trace(c, c->d_batch, n_cams, kind, 0, off, n_steps, sp, mode, t, r, th, ph, status,
-                     nsteps);
+                     nsteps, nullptr, nullptr, false, Extra(), range_ok, n_cams == 1 ? &h[0].pair : nullptr);
 }
 
 int gt_trace_rays(gt_ctx *c, int64_t n, const double *alpha, const double *beta,
@@ -936,7 +948,8 @@ int gt_surrogate_infer(gt_ctx *c, gt_surrogate *s, const gt_gate_cfg *gate, int6
     if (rc == GT_OK) rc = list_count(&n1);
     if (rc == GT_OK && n1 > 0)
         rc = run_trace(c, c->d_cam, 1, kind, 0, n1, n_steps, sp, mode, t, r, th, ph, status,
-                       nsteps, list, nullptr);
+                       nsteps, list, nullptr, false, Extra(), gt::pair_range(c->M, c->r0),
+                     &c->cam_pair);
     if (rc != GT_OK) return rc;
     // 3. probe records from the traced probes
     if (pg.stride > 0) {
@@ -953,7 +966,8 @@ int gt_surrogate_infer(gt_ctx *c, gt_surrogate *s, const gt_gate_cfg *gate, int6
     if (rc == GT_OK) rc = list_count(&n2);
     if (rc == GT_OK && n2 > 0)
         rc = run_trace(c, c->d_cam, 1, kind, 0, n2, n_steps, sp, mode, t, r, th, ph, status,
-                       nsteps, list, nullptr);
+                       nsteps, list, nullptr, false, Extra(), gt::pair_range(c->M, c->r0),
+                     &c->cam_pair);
     if (rc != GT_OK) return rc;
     if (n_fallback) *n_fallback = n1 - np + n2;
     if (n_probes) *n_probes = np;
@@ -1027,7 +1041,7 @@ int gt_autotune(gt_ctx *c, int mode, int64_t trial_rays, int64_t trial_steps, do
     int rc = GT_OK;
     for (int rpt = 1; rpt <= n_rpt && rc == GT_OK; rpt++) {
         for (int bi = 0; bi < 4 && rc == GT_OK; bi++) {
-            const int kmode = mode == GT_MODE_FP64 ? gt::KMODE_FP64 : gt::KMODE_MIXED_FP32;
+            const int kmode = mode == GT_MODE_FP64 ? gt::KMODE_FP64_PAIR : gt::KMODE_MIXED_FP32;
             const int fit = rpt == 2 ? gt::max_blocks_per_sm_two(kind, blocks[bi])
                                      : gt::max_blocks_per_sm(kmode, kind, blocks[bi]);
             for (int ki = 0; ki < 6 && rc == GT_OK; ki++) {

@@ -8,6 +8,7 @@
 
 #include "../../include/geotrace.h"
 #include "df.cuh"
+#include "pair.cuh"
 #include "spacetime.cuh"
 
 // The context's stream (capi.cu).
@@ -30,7 +31,7 @@ struct CamDesc {
     double gl_tt, gl_tph, gl_phph, gl_rr, gl_thth; // lower metric at the camera
     double r_escape;        // 1.5 r0
     double r_switch;        // FP32-mixed: zone radius
-    SpacetimeT<DF> st_df;   // the spacetime constants in double-float (the zone's field)
+    PairSpacetime pair;     // the spacetime constants of the double-float step
     int32_t valid;          // 1 when the camera sits where g_tt < 0
     int32_t pad_;
 };
@@ -46,8 +47,15 @@ enum : int {
     SCR_WORDS = 6
 };
 
-// Kernel modes (public GT_MODE_FP32_MIXED runs MIXED_FP32 and ZONE_FP64 in rounds).
-enum : int { KMODE_FP64 = 0, KMODE_MIXED_INLINE = 1, KMODE_MIXED_FP32 = 2, KMODE_ZONE_FP64 = 3 };
+// Kernel modes (public GT_MODE_FP32_MIXED runs MIXED_FP32 and a zone mode in rounds).
+enum : int {
+    KMODE_FP64 = 0,
+    KMODE_MIXED_INLINE = 1,
+    KMODE_MIXED_FP32 = 2,
+    KMODE_ZONE_FP64 = 3,  // zone steps in FP64 (GT_FLAG_ZONE_FP64)
+    KMODE_ZONE_PAIR = 4,  // zone steps in double-float (the default)
+    KMODE_FP64_PAIR = 5   // GT_MODE_FP64 with the double-float step (fp64_kmode)
+};
 
 // Kind of a launch: one spacetime kind for every camera (KIND_KERR, KIND_MN), per camera
 // (KIND_ANY), or per camera with the listing's forward-difference metric derivatives
@@ -104,7 +112,8 @@ struct TraceArgs {
     // float copies for the FP32 kernel, filled by launch_trace (kernel parameters the
     // loop reads directly, so no per-step conversions are rematerialised)
     float sp_f, w6_f, h_thr_f;
-    DF sp_df, w6_df; // double-float copies for the zone
+    TF sp_tf, w6_tf;           // copies for the double-float step
+    DF h_thr_df;
     int flags;
     int reproject_every;
     uint64_t timeout_ns; // 0 = no watchdog
@@ -120,6 +129,10 @@ struct TraceArgs {
     StateArrays states; // with states.t != null fresh rays start from these arrays and the
                         // end states (all 8 components) are written back to them
     int zone_df;        // FP32-mixed: the zone's Manko-Novikov field in double-float
+    // constants of the double-float step when the launch has one camera (pair_single): kernel
+    // parameters are read as instruction operands, descriptors in memory through registers
+    PairSpacetime pair;
+    int pair_single;
 };
 
 // Host-side validation shared by every entry point that takes a spacetime or a camera
@@ -156,6 +169,20 @@ inline void fill_desc(CamDesc &d, double M, double S, double Q, double r0, doubl
     d.res_x = rx;
     d.res_y = ry;
     d.offset = offset;
+}
+
+// Kernel mode of a GT_MODE_FP64 launch: the double-float step for camera rays with exact
+// derivatives under RK4, whose scales stay well inside the float range; FP64 arithmetic for
+// the listing's numerics, the ring, caller states, per-ray spacetimes (a set-up per ray) and
+// other scales.  `range_ok` is pair_range() over the launch's cameras.
+inline bool pair_range(double M, double r0) { return M >= 1e-3 && M <= 1e3 && r0 <= 1e5; }
+
+inline int fp64_kmode(const TraceArgs &a, int kind_hint, bool range_ok)
+{
+    return range_ok && a.sp >= 1e-9 && a.sp <= 1.0 && kind_hint != KIND_FD && !a.euler &&
+                   !a.f32_io && !a.disk.on && !a.states.t && !a.rays
+               ? KMODE_FP64_PAIR
+               : KMODE_FP64;
 }
 
 // Launchers (trace.cu).  Return a cudaError_t from the launch.

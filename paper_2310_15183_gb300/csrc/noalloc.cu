@@ -72,9 +72,10 @@ extern "C" int gt_trace_batch_noalloc(int device, void *cuda_stream, const gt_ca
 
     gt::CamDesc h[GT_NOALLOC_MAX_CAMS]; // host staging on the stack, not the heap
     int64_t total = 0;
-    bool any_mn = false, any_kerr = false;
+    bool any_mn = false, any_kerr = false, range_ok = true;
     for (int i = 0; i < n_cams; i++) {
         const gt_camera_desc &d = cams[i];
+        range_ok = range_ok && gt::pair_range(d.M, d.r0);
         if (!gt::valid_spacetime(d.M, d.S, d.Q) ||
             !gt::valid_camera(d.r0, d.theta0, d.fov_deg, d.res_x, d.res_y))
             return GT_ERR_INVALID_ARG;
@@ -142,14 +143,18 @@ extern "C" int gt_trace_batch_noalloc(int device, void *cuda_stream, const gt_ca
     a.nsteps = nsteps;
     a.scratch = words;
     a.zone_df = 1; // the context's default zone (double-float Manko-Novikov field)
+    if (n_cams == 1) {
+        a.pair = h[0].pair;
+        a.pair_single = 1;
+    }
     const int kind = any_mn && any_kerr ? 2 : (any_mn ? gt::KIND_MN : gt::KIND_KERR);
     const int block = 128;
-    const int fit = gt::max_blocks_per_sm(
-        mode == GT_MODE_FP64 ? gt::KMODE_FP64 : gt::KMODE_MIXED_INLINE, kind, block);
+    const int kmode =
+        mode == GT_MODE_FP64 ? gt::fp64_kmode(a, kind, range_ok) : gt::KMODE_MIXED_INLINE;
+    const int fit = gt::max_blocks_per_sm(kmode, kind, block);
     const int grid = (fit < 4 ? fit : 4) * sms;
     // FP32-mixed runs its zone inline here: the park lists of the context path
     // would need allocated memory
-    e = gt::launch_trace(a, mode == GT_MODE_FP64 ? gt::KMODE_FP64 : gt::KMODE_MIXED_INLINE, kind,
-                         block, grid, false, s);
+    e = gt::launch_trace(a, kmode, kind, block, grid, false, s);
     return e == cudaSuccess ? GT_OK : GT_ERR_CUDA;
 }

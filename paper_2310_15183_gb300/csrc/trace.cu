@@ -26,7 +26,6 @@
 #include "compensated.cuh"
 #include "internal.cuh"
 #include "spacetime.cuh"
-#include "zone_df.cuh"
 
 namespace gt {
 
@@ -43,6 +42,52 @@ __device__ __forceinline__ uint64_t globaltimer_ns()
 // Spacetime constants (Sec. 2.2.2: a = S/M; Sec. 2.2.3: alpha, k, beta), the pixel
 // ranges V = tan(FOV/2)/r0 and H = atan(tan(V) res_x/res_y) of the listing, and the
 // lower metric at the camera (inverse of g^{mu nu}'s (t, phi) block and diagonal).
+// Three-float form of a double-double.
+__device__ __forceinline__ TF tf_from2(double hi, double lo)
+{
+    TF t;
+    t.a = (float)hi;
+    const double r = (hi - (double)t.a) + lo;
+    t.b = (float)r;
+    t.c = (float)(r - (double)t.b);
+    return t;
+}
+
+// Constants of the double-float step.  Kerr's r_+ = M + sqrt(M^2 - a^2) and Manko-Novikov's
+// M + k are carried beyond 53 bits, so that r - r_+ vanishes where the metric's Delta does.
+__device__ void setup_pair(const SpacetimeC &st, PairSpacetime &p)
+{
+    p.kind = st.kind;
+    double rt, rt_lo = 0.0; // r_+ - M
+    if (st.kind == KIND_KERR) {
+        const double m2 = st.M * st.M, m2l = fma(st.M, st.M, -m2);
+        const double a2l = fma(st.a, st.a, -st.a2);
+        const double d = m2 - st.a2; // M >= a: the error of the difference
+        const double dl = ((m2 - d) - st.a2) + (m2l - a2l);
+        rt = sqrt(d + dl);
+        rt_lo = rt > 0.0 ? (fma(-rt, rt, d) + dl) / (2.0 * rt) : 0.0;
+        p.a = DF(st.a);
+        p.a2 = DF(st.a2);
+        p.r_hard = -1.0f;
+    } else {
+        rt = st.k;
+        p.ik = tf_from(st.ik);
+        p.alpha = tf_from(st.alpha);
+        p.two_beta = DF(st.two_beta);
+        p.three_beta2 = DF(st.three_beta2);
+        p.c_g = tf_from(st.c_g);
+        p.w_inf = tf_from(st.w_inf);
+        p.k2 = tf_from(st.k2);
+        p.inv_k2 = tf_from(st.inv_k2);
+        p.two_k = tf_from(st.two_k);
+        p.r_hard = (float)(4.0 * st.M - st.r_plus);
+    }
+    const double s = st.M + rt, e = rt - (s - st.M); // M >= rt: Fast2Sum
+    p.r_plus = tf_from2(s, e + rt_lo);
+    p.r_plus2 = DF(s);
+    p.split = DF(2.0 * rt);
+}
+
 __device__ void setup_desc(CamDesc &d, int flags, double r_switch)
 {
     SpacetimeC st = {};
@@ -71,7 +116,7 @@ __device__ void setup_desc(CamDesc &d, int flags, double r_switch)
         st.r_plus = d.M + sqrt(d.M * d.M - st.a2);
     }
     d.st = st;
-    d.st_df = to_df(st);
+    setup_pair(st, d.pair);
     d.V = tan(0.5 * d.fov_deg / 180.0 * M_PI) / d.r0;
     d.H = atan(tan(d.V) * (double)d.res_x / (double)d.res_y);
     d.inv_sin_th0 = (flags & GT_FLAG_COMPAT_CAMERA) ? 1.0 : 1.0 / sin(d.th0);
@@ -248,103 +293,128 @@ __device__ __forceinline__ double step64(const TraceArgs &A, const SpacetimeC &s
     return rk4_step64<KIND>(st, x, A.sp, A.w6, y);
 }
 
-// ------------------------------------------------------------------ the zone in double-float
-// The FP32-mixed path's zone steps an FP64 state.  Within a step the stage arithmetic --
-// the stage points, the sin/cos rotation, the field (Manko-Novikov, or Kerr when a zone
-// is set for it), the stage sums and the step length -- runs in double-float
-// (zone_df.cuh) on the FP32 pipes; the state is converted once into double-float at the
-// start of the step, the increments once back, and added in FP64.  A field evaluation
-// outside the double-float range (Manko-Novikov exponents out of bounds, or a rate that
-// is not finite) takes FP64; n_f64 counts those evaluations.
-template <int KIND>
-__device__ __forceinline__ void zone_rates(const SpacetimeC &st, const SpacetimeT<DF> *sd, DF r,
-                                           DF s, DF cs, DF pr, DF pth, DF pt, DF pph,
-                                           Rates<DF> &o, uint32_t &n_f64)
+// ------------------------------------------------------------------ the double-float step
+// Ray state of the double-float kernels (pair.cuh): three floats per coordinate.
+struct RayTF {
+    TF t, r, th, ph, pr, pth, pt, pph;
+};
+
+__device__ __forceinline__ void tf_state(const Ray64 &x, RayTF &s)
 {
-    const bool mn = KIND == KIND_MN || (KIND == KIND_ANY && st.kind == KIND_MN);
-    if (mn) {
-        if (mn_rates_df(*sd, r, s, cs, pr, pth, pt, pph, o)) return;
-    } else if (KIND != KIND_FD) {
-        kerr_rates_sc<DF>(*sd, r, s, cs, pr, pth, pt, pph, o);
-        if (isfinite(o.dt.hi) && isfinite(o.dr.hi) && isfinite(o.dth.hi) &&
-            isfinite(o.dph.hi) && isfinite(o.dpr.hi) && isfinite(o.dpth.hi))
-            return;
-    }
-    ++n_f64;
-    Rates<double> o64;
-    rates_any<KIND>(st, df_to(r), df_to(s), df_to(cs), df_to(pr), df_to(pth), df_to(pt),
-                    df_to(pph), o64);
-    o.dt = DF(o64.dt);
-    o.dr = DF(o64.dr);
-    o.dth = DF(o64.dth);
-    o.dph = DF(o64.dph);
-    o.dpr = DF(o64.dpr);
-    o.dpth = DF(o64.dpth);
+    s.t = tf_from(x.t);
+    s.r = tf_from(x.r);
+    s.th = tf_from(x.th);
+    s.ph = tf_from(x.ph);
+    s.pr = tf_from(x.pr);
+    s.pth = tf_from(x.pth);
+    s.pt = tf_from(x.pt);
+    s.pph = tf_from(x.pph);
 }
 
-__device__ __forceinline__ DF df_twice(DF a) { return DF(2.0f * a.hi, 2.0f * a.lo); }
-
-// One RK4 step of the zone: the stages of rk4_step64 (stage points x + h/2 k1, x + h/2 k2,
-// x + h k3; weights 1, 2, 2, 1 times h w6; h = |sp / k1.dt|) in a rolled stage loop, so one
-// copy of the double-float field is compiled.  sd: the spacetime constants in
-// double-float; sp_df, w6_df: step precision and RK4 weight in double-float.
-template <int KIND>
-__device__ __forceinline__ double rk4_step_zone(const SpacetimeC &st, const SpacetimeT<DF> *sd,
-                                                const Ray64 &x, DF sp_df, DF w6_df, Ray64 &y,
-                                                uint32_t &n_f64)
+// The evolving coordinates back in FP64 (the constants of motion of x are kept).
+__device__ __forceinline__ void tf_unstate(const RayTF &s, Ray64 &x)
 {
-    double s64, c64;
-    sincos(x.th, &s64, &c64);
-    const DF S1(s64), C1(c64), R0(x.r), PR0(x.pr), PTH0(x.pth), PT(x.pt), PPH(x.pph);
+    x.t = tf_to(s.t);
+    x.r = tf_to(s.r);
+    x.th = tf_to(s.th);
+    x.ph = tf_to(s.ph);
+    x.pr = tf_to(s.pr);
+    x.pth = tf_to(s.pth);
+}
+
+// Largest |exponent| of a Manko-Novikov evaluation taken in double-float: |2 beta Ea|,
+// |2 beta Eb| <= 24 and |2 psi|, |2 psi - 2 gamma''| <= 48.  Beyond, products of the metric
+// functions overflow the float range (an infinite high part turns the low part into NaN, so
+// the rates come out non-finite) or, silently, low parts fall below the normal floats.
+constexpr float PAIR_MAX_EF = 24.0f;
+constexpr float PAIR_MAX_EPSI = 48.0f;
+
+// The tables of pair.cuh, copied by each block into shared memory.
+__device__ const PairTables g_pair_tables = make_pair_tables();
+
+struct PairExp {
+    const PairTables *tab;
+    __device__ __forceinline__ DF operator()(DF a) const { return p_exp(a, tab); }
+};
+
+__device__ __forceinline__ bool finite_rates(const Rates<DF> &o)
+{
+    return isfinite(o.dt.hi) && isfinite(o.dr.hi) && isfinite(o.dth.hi) && isfinite(o.dph.hi) &&
+           isfinite(o.dpr.hi) && isfinite(o.dpth.hi);
+}
+
+// One RK4 step of x in double-float: the stages of rk4_step64 (stage points x + h/2 k1,
+// x + h/2 k2, x + h k3; weights 1, 2, 2, 1 times h w6; h = |sp / k1.dt|) in a rolled loop, so
+// one copy of the field is compiled.  Returns false, x untouched, where an evaluation leaves
+// the double-float range (exponents, the axis, |theta| beyond the table reduction, a rate
+// that is not finite): the caller repeats the step in FP64.
+template <int KIND>
+__device__ __forceinline__ bool pair_step(const PairSpacetime &c, const PairTables *tab, RayTF &x,
+                                          TF sp, TF w6, DF &h_out)
+{
+    const DF rp0 = tf_diff(x.r, c.r_plus);
+    DF rp = rp0, pr = tf_pair(x.pr), pth = tf_pair(x.pth), th = tf_pair(x.th);
     Rates<DF> k, acc;
-    DF h(0.0f, 0.0f), r = R0, pr = PR0, pth = PTH0, s = S1, c = C1;
+    DF h(0.0f, 0.0f);
+    bool ok = fabsf(x.th.a) <= 128.0f;
 #pragma unroll 1
     for (int stage = 0; stage < 4; stage++) {
-        zone_rates<KIND>(st, sd, r, s, c, pr, pth, PT, PPH, k, n_f64);
-        if (stage == 0) {
-            h = sp_df * rcp_t(k.dt);
-            if (h.hi < 0.0f) h = -h;
-            acc = k;
-        } else if (stage < 3) {
-            acc.dt = acc.dt + df_twice(k.dt);
-            acc.dr = acc.dr + df_twice(k.dr);
-            acc.dth = acc.dth + df_twice(k.dth);
-            acc.dph = acc.dph + df_twice(k.dph);
-            acc.dpr = acc.dpr + df_twice(k.dpr);
-            acc.dpth = acc.dpth + df_twice(k.dpth);
+        DF s, cs;
+        p_sincos(th, x.th.c, tab, &s, &cs);
+        if (KIND == KIND_MN || (KIND == KIND_ANY && c.kind == KIND_MN)) {
+            float ex[4];
+            mn_rates_pair(c, rp, s, cs, pr, pth, x.pt, x.pph, PairExp{tab}, k, ex);
+            ok = ok && fmaxf(fabsf(ex[0]), fabsf(ex[1])) <= PAIR_MAX_EF &&
+                 fmaxf(fabsf(ex[2]), fabsf(ex[3])) <= PAIR_MAX_EPSI;
         } else {
-            acc.dt = acc.dt + k.dt;
-            acc.dr = acc.dr + k.dr;
-            acc.dth = acc.dth + k.dth;
-            acc.dph = acc.dph + k.dph;
-            acc.dpr = acc.dpr + k.dpr;
-            acc.dpth = acc.dpth + k.dpth;
+            kerr_rates_pair(c, rp, s, cs, pr, pth, x.pt, x.pph, k);
+        }
+        ok = ok && fabsf(s.hi) >= 1e-6f;
+        if (stage == 0) {
+            h = p_norm(p_mul3(p_rcp(k.dt), sp));
+            if (h.hi < 0.0f) h = p_neg(h);
+            acc = k;
+        } else {
+            const float w = stage < 3 ? 2.0f : 1.0f;
+            acc.dt = p_add(acc.dt, p_scale(k.dt, w));
+            acc.dr = p_add(acc.dr, p_scale(k.dr, w));
+            acc.dth = p_add(acc.dth, p_scale(k.dth, w));
+            acc.dph = p_add(acc.dph, p_scale(k.dph, w));
+            acc.dpr = p_add(acc.dpr, p_scale(k.dpr, w));
+            acc.dpth = p_add(acc.dpth, p_scale(k.dpth, w));
         }
         if (stage < 3) {
-            const DF d = stage < 2 ? DF(0.5f * h.hi, 0.5f * h.lo) : h;
-            r = R0 + d * k.dr;
-            pr = PR0 + d * k.dpr;
-            pth = PTH0 + d * k.dpth;
-            const DF dth = d * k.dth;
-            if (!rotate_sc_df(S1, C1, dth, &s, &c)) {
-                double s2, c2;
-                sincos(x.th + df_to(dth), &s2, &c2);
-                s = DF(s2);
-                c = DF(c2);
-            }
+            const DF d = p_scale(h, stage < 2 ? 0.5f : 1.0f);
+            rp = p_norm(p_fma(d, k.dr, rp0));
+            pr = p_norm(p_fma(d, k.dpr, tf_pair(x.pr)));
+            pth = p_norm(p_fma(d, k.dpth, tf_pair(x.pth)));
+            th = p_norm(p_fma(d, k.dth, tf_pair(x.th)));
         }
     }
-    if (!isfinite(h.hi)) return nan("");
-    const DF hw = h * w6_df;
-    y.t = x.t + df_to(hw * acc.dt);
-    y.r = x.r + df_to(hw * acc.dr);
-    y.th = x.th + df_to(hw * acc.dth);
-    y.ph = x.ph + df_to(hw * acc.dph);
-    y.pr = x.pr + df_to(hw * acc.dpr);
-    y.pth = x.pth + df_to(hw * acc.dpth);
-    y.pt = x.pt;
-    y.pph = x.pph;
-    return df_to(h);
+    // the sums of the stages are finite only if every rate was
+    if (!ok || !finite_rates(acc) || !isfinite(h.hi)) return false;
+    const DF hw = p_norm(p_mul3(h, w6));
+    x.t = tf_add(x.t, p_norm(p_mul(hw, acc.dt)));
+    x.r = tf_add(x.r, p_norm(p_mul(hw, acc.dr)));
+    x.th = tf_add(x.th, p_norm(p_mul(hw, acc.dth)));
+    x.ph = tf_add(x.ph, p_norm(p_mul(hw, acc.dph)));
+    x.pr = tf_add(x.pr, p_norm(p_mul(hw, acc.dpr)));
+    x.pth = tf_add(x.pth, p_norm(p_mul(hw, acc.dpth)));
+    h_out = h;
+    return true;
+}
+
+// The same step in FP64, out of line: the double-float kernels keep their registers.
+template <int KIND>
+__device__ __noinline__ double rk4_step64_call(const SpacetimeC &st, const Ray64 &x, double sp,
+                                               double w6, Ray64 &y)
+{
+    return rk4_step64<KIND>(st, x, sp, w6, y);
+}
+
+__device__ __forceinline__ bool tf_greater(TF x, TF y)
+{
+    return x.a > y.a || (x.a == y.a && (x.b > y.b || (x.b == y.b && x.c > y.c)));
 }
 
 // ------------------------------------------------------------------ ring and redshift
@@ -584,6 +654,8 @@ __device__ __forceinline__ void reproject_pr(const SpacetimeC &st, Ray64 &x)
 //         parked on the output list; input list items continue in FP32.
 // MODE 3: FP64 zone steps for parked rays; a ray leaving the zone (r > 1.25 r_switch)
 //         is parked on the output list for the next FP32 launch.
+// MODE 4: MODE 3 with the double-float step.
+// MODE 5: MODE 0 with the double-float step.
 // KIND: 0 Kerr, 1 Manko-Novikov, 2 per-camera, 3 per-camera with forward-difference
 // derivatives (MODE 0 only).
 // Work of a launch: fresh rays [0, n_fresh) then input-list items [0, *in_count).
@@ -614,6 +686,21 @@ __device__ __forceinline__ void park(const TraceArgs &A, int64_t id, uint32_t n,
 template <int MODE, int KIND, bool PRECISE>
 __device__ __forceinline__ void trace_body(const TraceArgs &A, int one_shot)
 {
+    constexpr bool ZONE = MODE == 3 || MODE == 4;  // zone rays, parked when they leave
+    constexpr bool PAIR = MODE == 4 || MODE == 5;  // three-float state, double-float step
+    constexpr bool TABLES = PAIR || MODE == 1;
+    constexpr bool SINGLE = PAIR && PRECISE;       // one camera, its constants in A.pair
+    // per-ray spacetimes come with KIND_ANY only, and never to the double-float MODE 5
+    const RayParams *const rays = KIND == KIND_ANY && MODE != 5 ? A.rays : nullptr;
+    __shared__ PairTables tab_s[1];
+    const PairTables *tab = tab_s;
+    if (TABLES) {
+        const float *src = reinterpret_cast<const float *>(&g_pair_tables);
+        float *dst = reinterpret_cast<float *>(tab_s);
+        for (int i = threadIdx.x; i < (int)(sizeof(PairTables) / sizeof(float)); i += blockDim.x)
+            dst[i] = src[i];
+        __syncthreads();
+    }
     const int lane = threadIdx.x & 31;
     const unsigned lt_mask = (1u << lane) - 1u;
     unsigned long long *next = A.scratch + SCR_NEXT_RAY;
@@ -631,7 +718,8 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A, int one_shot)
     uint32_t n = 0;
     uint32_t n_entry = 0;           // step count when the ray entered this launch (zone steps)
     uint32_t n_f64 = 0;             // zone field evaluations of the ray in FP64 (this launch)
-    SpacetimeT<DF> sd_ray;          // double-float constants of a per-ray spacetime
+    PairSpacetime pr_ray;           // double-float constants of a per-ray spacetime
+    RayTF T;                        // state of the double-float kernels
     uint32_t rp_next = 0xFFFFFFFFu; // next step count that is a multiple of reproject_every
     Ray64 x;
     RayMixed m;
@@ -643,12 +731,13 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A, int one_shot)
     const float h_thr_f = A.h_thr_f;
     F2 r_esc_f = f2_from(r_esc);
     float r_sw_f = (float)r_sw;
+    TF r_esc_t = tf_from(r_esc), r_out_t = tf_from(1.25 * r_sw);
 
     auto load_camera = [&](int c) {
         cam = c;
         // the FP32-only kernel keeps just the float constants live; the FP64 ones are
         // reloaded for the occasional re-projection
-        if (MODE != 2) st = cams[c].st;
+        if (MODE != 2 && !PAIR) st = cams[c].st;
         r_esc = cams[c].r_escape;
         r_sw = cams[c].r_switch;
         if (MODE == 1 || MODE == 2) stf = to_float(cams[c].st);
@@ -656,20 +745,24 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A, int one_shot)
             r_esc_f = f2_from(r_esc);
             r_sw_f = (float)r_sw;
         }
+        if (PAIR) {
+            r_esc_t = tf_from(r_esc);
+            r_out_t = tf_from(1.25 * r_sw);
+        }
     };
     auto load_rayparams = [&](int64_t rid, bool init) {
         CamDesc d;
-        d.M = A.rays->M;
-        d.S = A.rays->spin[rid] * A.rays->M * A.rays->M; // spin = a/M
-        d.Q = A.rays->q[rid];
-        d.r0 = A.rays->r0;
-        d.th0 = A.rays->theta0[rid];
+        d.M = rays->M;
+        d.S = rays->spin[rid] * rays->M * rays->M; // spin = a/M
+        d.Q = rays->q[rid];
+        d.r0 = rays->r0;
+        d.th0 = rays->theta0[rid];
         d.fov_deg = 90.0;
         d.res_x = d.res_y = 1;
         d.offset = 0;
-        setup_desc(d, A.flags, A.rays->r_switch);
+        setup_desc(d, A.flags, rays->r_switch);
         if (MODE != 2) st = d.st;
-        if (MODE == 1 || MODE == 3) sd_ray = d.st_df;
+        if (MODE == 1 || MODE == 4) pr_ray = d.pair;
         r_esc = d.r_escape;
         r_sw = d.r_switch;
         if (MODE == 1 || MODE == 2) stf = to_float(d.st);
@@ -677,7 +770,11 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A, int one_shot)
             r_esc_f = f2_from(r_esc);
             r_sw_f = (float)r_sw;
         }
-        if (init) camera_init_dir(d, A.rays->alpha[rid], A.rays->beta[rid], x);
+        if (PAIR) {
+            r_esc_t = tf_from(r_esc);
+            r_out_t = tf_from(1.25 * r_sw);
+        }
+        if (init) camera_init_dir(d, rays->alpha[rid], rays->beta[rid], x);
         return d.valid != 0;
     };
 
@@ -686,7 +783,7 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A, int one_shot)
         if (w < A.n_fresh) { // a fresh ray: initial data from the camera
             const int64_t pix = A.fresh_ids ? A.fresh_ids[w] : w;
             id = (A.fresh_ids && A.compact_out) ? w : pix;
-            if (A.rays) {
+            if (rays) {
                 const bool valid = load_rayparams(pix, true);
                 n = 0;
                 if (!valid || A.n_steps <= 0) {
@@ -730,7 +827,7 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A, int one_shot)
             const ParkItem &it = A.in_items[w - A.n_fresh];
             id = it.id;
             n = it.n;
-            if (A.rays)
+            if (rays)
                 load_rayparams(id, false);
             else if (KIND >= KIND_ANY || A.n_cams > 1)
                 load_camera(it.cam);
@@ -745,6 +842,7 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A, int one_shot)
         }
         n_entry = n;
         n_f64 = 0;
+        if (PAIR) tf_state(x, T);
         if (MODE == 1 || MODE == 2) {
             mixed_from64(x, m);
             if (A.reproject_every > 0) {
@@ -798,6 +896,7 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A, int one_shot)
             if (stop) {
                 if (active) {
                     if (MODE == 1 || MODE == 2) mixed_to64(m, x);
+                    if (PAIR) tf_unstate(T, x);
                     store_full(A, id, x, GT_RAY_TIMEOUT, n, nan(""));
                 }
                 if (!one_shot) {
@@ -814,8 +913,8 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A, int one_shot)
                             } else if (w < A.n_fresh) {
                                 const int64_t pix = A.fresh_ids ? A.fresh_ids[w] : w;
                                 const int c = A.n_cams > 1 ? find_camera(cams, A.n_cams, pix) : 0;
-                                const double r0 = A.rays ? A.rays->r0 : cams[c].r0;
-                                const double th0 = A.rays ? A.rays->theta0[pix] : cams[c].th0;
+                                const double r0 = rays ? rays->r0 : cams[c].r0;
+                                const double th0 = rays ? rays->theta0[pix] : cams[c].th0;
                                 store_ray(A, (A.fresh_ids && A.compact_out) ? w : pix, 0.0, r0,
                                           th0, 0.0, GT_RAY_TIMEOUT, 0);
                             } else {
@@ -841,16 +940,56 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A, int one_shot)
 
         // ---- one RK4 step
         int status = -1;
-        if (MODE == 0 || MODE == 3) {
-            Ray64 y;
-            double h;
-            if (MODE == 3 && A.zone_df) {
-                h = rk4_step_zone<KIND>(st, A.rays ? &sd_ray : &cams[cam].st_df, x, A.sp_df,
-                                        A.w6_df, y, n_f64);
+        if (PAIR) {
+            // GT_MODE_FP64 takes Manko-Novikov steps below 4M in FP64: next to the ergosurface
+            // 1/A^2 amplifies the rounding of the field, where 48 bits show against 53
+            const PairSpacetime &pc = SINGLE ? A.pair : rays ? pr_ray : cams[cam].pair;
+            const bool hard = MODE == 5 && KIND != KIND_KERR &&
+                              T.r.a - pc.r_plus.a < pc.r_hard;
+            DF h;
+            ++n;
+            if (!hard && pair_step<KIND>(pc, tab, T, A.sp_tf, A.w6_tf, h)) {
+                if (tf_greater(T.r, r_esc_t))
+                    status = GT_RAY_ESCAPED;
+                else if (h.hi < A.h_thr_df.hi || (h.hi == A.h_thr_df.hi && h.lo < A.h_thr_df.lo))
+                    status = GT_RAY_HORIZON;
+                else if ((int64_t)n >= A.n_steps)
+                    status = GT_RAY_MAXSTEPS;
+                // the ring is tested after the escape and before the horizon
+                if (MODE == 4 && A.disk.on && status != GT_RAY_ESCAPED &&
+                    in_disk(A.disk, tf_to(T.r), tf_to(T.th)))
+                    status = GT_RAY_DISK;
+                if (status >= 0) tf_unstate(T, x);
             } else {
-                h = step64<KIND>(A, st, x, y);
-                if (MODE == 3) n_f64 += 4;
+                Ray64 y;
+                tf_unstate(T, x);
+                const double h64 = rk4_step64_call<KIND>(rays ? st : cams[cam].st, x, A.sp, A.w6, y);
+                n_f64 += 4;
+                if (!isfinite(h64) || !finite6(y)) {
+                    status = GT_RAY_NONFINITE;
+                } else {
+                    x = y;
+                    status = exit_status(x.r, h64, r_esc, A.sp, n, A.n_steps);
+                    if (MODE == 4 && A.disk.on && status != GT_RAY_ESCAPED &&
+                        in_disk(A.disk, x.r, x.th))
+                        status = GT_RAY_DISK;
+                    tf_state(x, T);
+                }
             }
+            if (ZONE && status < 0 && tf_greater(T.r, r_out_t)) { // leave the zone
+                bool ok;
+                tf_unstate(T, x);
+                park(A, id, n, cam, x, &ok);
+                if (ok) {
+                    active = false;
+                    atomicAdd(A.scratch + SCR_ZONE_STEPS, (unsigned long long)(n - n_entry));
+                    if (n_f64) atomicAdd(A.scratch + SCR_ZONE_F64, (unsigned long long)n_f64);
+                }
+            }
+        } else if (MODE == 0 || MODE == 3) {
+            Ray64 y;
+            const double h = step64<KIND>(A, st, x, y);
+            if (MODE == 3) n_f64 += 4;
             ++n;
             if (!isfinite(h) || !finite6(y)) {
                 status = GT_RAY_NONFINITE;
@@ -874,17 +1013,21 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A, int one_shot)
             double h;
             bool ok = true;
             if ((double)m.r.hi < r_sw) { // the zone inline
-                Ray64 y;
+                DF hd;
                 mixed_to64(m, x);
-                if (A.zone_df) {
-                    h = rk4_step_zone<KIND>(st, A.rays ? &sd_ray : &cams[cam].st_df, x,
-                                            A.sp_df, A.w6_df, y, n_f64);
+                tf_state(x, T);
+                if (A.zone_df && pair_step<KIND>(rays ? pr_ray : cams[cam].pair, tab, T, A.sp_tf,
+                                                 A.w6_tf, hd)) {
+                    h = df_to(hd);
+                    tf_unstate(T, x);
+                    mixed_from64(x, m);
                 } else {
-                    h = step64<KIND>(A, st, x, y);
+                    Ray64 y;
+                    h = rk4_step64_call<KIND>(st, x, A.sp, A.w6, y);
                     n_f64 += 4;
+                    ok = isfinite(h) && finite6(y);
+                    if (ok) mixed_from64(y, m);
                 }
-                ok = isfinite(h) && finite6(y);
-                if (ok) mixed_from64(y, m);
             } else {
                 RayMixed keep = m;
                 h = (double)rk4_step32<KIND>(stf, m, spf, w6f);
@@ -941,17 +1084,17 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A, int one_shot)
                               : rp_next + (uint32_t)A.reproject_every;
                 mixed_to64(m, x);
                 SpacetimeC st64;
-                if (A.rays) {
+                if (rays) {
                     CamDesc d;
-                    d.M = A.rays->M;
-                    d.S = A.rays->spin[id] * A.rays->M * A.rays->M;
-                    d.Q = A.rays->q[id];
-                    d.r0 = A.rays->r0;
-                    d.th0 = A.rays->theta0[id];
+                    d.M = rays->M;
+                    d.S = rays->spin[id] * rays->M * rays->M;
+                    d.Q = rays->q[id];
+                    d.r0 = rays->r0;
+                    d.th0 = rays->theta0[id];
                     d.fov_deg = 90.0;
                     d.res_x = d.res_y = 1;
                     d.offset = 0;
-                    setup_desc(d, A.flags, A.rays->r_switch);
+                    setup_desc(d, A.flags, rays->r_switch);
                     st64 = d.st;
                 } else {
                     st64 = cams[cam].st;
@@ -962,7 +1105,7 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A, int one_shot)
             if (status >= 0) mixed_to64(m, x);
         }
         if (status >= 0) {
-            if (MODE == 3) {
+            if (ZONE) {
                 atomicAdd(A.scratch + SCR_ZONE_STEPS, (unsigned long long)(n - n_entry));
                 if (n_f64) atomicAdd(A.scratch + SCR_ZONE_F64, (unsigned long long)n_f64);
             }
@@ -980,6 +1123,18 @@ template <int MODE, int KIND, bool PRECISE = false>
 __global__ void __launch_bounds__(256, MODE == 2 ? 2 : 1) trace_kernel(TraceArgs A, int one_shot)
 {
     trace_body<MODE, KIND, PRECISE>(A, one_shot);
+}
+
+// The double-float kernels: 168 registers, 12 warps an SM.  The Manko-Novikov sweep spills
+// ~250 bytes a thread at that, which costs less than the third warp per scheduler gives:
+// 200,000 Manko-Novikov rays x 1,000 steps take 67.9 ms against 69.5 ms with 252 registers
+// and 8 warps (208: 69.9 ms), 48,000 rays 40.5 against 46.3 ms; Kerr (160) is the same either
+// way.  A per-ray spacetime lives in registers and local memory already: it keeps 255.
+template <int MODE, int KIND, bool SINGLE>
+__global__ void __maxnreg__(KIND == KIND_ANY ? 255 : 168)
+    pair_kernel(const __grid_constant__ TraceArgs A, int one_shot)
+{
+    trace_body<MODE, KIND, SINGLE>(A, one_shot);
 }
 
 // ------------------------------------------------------------------ two rays per thread
@@ -1154,8 +1309,9 @@ cudaError_t launch_trace_two(const TraceArgs &args, int kind_hint, int block, in
     a.sp_f = (float)a.sp;
     a.w6_f = (float)a.w6;
     a.h_thr_f = (float)(a.sp * 0.00003);
-    a.sp_df = DF(a.sp);
-    a.w6_df = DF(a.w6);
+    a.sp_tf = tf_from(a.sp);
+    a.w6_tf = tf_from(a.w6);
+    a.h_thr_df = DF(a.sp * 0.00003);
     return kind_hint == KIND_KERR ? launch_two<KIND_KERR>(a, block, grid, s)
                                   : launch_two<KIND_MN>(a, block, grid, s);
 }
@@ -1192,7 +1348,13 @@ static cudaError_t launch_one(const TraceArgs &a, int block, int grid, bool one_
             return cudaGetLastError();
         }
     }
-    trace_kernel<MODE, KIND><<<grid, block, 0, s>>>(a, one_shot ? 1 : 0);
+    if constexpr (MODE >= 4) {
+        if (KIND < KIND_ANY && a.pair_single)
+            pair_kernel<MODE, KIND, KIND < KIND_ANY><<<grid, block, 0, s>>>(a, one_shot ? 1 : 0);
+        else
+            pair_kernel<MODE, KIND, false><<<grid, block, 0, s>>>(a, one_shot ? 1 : 0);
+    } else
+        trace_kernel<MODE, KIND><<<grid, block, 0, s>>>(a, one_shot ? 1 : 0);
     return cudaGetLastError();
 }
 
@@ -1216,13 +1378,16 @@ cudaError_t launch_trace(const TraceArgs &args, int kmode, int kind_hint, int bl
     a.sp_f = (float)a.sp;
     a.w6_f = (float)a.w6;
     a.h_thr_f = (float)(a.sp * 0.00003);
-    a.sp_df = DF(a.sp);
-    a.w6_df = DF(a.w6);
+    a.sp_tf = tf_from(a.sp);
+    a.w6_tf = tf_from(a.w6);
+    a.h_thr_df = DF(a.sp * 0.00003);
     switch (kmode) {
     case KMODE_FP64: return launch_mode<0>(a, kind_hint, block, grid, one_shot, s);
     case KMODE_MIXED_INLINE: return launch_mode<1>(a, kind_hint, block, grid, one_shot, s);
     case KMODE_MIXED_FP32: return launch_mode<2>(a, kind_hint, block, grid, one_shot, s);
     case KMODE_ZONE_FP64: return launch_mode<3>(a, kind_hint, block, grid, one_shot, s);
+    case KMODE_ZONE_PAIR: return launch_mode<4>(a, kind_hint, block, grid, one_shot, s);
+    case KMODE_FP64_PAIR: return launch_mode<5>(a, kind_hint, block, grid, one_shot, s);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -1231,9 +1396,12 @@ template <int MODE, int KIND>
 static int occupancy_one(int block)
 {
     int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, trace_kernel<MODE, KIND>, block, 0) !=
-        cudaSuccess)
-        return 1;
+    cudaError_t e;
+    if constexpr (MODE >= 4)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, pair_kernel<MODE, KIND, (KIND < KIND_ANY)>, block, 0);
+    else
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, trace_kernel<MODE, KIND>, block, 0);
+    if (e != cudaSuccess) return 1;
     return n > 0 ? n : 1;
 }
 
@@ -1256,6 +1424,8 @@ int max_blocks_per_sm(int kmode, int kind_hint, int block)
     case KMODE_MIXED_INLINE: return occupancy_mode<1>(kind_hint, block);
     case KMODE_MIXED_FP32: return occupancy_mode<2>(kind_hint, block);
     case KMODE_ZONE_FP64: return occupancy_mode<3>(kind_hint, block);
+    case KMODE_ZONE_PAIR: return occupancy_mode<4>(kind_hint, block);
+    case KMODE_FP64_PAIR: return occupancy_mode<5>(kind_hint, block);
     default: return 1;
     }
 }

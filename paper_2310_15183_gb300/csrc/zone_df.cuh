@@ -1,7 +1,7 @@
-// zone_df.cuh -- the Manko-Novikov rates of the FP32-mixed path's zone in double-float
-// (df.cuh): the FP64 state goes in, FP64 rates come out, and the evaluation between runs
-// on the FP32 pipes.  Where the evaluation would leave the range in which double-float
-// keeps its precision, mn_rates_df returns false and the caller evaluates in FP64.
+// zone_df.cuh -- the Manko-Novikov rates in the renormalised double-float arithmetic of
+// df.cuh: the form the kernels' pair step (pair.cuh) is held to by the host tests, which
+// compare both with FP64 and extended precision.  Where the evaluation would leave the range
+// in which double-float keeps its precision, mn_rates_df returns false.
 #pragma once
 
 #include "df.cuh"
