@@ -96,8 +96,9 @@ typedef struct gt_ctx gt_ctx;
 
 /* Launch and precision options; zero fields take the defaults noted. */
 typedef struct gt_options {
-    int block_size;          /* threads per block, multiple of 32 in [32, 256]; 0 = 128 */
-    int blocks_per_sm;       /* persistent grid = min(blocks_per_sm, resident limit) * SMs; 0 = 4 */
+    int block_size;          /* threads per block, multiple of 32 in [32, 256] */
+    int blocks_per_sm;       /* persistent grid = min(blocks_per_sm, resident limit) * SMs */
+                             /* (one of the two 0: 128 or 4; both 0: chosen by the launch) */
     int flags;               /* GT_FLAG_* */
     int reproject_every;     /* FP32-mixed: steps between H = 0 re-projections; 0 = 4096 */
     double r_switch;         /* FP32-mixed: zone r < r_switch; < 0 = none; 0 = automatic:
