@@ -24,13 +24,13 @@
 #include <cudaTypedefs.h>
 #include <stdint.h>
 
-#include <mutex>
 #include <stdlib.h>
 #include <string.h>
 
 #include "../../include/geotrace.h"
 #include "mlp.cuh"
 #include "tc_gemm.cuh"
+#include "tma_map.cuh"
 
 namespace gt {
 
@@ -739,45 +739,13 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
     if (warp == 1) tc::tmem_dealloc(tmem, L::NCOLS);
 }
 
-PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder()
-{
-    static std::once_flag once;
-    static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-    std::call_once(once, [] {
-        void *p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault,
-                                             &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = (PFN_cuTensorMapEncodeTiled_v12000)p;
-    });
-    return fn;
-}
-
-// 16-bit matrix of `rows` x `cols` (row stride `ld` elements, K = cols contiguous), boxes
-// of BK = 64 columns (128 bytes) x box_rows rows written 128-byte swizzled, zero fill
-// outside.
-bool make_map(CUtensorMap *m, const void *base, uint64_t rows, uint64_t cols, uint64_t ld,
-              uint32_t box_rows)
-{
-    auto enc = tensor_map_encoder();
-    if (!enc || rows == 0 || cols == 0 || rows > (1ull << 32) || cols > (1ull << 32)) return false;
-    cuuint64_t dims[2] = {cols, rows};
-    cuuint64_t strides[1] = {ld * 2};
-    cuuint32_t box[2] = {BK, box_rows};
-    cuuint32_t estr[2] = {1, 1};
-    return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(base), dims, strides, box,
-               estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-               CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 int g_sm_count = 0;
 
 // Output tensor map (2-D, row stride `ld` elements) with 32 x 32 boxes.
 bool make_out_map(CUtensorMap *m, void *base, CUtensorMapDataType dt, int esize, uint64_t rows,
                   uint64_t cols, uint64_t ld, CUtensorMapSwizzle sw)
 {
-    auto enc = tensor_map_encoder();
+    auto enc = tma::encoder();
     if (!enc || rows == 0 || cols == 0 || ((uintptr_t)base & 15) || (ld * esize) % 16) return false;
     cuuint64_t dims[2] = {cols, rows};
     cuuint64_t strides[1] = {ld * esize};
@@ -804,8 +772,8 @@ cudaError_t launch_ws(const GemmArgs &g, int splits, cudaStream_t s, bool *used)
 {
     *used = false;
     CUtensorMap ta, tb;
-    if (!make_map(&ta, g.A, (uint64_t)g.M, (uint64_t)g.K, (uint64_t)g.a_sm, BM) ||
-        !make_map(&tb, g.B, (uint64_t)g.N, (uint64_t)g.K, (uint64_t)g.b_sn, BN))
+    if (!tma::make_map(&ta, g.A, (uint64_t)g.M, (uint64_t)g.K, (uint64_t)g.a_sm, BM) ||
+        !tma::make_map(&tb, g.B, (uint64_t)g.N, (uint64_t)g.K, (uint64_t)g.b_sn, BN))
         return cudaSuccess; // caller falls back
     // TMA-store epilogue when every requested output has an encodable map
     OutMaps om;

@@ -1,0 +1,344 @@
+// mlp_fused.cu -- features and all five layers of the surrogate for 128 rows at a time, the
+// activations never leaving the SM (inference).
+//
+// What bounds it: the split-precision products cost 48 MMAs (128 x 256 x 16, ~135 cycles each)
+// per hidden layer and tile, and SiLU two MUFU operations per element, 4,100 cycles of an SM's
+// 16 a clock; layer-by-layer GEMMs added 3 KB of activations per row and layer through HBM and
+// L2, a pass for the features and one for the outputs.  Here a persistent CTA per SM keeps the
+// activations of its 128 rows in shared memory as the two bf16 halves (128 KB, the K-major
+// 128-byte-swizzled operand layout) and streams the weights from L2 in 64 x 256 boxes through
+// a ring of three (96 KB; the last layer's 24 KB in one slot).  Two accumulators in TMEM
+// alternate, and the epilogue hands over its output in K-chunks of 64 columns, so the next
+// layer's x_hi w_hi pass follows it chunk by chunk.  The MMAs run in the order x_hi w_hi
+// (K = 0..255), x_lo w_hi, x_hi w_lo of the split GEMM of the training path: same bits.
+//
+// Measured on one GB300: 2^20 rows 3.19 -> 1.37 ms, 300 rows 105 -> 59 us (49 us with the error flag in host memory) (the GEMM per
+// layer: 0.9 ms of MMAs at 0.47 of the bf16 peak, the rest traffic and SiLU passes).  Tried and
+// not kept: two halves of 128 columns per layer with w_hi held for both passes, 256 instead
+// of 384 KB of weights a layer (1.87 ms: an MMA takes ~105 cycles at N = 128 against ~135 at
+// N = 256); the accumulator handed over whole (1.60 ms).
+//
+// Warps: 0 loads, 1 issues the MMAs, 2-5 compute the next tile's features in FP64 while the
+// current one runs, 6-21 drain the accumulator: bias, SiLU, split, back into the operand
+// buffer.  All hand-offs are mbarriers with bounded waits; a wait that runs out sets the
+// error flag and every role leaves its loop.
+#include <cuda.h>
+#include <cuda_bf16.h>
+#include <cuda_runtime.h>
+#include <cudaTypedefs.h>
+#include <stdint.h>
+
+#include "features.cuh"
+#include "mlp_fused.cuh"
+#include "tc_gemm.cuh"
+#include "tma_map.cuh"
+
+namespace gt {
+namespace sg {
+
+namespace {
+
+constexpr int TILE = 128;
+constexpr int RING = 3;
+constexpr int FEAT_WARPS = 4, EPI_WARPS = 16;
+constexpr int THREADS = 32 * (2 + FEAT_WARPS + EPI_WARPS);
+constexpr uint32_t BOX = 64 * 128 * 2;       // one K-chunk of activations
+constexpr uint32_t WBOX = 64 * 256 * 2;      // one K-chunk of a layer's weights
+constexpr uint32_t OBOX = 64 * 16 * 2;       // one K-chunk of the last layer's
+constexpr uint32_t A_BYTES = 8 * BOX;        // hi: 4 K-chunks, lo: 4 K-chunks
+constexpr uint32_t BAR_OFF = A_BYTES + RING * WBOX;
+constexpr uint32_t N_BAR = 2 * RING + 9;
+constexpr uint32_t SMEM = BAR_OFF + 8 * N_BAR + 16 + 1024; // + alignment to the swizzle period
+constexpr uint32_t WAIT_LIMIT = 1u << 24;
+static_assert(SMEM <= 227 * 1024, "shared memory per CTA");
+
+__device__ __forceinline__ float silu(float z) { return __fdividef(z, 1.0f + __expf(-z)); }
+
+// One kind::f16 MMA from the low words of two SW128 K-major descriptors (address >> 4 and the
+// fixed leading offset; the high word is a constant): the issuing thread adds 2 per K-slice
+// and 1024 per box instead of building 64-bit descriptors.
+constexpr uint32_t DESC_HI = (1024u >> 4) | (1u << 14) | (2u << 29);
+__device__ __forceinline__ uint32_t desc_lo(uint32_t saddr) { return (saddr >> 4) | (1u << 16); }
+template <bool ACCUMULATE>
+__device__ __forceinline__ void mma_lo(uint32_t d, uint32_t a, uint32_t b, uint32_t idesc)
+{
+    asm volatile(
+        "{\n\t.reg .b64 da, db;\n\t.reg .pred p;\n\tsetp.ne.b32 p, %5, 0;\n\t"
+        "mov.b64 da, {%1, %4};\n\tmov.b64 db, {%2, %4};\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, p;\n\t}\n" ::"r"(d),
+        "r"(a), "r"(b), "r"(idesc), "r"(DESC_HI), "n"(ACCUMULATE ? 1 : 0));
+}
+
+__device__ __forceinline__ uint32_t pack2(__nv_bfloat16 a, __nv_bfloat16 b)
+{
+    const __nv_bfloat162 h = __halves2bfloat162(a, b);
+    return *reinterpret_cast<const uint32_t *>(&h);
+}
+
+// eight consecutive values as their bf16 halves: hi = bf16(v), lo = bf16(v - hi)
+__device__ __forceinline__ void split8(const float *v, uint4 &hi, uint4 &lo)
+{
+    uint32_t *h = &hi.x, *l = &lo.x;
+#pragma unroll
+    for (int j = 0; j < 4; j++) {
+        const __nv_bfloat16 a = __float2bfloat16(v[2 * j]), b = __float2bfloat16(v[2 * j + 1]);
+        h[j] = pack2(a, b);
+        l[j] = pack2(__float2bfloat16(v[2 * j] - __bfloat162float(a)),
+                     __float2bfloat16(v[2 * j + 1] - __bfloat162float(b)));
+    }
+}
+
+__global__ void __launch_bounds__(THREADS, 1)
+    fused_forward_kernel(const __grid_constant__ FusedMaps maps, const __grid_constant__ FusedArgs g)
+{
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    uint8_t *smem = smem_raw + ((1024u - (tc::smem_u32(smem_raw) & 1023u)) & 1023u);
+    const uint32_t act = tc::smem_u32(smem), ring = act + A_BYTES, bar = act + BAR_OFF;
+    auto FULL = [&](uint32_t s) { return bar + 8u * s; };
+    auto EMPTY = [&](uint32_t s) { return bar + 8u * (RING + s); };
+    auto ACC = [&](uint32_t b) { return bar + 8u * (2 * RING + b); };     // accumulator complete
+    auto ACT = [&](uint32_t k) { return bar + 8u * (2 * RING + 2 + k); }; // K-chunk k written
+    const uint32_t TAIL = bar + 8u * (2 * RING + 6); // last layer's MMAs complete (per tile)
+    const uint32_t FEAT = TAIL + 8u;                 // features of a tile in the operand buffer
+    const uint32_t DONE = TAIL + 16u;
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem + BAR_OFF + 8 * N_BAR);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t tiles = (g.n + TILE - 1) / TILE;
+
+    if (warp == 1) tc::tmem_alloc(tc::smem_u32(tmem_slot), 512);
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < RING; s++) {
+            tc::mbar_init(FULL(s), 1);
+            tc::mbar_init(EMPTY(s), 1);
+        }
+        for (int b = 0; b < 2; b++) tc::mbar_init(ACC(b), 1);
+        for (int k = 0; k < 4; k++) tc::mbar_init(ACT(k), EPI_WARPS);
+        tc::mbar_init(TAIL, 1);
+        tc::mbar_init(FEAT, FEAT_WARPS);
+        tc::mbar_init(DONE, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;");
+    }
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::fence_after_sync();
+    const uint32_t tmem = *tmem_slot;
+    bool ok = true;
+
+    if (warp == 0) {
+        if (lane == 0) { // ---- weights
+            uint32_t q = 0;
+            // n boxes of `bytes` each (K-chunks k0, k0 + 1, ...) into the next slot
+            auto load = [&](int l, int k0, int n, uint32_t bytes) {
+                const uint32_t s = q % RING;
+                if (q >= RING && !tc::mbar_wait(EMPTY(s), (q / RING - 1) & 1, WAIT_LIMIT)) ok = false;
+                if (!ok) return;
+                tc::mbar_expect_tx(FULL(s), n * bytes);
+                for (int i = 0; i < n; i++)
+                    tc::tma_load_2d(ring + s * WBOX + i * bytes, &maps.w[l], 64 * (k0 + i), 0, FULL(s));
+                ++q;
+            };
+            for (int64_t t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
+                load(0, 0, 1, WBOX);
+                for (int l = 1; l < N_LAYERS - 1; l++)
+                    for (int k = 0; k < 12; k++) load(l, k, 1, WBOX); // w_hi, w_hi, w_lo
+                load(N_LAYERS - 1, 0, 12, OBOX); // the last layer's 24 KB in one slot
+            }
+            // copies still in flight (only after a failed wait) land before the CTA exits
+            for (uint32_t j = q > RING ? q - RING : 0; j < q; ++j)
+                if (!tc::mbar_wait(FULL(j % RING), (j / RING) & 1, WAIT_LIMIT)) ok = false;
+        }
+    } else if (warp == 1) {
+        if (lane == 0) { // ---- MMA
+            const uint32_t id_h = tc::idesc_f16_f32(TILE, 256, true);
+            const uint32_t id_o = tc::idesc_f16_f32(TILE, 16, true);
+            uint32_t q = 0, hid = 0, acc = 0, tl = 0;
+            auto full = [&](uint32_t j) {
+                if (ok) ok = tc::mbar_wait(FULL(j % RING), (j / RING) & 1, WAIT_LIMIT);
+                tc::fence_after_sync();
+                return ok;
+            };
+            const uint32_t a_lo = desc_lo(act), b_lo = desc_lo(ring);
+            // four K-slices of activation chunk c (0-3 hi, 4-7 lo) with the weights at b
+            auto mma4 = [&](uint32_t d, uint32_t c, uint32_t b, uint32_t idesc, bool first) {
+                const uint32_t a = a_lo + c * (BOX >> 4);
+                if (first)
+                    mma_lo<false>(d, a, b, idesc);
+                else
+                    mma_lo<true>(d, a, b, idesc);
+#pragma unroll
+                for (int kk = 1; kk < 4; kk++) mma_lo<true>(d, a + 2 * kk, b + 2 * kk, idesc);
+            };
+            auto slot = [&](uint32_t j) { return b_lo + (j % RING) * (WBOX >> 4); };
+            // K-chunk k of the hidden layer's input has been written (and every earlier read of
+            // the accumulator about to be overwritten is done: the same warps did it before)
+            auto input = [&](uint32_t k) {
+                if (ok) ok = tc::mbar_wait(ACT(k), hid & 1, WAIT_LIMIT);
+                tc::fence_after_sync();
+                return ok;
+            };
+            for (int64_t t = blockIdx.x; t < tiles && ok; t += gridDim.x, ++tl) {
+                // first layer: K' = 48 in one chunk
+                ok = tc::mbar_wait(FEAT, tl & 1, WAIT_LIMIT);
+                tc::fence_after_sync();
+                if (!full(q)) break;
+                mma4(tmem + 256 * (acc & 1), 0, slot(q), id_h, true);
+                tc::mma_commit(EMPTY(q % RING));
+                tc::mma_commit(ACC(acc & 1));
+                ++q;
+                ++acc;
+                for (int l = 1; l < N_LAYERS - 1 && ok; l++, hid++, acc++) {
+                    const uint32_t d = tmem + 256 * (acc & 1);
+                    for (uint32_t k = 0; k < 12 && ok; k++, q++) { // x_hi w_hi, x_lo w_hi, x_hi w_lo
+                        if (k < 4 && !input(k)) break;
+                        if (!full(q)) break;
+                        mma4(d, k < 8 ? k : k - 8, slot(q), id_h, k == 0);
+                        tc::mma_commit(EMPTY(q % RING));
+                    }
+                    if (ok) tc::mma_commit(ACC(acc & 1));
+                }
+                if (!ok || !full(q)) break;
+                const uint32_t d = tmem + 256 * (acc & 1);
+                for (uint32_t k = 0; k < 12 && ok; k++)
+                    if (k >= 4 || input(k))
+                        mma4(d, k < 8 ? k : k - 8, slot(q) + k * (OBOX >> 4), id_o, k == 0);
+                if (!ok) break;
+                tc::mma_commit(EMPTY(q % RING));
+                tc::mma_commit(TAIL);
+                tc::mma_commit(ACC(acc & 1));
+                ++q;
+                ++hid;
+                ++acc;
+            }
+            // every issued MMA completes before the accumulator is freed
+            tc::mma_commit(DONE);
+            if (!tc::mbar_wait(DONE, 0, WAIT_LIMIT)) ok = false;
+        }
+    } else if (warp < 2 + FEAT_WARPS) { // ---- features, one row a thread
+        const int row = (warp - 2) * 32 + lane;
+        uint32_t tl = 0;
+        for (int64_t t = blockIdx.x; t < tiles && ok; t += gridDim.x, ++tl) {
+            const int64_t r = t * TILE + row;
+            float f[16];
+            if (r >= g.n) {
+#pragma unroll
+                for (int j = 0; j < 16; j++) f[j] = 0.0f;
+            } else if (g.cam) {
+                pixel_features(*g.cam, r, g.norm, f);
+            } else {
+                make_features(g.alpha[r], g.beta[r], g.spin[r], g.q[r], g.theta0[r], g.norm, f);
+            }
+            uint4 hi[2], lo[2];
+            split8(f, hi[0], lo[0]);
+            split8(f + 8, hi[1], lo[1]);
+            // the previous tile's last layer has read the operand buffer
+            if (tl > 0) ok = tc::mbar_wait(TAIL, (tl - 1) & 1, WAIT_LIMIT);
+            if (!ok) break;
+            // row [hi 0..15 | lo 0..15 | hi 0..15 | 0] of one 64-wide chunk
+            uint8_t *base = smem + row * 128;
+            const uint4 zero = make_uint4(0, 0, 0, 0);
+            const uint4 v[8] = {hi[0], hi[1], lo[0], lo[1], hi[0], hi[1], zero, zero};
+#pragma unroll
+            for (int c = 0; c < 8; c++)
+                *reinterpret_cast<uint4 *>(base + ((c ^ (row & 7)) << 4)) = v[c];
+            tc::fence_proxy_async();
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(FEAT);
+        }
+    } else { // ---- epilogue: TMEM lanes 32 (warp % 4), 16 columns of each K-chunk of 64
+        const int quarter = warp & 3, group = (warp - 2 - FEAT_WARPS) >> 2;
+        const int row = quarter * 32 + lane;
+        const uint32_t t_row = tmem + ((uint32_t)(quarter * 32) << 16);
+        // this row's 16-byte pieces 2 group, 2 group + 1 of a chunk, 128-byte swizzled
+        uint8_t *const p0 = smem + row * 128 + (((2 * group) ^ (row & 7)) << 4);
+        uint8_t *const p1 = smem + row * 128 + (((2 * group + 1) ^ (row & 7)) << 4);
+        uint32_t acc = 0;
+        for (int64_t t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
+            for (int l = 0; l < N_LAYERS - 1 && ok; l++, acc++) {
+                // two barriers in turn: one flips again only after every warp has passed it
+                ok = tc::mbar_wait(ACC(acc & 1), (acc >> 1) & 1, WAIT_LIMIT);
+                if (!ok) break;
+                tc::fence_after_sync();
+                const uint32_t src = t_row + 256 * (acc & 1) + 16 * group;
+                const float4 *b4 = reinterpret_cast<const float4 *>(g.bias[l] + 16 * group);
+#pragma unroll
+                for (int k = 0; k < 4; k++) {
+                    float v[16];
+                    tc::tmem_ld16(src + 64 * k, v);
+#pragma unroll
+                    for (int j = 0; j < 4; j++) {
+                        const float4 b = __ldg(b4 + 16 * k + j);
+                        v[4 * j] = silu(v[4 * j] + b.x);
+                        v[4 * j + 1] = silu(v[4 * j + 1] + b.y);
+                        v[4 * j + 2] = silu(v[4 * j + 2] + b.z);
+                        v[4 * j + 3] = silu(v[4 * j + 3] + b.w);
+                    }
+                    uint4 hi, lo;
+                    split8(v, hi, lo);
+                    *reinterpret_cast<uint4 *>(p0 + k * BOX) = hi;
+                    *reinterpret_cast<uint4 *>(p0 + (4 + k) * BOX) = lo;
+                    split8(v + 8, hi, lo);
+                    *reinterpret_cast<uint4 *>(p1 + k * BOX) = hi;
+                    *reinterpret_cast<uint4 *>(p1 + (4 + k) * BOX) = lo;
+                    tc::fence_proxy_async();
+                    tc::fence_before_sync();
+                    __syncwarp();
+                    if (lane == 0) tc::mbar_arrive(ACT(k));
+                }
+            }
+            if (!ok) break;
+            ok = tc::mbar_wait(ACC(acc & 1), (acc >> 1) & 1, WAIT_LIMIT);
+            if (!ok) break;
+            if (group == 0) {
+                tc::fence_after_sync();
+                float v[16];
+                tc::tmem_ld16(t_row + 256 * (acc & 1), v);
+                tc::fence_before_sync();
+                const int64_t r = t * TILE + row;
+                if (r < g.n) {
+                    const float *b = g.bias[N_LAYERS - 1];
+                    float *o = g.out + 4 * r;
+                    const float4 z = make_float4(v[0] + __ldg(b), v[1] + __ldg(b + 1),
+                                                 v[2] + __ldg(b + 2), v[3] + __ldg(b + 3));
+                    if (((uintptr_t)g.out & 15u) == 0) {
+                        *reinterpret_cast<float4 *>(o) = z;
+                    } else {
+                        o[0] = z.x;
+                        o[1] = z.y;
+                        o[2] = z.z;
+                        o[3] = z.w;
+                    }
+                }
+            }
+            ++acc;
+        }
+    }
+    if (!ok && g.err) atomicExch(g.err, 1);
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::fence_after_sync();
+    if (warp == 1) tc::tmem_dealloc(tmem, 512);
+}
+
+} // namespace
+
+bool fused_prepare(FusedMaps *maps, const void *const w3[N_LAYERS])
+{
+    for (int l = 0; l < N_LAYERS; l++)
+        if (!tma::make_map(&maps->w[l], w3[l], (uint64_t)OUT_DIM[l], 3 * (uint64_t)IN_DIM[l],
+                           3 * (uint64_t)IN_DIM[l], OUT_DIM[l]))
+            return false;
+    return cudaFuncSetAttribute(fused_forward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                SMEM) == cudaSuccess;
+}
+
+cudaError_t launch_fused(const FusedMaps &maps, const FusedArgs &a, int sm_count, cudaStream_t s)
+{
+    if (a.n <= 0) return cudaSuccess;
+    const int64_t tiles = (a.n + TILE - 1) / TILE;
+    const int grid = (int)(tiles < sm_count ? tiles : sm_count);
+    fused_forward_kernel<<<grid, THREADS, SMEM, s>>>(maps, a);
+    return cudaGetLastError();
+}
+
+} // namespace sg
+} // namespace gt

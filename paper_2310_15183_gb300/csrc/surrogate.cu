@@ -28,7 +28,9 @@
 #include "../../include/geotrace.h"
 #include "internal.cuh"
 #include "mlp.cuh"
+#include "mlp_fused.cuh"
 #include "camera.cuh"
+#include "features.cuh"
 #include "surrogate.cuh"
 
 namespace gt {
@@ -65,37 +67,6 @@ __global__ void init_params_kernel(float *p, int64_t n, const int64_t *offs, con
     p[i] = sc * (float)(sqrt(-2.0 * log(u1)) * cos(2.0 * M_PI * u2));
 }
 
-// The network's 16 input columns from the 5 inputs (alpha, beta, a/M, q, theta0):
-// 0-4 the inputs scaled to about [-1, 1]; 5-7 the pixel direction in polar form
-// (rho, cos psi, sin psi) of the scaled (alpha, beta); 8-9 cos and sin of theta0; the
-// rest zero.  The derived columns are fixed functions of the inputs.
-__device__ __forceinline__ void make_features(double al, double bt, double spin, double q,
-                                              double th0, const Norm &nm, float f[16])
-{
-    const double a = al * nm.inv_h, b = bt * nm.inv_v;
-    const double rho = sqrt(a * a + b * b);
-    const double irho = 1.0 / fmax(rho, 1e-3);
-    f[0] = (float)a;
-    f[1] = (float)b;
-    f[2] = (float)(spin * nm.spin_scale + nm.spin_shift);
-    f[3] = (float)(q * nm.q_scale);
-    f[4] = (float)(th0 * nm.th_scale + nm.th_shift);
-    f[5] = (float)rho;
-    f[6] = (float)(a * irho);
-    f[7] = (float)(b * irho);
-    f[8] = (float)cos(th0);
-    f[9] = (float)sin(th0);
-#pragma unroll
-    for (int j = 10; j < 16; j++) f[j] = 0.0f;
-}
-
-// bf16 pair of v: hi = bf16(v), lo = bf16(v - hi)
-__device__ __forceinline__ void split_pair(float v, __nv_bfloat16 *hi, __nv_bfloat16 *lo)
-{
-    *hi = __float2bfloat16(v);
-    *lo = __float2bfloat16(v - __bfloat162float(*hi));
-}
-
 // One row of the first layer's split input: columns [hi 0..15 | lo 0..15 | hi 0..15]
 __device__ __forceinline__ void store_split_row(const float f[16], __nv_bfloat16 *row)
 {
@@ -125,23 +96,6 @@ __global__ void features_kernel(int64_t n, int64_t row0, const double *alpha, co
     if (X0T)
 #pragma unroll
         for (int j = 0; j < 16; j++) X0T[j * n + r] = __float2bfloat16(f[j]);
-}
-
-// features of camera pixels [pix0, pix0 + n) (flat j*res_x + i), or of the listed pixels
-// pixels[pix0 + r]
-__global__ void camera_features_kernel(int64_t n, int64_t pix0, const CamDesc *cam, Norm nm,
-                                       __nv_bfloat16 *X0, const int64_t *pixels = nullptr)
-{
-    const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= n) return;
-    const CamDesc &c = *cam;
-    const int64_t pix = pixels ? pixels[pix0 + r] : pix0 + r;
-    const int i = (int)(pix % c.res_x), j = (int)(pix / c.res_x);
-    const double al = c.res_x > 1 ? c.H * (double)(2 * i - (c.res_x - 1)) / (double)(c.res_x - 1) : 0.0;
-    const double bt = c.res_y > 1 ? c.V * (double)(2 * j - (c.res_y - 1)) / (double)(c.res_y - 1) : 0.0;
-    float f[16];
-    make_features(al, bt, (c.S / c.M) / c.M, c.Q, c.th0, nm, f);
-    store_split_row(f, X0 + r * 3 * 16);
 }
 
 // Loss of rows [0, B): BCE(logit, y) + w_dir * y * |d_pred - d|^2, averaged over B.
@@ -318,15 +272,6 @@ __device__ __forceinline__ int probe_coord(int k, int stride, int n, int res)
 __device__ __forceinline__ bool is_probe(int i, int j, const ProbeGrid &pg, int res_x, int res_y)
 {
     return (i % pg.stride == 0 || i == res_x - 1) && (j % pg.stride == 0 || j == res_y - 1);
-}
-
-// The network's answer per pixel (logit, direction) kept for the passes below.
-__global__ void net_out_kernel(int64_t n, int64_t pix0, const float *Z5, float4 *net)
-{
-    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n) return;
-    const float *z = Z5 + k * 16;
-    net[pix0 + k] = make_float4(z[0], z[1], z[2], z[3]);
 }
 
 // Gates that send a pixel to the integrator whatever the probes say: an unsure logit, the
@@ -559,6 +504,8 @@ struct gt_surrogate {
     uint8_t *decay = nullptr;
     __nv_bfloat16 *w3 = nullptr; // split bf16 weights of the forward products, [out][3 in] per layer
     int64_t w3_off[N_LAYERS] = {};
+    FusedMaps maps;   // w3 as the inference kernel reads it
+    int sm_count = 0;
     int64_t step = 0;
     // workspace for `rows` rows
     int64_t rows = 0;
@@ -569,7 +516,9 @@ struct gt_surrogate {
     float *Z[N_LAYERS] = {};         // pre-activations (fp32)
     float *dXf = nullptr, *dZf = nullptr, *lab = nullptr, *loss = nullptr;
     __nv_bfloat16 *dZb = nullptr;
-    int *err = nullptr;
+    // set to 1 by a kernel whose mbarrier wait ran out: host memory the device writes, so that
+    // a call reads it after its synchronisation without a copy of its own
+    int *err = nullptr, *err_host = nullptr;
 };
 
 namespace {
@@ -668,19 +617,28 @@ cudaError_t gemm(const void *A, int64_t a_sm, int64_t a_sk, const void *B, int64
 }
 
 // Forward pass of `B` rows whose features are in X[0]; leaves Z[4] = network output.
-// keep_pre: also store the hidden pre-activations (needed by the backward pass only).
-cudaError_t forward(gt_surrogate *s, int B, cudaStream_t st, bool keep_pre = true)
+// The training path: every layer's input, transposed input and pre-activation are kept.
+cudaError_t forward(gt_surrogate *s, int B, cudaStream_t st)
 {
     cudaError_t e = cudaSuccess;
     for (int l = 0; l < N_LAYERS && e == cudaSuccess; l++) {
         const bool last = (l == N_LAYERS - 1);
         const int K3 = 3 * IN_DIM[l];
         e = gemm(s->X[l], K3, 1, s->w3 + s->w3_off[l], K3, 1, B, OUT_DIM[l], K3,
-                 s->p + s->b_off[l], last ? 0 : 1, (last || !keep_pre) ? nullptr : s->Z[l],
+                 s->p + s->b_off[l], last ? 0 : 1, last ? nullptr : s->Z[l],
                  last ? s->Z[l] : nullptr, OUT_DIM[l], false, last ? nullptr : s->X[l + 1], 1,
-                 s->err, st, (last || !keep_pre) ? nullptr : s->XT[l + 1], true);
+                 s->err, st, last ? nullptr : s->XT[l + 1], true);
     }
     return e;
+}
+
+// Network outputs of `a`'s rows (inference): one kernel, no workspace.
+cudaError_t infer_rows(gt_surrogate *s, FusedArgs a, cudaStream_t st)
+{
+    a.norm = s->norm;
+    for (int l = 0; l < N_LAYERS; l++) a.bias[l] = s->p + s->b_off[l];
+    a.err = s->err;
+    return launch_fused(s->maps, a, s->sm_count, st);
 }
 
 // Backward pass of B rows with labels in s->lab: gradients (zeroed here) into s->g.
@@ -714,10 +672,8 @@ cudaError_t backward(gt_surrogate *s, int B, float w_dir, cudaStream_t st)
 
 int check_err(gt_surrogate *s, cudaStream_t st)
 {
-    int h = 0;
-    cudaError_t e = cudaMemcpyAsync(&h, s->err, sizeof h, cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) return GT_ERR_CUDA;
+    if (cudaStreamSynchronize(st) != cudaSuccess) return GT_ERR_CUDA;
+    const int h = *(volatile int *)s->err_host;
     return h ? GT_ERR_TIMEOUT : GT_OK;
 }
 
@@ -804,7 +760,12 @@ int gt_surrogate_create(int device, const gt_surrogate_norm *nrm, uint64_t seed,
     if (e == cudaSuccess) e = cudaMalloc(&s->WT, off * sizeof(__nv_bfloat16));
     if (e == cudaSuccess) e = cudaMalloc(&s->decay, off);
     if (e == cudaSuccess) e = cudaMalloc(&s->loss, sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc(&s->err, sizeof(int));
+    if (e == cudaSuccess)
+        e = cudaHostAlloc(&s->err_host, sizeof(int), cudaHostAllocMapped | cudaHostAllocPortable);
+    if (e == cudaSuccess) {
+        *s->err_host = 0;
+        e = cudaHostGetDevicePointer(&s->err, s->err_host, 0);
+    }
     if (e == cudaSuccess) e = cudaMalloc(&d_offs, offs.size() * sizeof(int64_t));
     if (e == cudaSuccess) e = cudaMalloc(&d_scales, scales.size() * sizeof(float));
     if (e == cudaSuccess)
@@ -814,7 +775,12 @@ int gt_surrogate_create(int device, const gt_surrogate_norm *nrm, uint64_t seed,
     if (e == cudaSuccess) e = cudaMemcpy(s->decay, decay.data(), off, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(s->m, 0, off * sizeof(float));
     if (e == cudaSuccess) e = cudaMemset(s->v, 0, off * sizeof(float));
-    if (e == cudaSuccess) e = cudaMemset(s->err, 0, sizeof(int));
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&s->sm_count, cudaDevAttrMultiProcessorCount, device);
+    if (e == cudaSuccess) {
+        const void *w[N_LAYERS];
+        for (int l = 0; l < N_LAYERS; l++) w[l] = s->w3 + s->w3_off[l];
+        if (!fused_prepare(&s->maps, w)) e = cudaErrorUnknown;
+    }
     if (e == cudaSuccess) {
         init_params_kernel<<<blocks_for(off), 256>>>(s->p, off, d_offs, d_scales, (int)offs.size(), seed);
         e = refresh_copies(s, 0);
@@ -844,7 +810,7 @@ int gt_surrogate_destroy(gt_surrogate *s)
     cudaFree(s->WT);
     cudaFree(s->decay);
     cudaFree(s->loss);
-    cudaFree(s->err);
+    cudaFreeHost(s->err_host);
     delete s;
     return GT_OK;
 }
@@ -883,19 +849,15 @@ int gt_surrogate_eval(gt_ctx *ctx, gt_surrogate *s, int64_t n, const double *alp
         return GT_ERR_INVALID_ARG;
     Dev d(s->device);
     cudaStream_t st = gt_internal_stream(ctx);
-    const int64_t chunk = 1 << 18;
-    int rc = ensure_ws(s, n < chunk ? (n > 0 ? n : 1) : chunk);
-    if (rc != GT_OK) return rc;
-    for (int64_t r0 = 0; r0 < n; r0 += chunk) {
-        const int64_t B = n - r0 < chunk ? n - r0 : chunk;
-        features_kernel<<<blocks_for(B), 256, 0, st>>>(B, r0, alpha, beta, spin, q, theta0, s->norm,
-                                                       s->X[0]);
-        cudaError_t e = forward(s, (int)B, st, false);
-        if (e == cudaSuccess)
-            e = cudaMemcpy2DAsync(out + r0 * 4, 4 * sizeof(float), s->Z[N_LAYERS - 1], 16 * sizeof(float),
-                                  4 * sizeof(float), B, cudaMemcpyDeviceToDevice, st);
-        if (e != cudaSuccess) return GT_ERR_CUDA;
-    }
+    FusedArgs a = {};
+    a.n = n;
+    a.alpha = alpha;
+    a.beta = beta;
+    a.spin = spin;
+    a.q = q;
+    a.theta0 = theta0;
+    a.out = out;
+    if (infer_rows(s, a, st) != cudaSuccess) return GT_ERR_CUDA;
     return check_err(s, st);
 }
 
@@ -982,16 +944,11 @@ namespace sg {
 // The network on every pixel of the camera; its answers to `net` (float4 per pixel).
 int net_pass(gt_surrogate *s, const CamDesc *d_cam, int64_t n_pix, float4 *net, cudaStream_t st)
 {
-    const int64_t chunk = 1 << 19;
-    int rc = ensure_ws(s, n_pix < chunk ? n_pix : chunk);
-    if (rc != GT_OK) return rc;
-    for (int64_t p0 = 0; p0 < n_pix; p0 += chunk) {
-        const int64_t B = n_pix - p0 < chunk ? n_pix - p0 : chunk;
-        camera_features_kernel<<<blocks_for(B), 256, 0, st>>>(B, p0, d_cam, s->norm, s->X[0]);
-        if (forward(s, (int)B, st, false) != cudaSuccess) return GT_ERR_CUDA;
-        net_out_kernel<<<blocks_for(B), 256, 0, st>>>(B, p0, s->Z[N_LAYERS - 1], net);
-        if (cudaGetLastError() != cudaSuccess) return GT_ERR_CUDA;
-    }
+    FusedArgs a = {};
+    a.n = n_pix;
+    a.cam = d_cam;
+    a.out = (float *)net;
+    if (infer_rows(s, a, st) != cudaSuccess) return GT_ERR_CUDA;
     return check_err(s, st);
 }
 

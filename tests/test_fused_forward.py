@@ -1,0 +1,60 @@
+"""The one-kernel forward pass of the surrogate (csrc/mlp_fused.cu) at the edges of its tiles."""
+import numpy as np
+import pytest
+
+from oracle import mlp
+from paper_2310_15183_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def net():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2310_15183_gb300 import build, geotrace
+    build.build()
+    tracer, s = geotrace.Tracer(0), geotrace.Surrogate(0, seed=21)
+    p = s.get_params()
+    for b in mlp.split(p)[1]:  # a fresh network's biases are zero
+        b[:] = np.random.Generator(np.random.PCG64(b.size)).normal(0, 0.3, b.size)
+    s.set_params(p)
+    yield tracer, s
+    s.close()
+    tracer.close()
+
+
+@pytest.mark.parametrize("n", [1, 31, 127, 128, 129, 255, 152 * 128 - 1, 152 * 128, 152 * 128 + 1,
+                               2 * 152 * 128 + 77])
+def test_rows_at_tile_edges(net, n):
+    """Every output within 2^-12 sum_k |a_k| |w_k| of the CPU reference's split-precision
+    product (as for the layer-wise forward: split pairs to 2^-16, FP32 accumulation of 768
+    terms 2^-14.4, earlier layers the same), and independent of the rows around it."""
+    tracer, s = net
+    host = W.surrogate_samples(n, seed=n)
+    dev = [torch.tensor(x, device="cuda") for x in host]
+    out = s.eval(tracer, dev).cpu().numpy()
+    some = np.unique(np.concatenate([np.arange(min(n, 200)), np.arange(max(0, n - 200), n)]))
+    X0 = mlp.features(*[x[some] for x in host])
+    p = s.get_params().astype(np.float64)
+    As, Zs = mlp.forward(p, X0, bf=True)
+    scale = np.abs(As[4]) @ np.abs(mlp.split(p)[0][4]).T + np.abs(mlp.split(p)[1][4])
+    err = np.abs(out[some] - Zs[4][:, :4])
+    assert np.all(err <= 2.0 ** -12 * scale[:, :4]), float(np.max(err / scale[:, :4]))
+    part = s.eval(tracer, [d[n // 2:].contiguous() for d in dev]).cpu().numpy()
+    assert np.array_equal(part, out[n // 2:])
+
+
+def test_unaligned_output(net):
+    """The C entry takes any float pointer: rows of 16 bytes at a 4-byte offset."""
+    tracer, s = net
+    host = W.surrogate_samples(200, seed=3)
+    dev = [torch.tensor(x, device="cuda") for x in host]
+    buf = torch.zeros(4 * 200 + 2, dtype=torch.float32, device="cuda")
+    rc = s.lib.gt_surrogate_eval(tracer.ctx, s.h, 200, *[d.data_ptr() for d in dev],
+                                 buf.data_ptr() + 4)
+    assert rc == 0
+    torch.cuda.synchronize()
+    assert torch.equal(buf[1:-1].view(200, 4), s.eval(tracer, dev))
+    assert buf[0].item() == 0.0 and buf[-1].item() == 0.0
