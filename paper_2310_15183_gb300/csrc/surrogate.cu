@@ -37,8 +37,6 @@ namespace gt {
 namespace sg {
 
 // ------------------------------------------------------------------ kernels
-__device__ __forceinline__ float sigmoidf(float z) { return 1.0f / (1.0f + __expf(-z)); }
-
 // counter-based normal deviates: splitmix64 -> two uniforms -> Box-Muller
 __device__ __forceinline__ uint64_t splitmix64(uint64_t x)
 {
@@ -67,141 +65,46 @@ __global__ void init_params_kernel(float *p, int64_t n, const int64_t *offs, con
     p[i] = sc * (float)(sqrt(-2.0 * log(u1)) * cos(2.0 * M_PI * u2));
 }
 
-// One row of the first layer's split input: columns [hi 0..15 | lo 0..15 | hi 0..15]
-__device__ __forceinline__ void store_split_row(const float f[16], __nv_bfloat16 *row)
-{
-#pragma unroll
-    for (int j = 0; j < 16; j++) {
-        __nv_bfloat16 hi, lo;
-        split_pair(f[j], &hi, &lo);
-        row[j] = hi;
-        row[16 + j] = lo;
-        row[32 + j] = hi;
-    }
-}
+// Offsets of the layers in the flat parameter vector and in the split weights.
+struct Offsets {
+    int64_t w[N_LAYERS], b[N_LAYERS], w3[N_LAYERS];
+};
 
-// features of samples [row0, row0 + n): X0[r, 0..47] (split bf16, input of the forward
-// product) and optionally X0T (bf16 of the features, transposed, input of the
-// weight-gradient product)
-__global__ void features_kernel(int64_t n, int64_t row0, const double *alpha, const double *beta,
-                                const double *spin, const double *q, const double *theta0,
-                                Norm nm, __nv_bfloat16 *X0, __nv_bfloat16 *X0T = nullptr)
-{
-    const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= n) return;
-    const int64_t k = row0 + r;
-    float f[16];
-    make_features(alpha[k], beta[k], spin[k], q[k], theta0[k], nm, f);
-    store_split_row(f, X0 + r * 3 * 16);
-    if (X0T)
-#pragma unroll
-        for (int j = 0; j < 16; j++) X0T[j * n + r] = __float2bfloat16(f[j]);
-}
-
-// Loss of rows [0, B): BCE(logit, y) + w_dir * y * |d_pred - d|^2, averaged over B.
-// labels: [B x 4] = (y, dx, dy, dz).  Writes dZ5 (fp32 and bf16, 16 columns, zeros
-// beyond 4) and accumulates the loss sum.
-__global__ void head_kernel(int B, const float *Z5, const float *labels, float w_dir, float inv_b,
-                            float *dZ5f, __nv_bfloat16 *dZ5b, __nv_bfloat16 *dZ5T, float *loss_acc)
-{
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    float l = 0.0f;
-    if (r < B) {
-        const float *z = Z5 + (int64_t)r * 16;
-        const float *lab = labels + (int64_t)r * 4;
-        const float y = lab[0];
-        const float zl = z[0];
-        // numerically stable BCE with logits
-        l = fmaxf(zl, 0.0f) - zl * y + log1pf(__expf(-fabsf(zl)));
-        float g[16];
-        g[0] = (sigmoidf(zl) - y) * inv_b;
-        for (int j = 1; j < 4; j++) {
-            const float d = z[j] - lab[j];
-            l += w_dir * y * d * d;
-            g[j] = 2.0f * w_dir * y * d * inv_b;
-        }
-        for (int j = 4; j < 16; j++) g[j] = 0.0f;
-        for (int j = 0; j < 16; j++) {
-            dZ5f[(int64_t)r * 16 + j] = g[j];
-            dZ5b[(int64_t)r * 16 + j] = __float2bfloat16(g[j]);
-            dZ5T[(int64_t)j * B + r] = __float2bfloat16(g[j]);
-        }
-    }
-    // warp-reduce the loss, one atomic per warp
-    for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
-    if ((threadIdx.x & 31) == 0) atomicAdd(loss_acc, l);
-}
-
-// dZ = dX * SiLU'(Z), SiLU'(z) = s (1 + z (1 - s)), s = sigmoid(z)
-// dZT is the transposed (cols x rows) bf16 copy used by the weight-gradient product.
-__global__ void silu_backward_kernel(int64_t rows, int cols, const float *dX, const float *Z,
-                                     float *dZf, __nv_bfloat16 *dZb, __nv_bfloat16 *dZT)
-{
-    // consecutive threads take consecutive rows of one column: coalesced transposed stores
-    const int64_t n = rows * cols;
-    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n) return;
-    const int64_t r = k % rows, c = k / rows;
-    const int64_t i = r * cols + c;
-    const float z = Z[i];
-    const float s = sigmoidf(z);
-    const float g = dX[i] * s * (1.0f + z * (1.0f - s));
-    dZf[i] = g;
-    dZb[i] = __float2bfloat16(g);
-    dZT[c * rows + r] = __float2bfloat16(g);
-}
-
-// WT[l] = bf16 transpose of the fp32 weights [out][in] -> [in][out]
-__global__ void weights_t_kernel(const float *W, int out_dim, int in_dim, __nv_bfloat16 *WT)
-{
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= out_dim * in_dim) return;
-    const int o = k / in_dim, i = k % in_dim;
-    WT[(int64_t)i * out_dim + o] = __float2bfloat16(W[k]);
-}
-
-// out[c] += sum_r M[r, c]  (rows x cols, row-major)
-__global__ void colsum_kernel(const float *Mx, int64_t rows, int cols, float *out)
-{
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= cols) return;
-    const int64_t per = (rows + gridDim.y - 1) / gridDim.y;
-    const int64_t r0 = blockIdx.y * per, r1 = min(rows, r0 + per);
-    float s = 0.0f;
-    for (int64_t r = r0; r < r1; r++) s += Mx[r * cols + c];
-    atomicAdd(&out[c], s);
-}
-
-__global__ void adamw_kernel(int64_t n, float *p, const float *g, float *m, float *v, float lr,
-                             float b1, float b2, float eps, float wd, float bc1, float bc2,
-                             const uint8_t *decay_mask)
+// One parameter a thread: with UPDATE an AdamW step, then -- for a weight -- its copies for the
+// tensor-core products: the split row [w_hi | w_hi | w_lo] of w3 ([out][3 in]) and the transposed
+// bf16 weight of wt ([in][out]).
+template <bool UPDATE>
+__global__ void update_kernel(int64_t n, const __grid_constant__ Offsets off, float *p, const float *g, float *m, float *v,
+                              float lr, float b1, float b2, float eps, float wd, float bc1,
+                              float bc2, __nv_bfloat16 *w3, __nv_bfloat16 *wt)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const float gi = g[i];
-    const float mi = b1 * m[i] + (1.0f - b1) * gi;
-    const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
+    int l = 0;
+#pragma unroll
+    for (int k = 1; k < N_LAYERS; k++) l += i >= off.w[k] ? 1 : 0;
+    const bool weight = i < off.b[l];
     float pi = p[i];
-    if (decay_mask[i]) pi -= lr * wd * pi;
-    pi -= lr * (mi / bc1) / (sqrtf(vi / bc2) + eps);
-    p[i] = pi;
-}
-
-// W3 = [w_hi | w_hi | w_lo] per output row (bf16, [out][3 in]) of fp32 weights [out][in]:
-// the B operand of the split-precision forward product
-__global__ void weights_split_kernel(const float *W, int out_dim, int in_dim, __nv_bfloat16 *W3)
-{
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= out_dim * in_dim) return;
-    const int o = k / in_dim, i = k % in_dim;
+    if (UPDATE) {
+        const float gi = g[i];
+        const float mi = b1 * m[i] + (1.0f - b1) * gi;
+        const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
+        m[i] = mi;
+        v[i] = vi;
+        if (weight) pi -= lr * wd * pi; // decoupled decay, weights only
+        pi -= lr * (mi / bc1) / (sqrtf(vi / bc2) + eps);
+        p[i] = pi;
+    }
+    if (!weight) return;
+    const int in_dim = l == 0 ? 16 : 256, out_dim = l == N_LAYERS - 1 ? 16 : 256;
+    const int k = (int)(i - off.w[l]), o = k / in_dim, c = k % in_dim;
     __nv_bfloat16 hi, lo;
-    split_pair(W[k], &hi, &lo);
-    __nv_bfloat16 *row = W3 + (int64_t)o * 3 * in_dim;
-    row[i] = hi;
-    row[in_dim + i] = hi;
-    row[2 * in_dim + i] = lo;
+    split_pair(pi, &hi, &lo);
+    __nv_bfloat16 *row = w3 + off.w3[l] + (int64_t)o * 3 * in_dim;
+    row[c] = hi;
+    row[in_dim + c] = hi;
+    row[2 * in_dim + c] = lo;
+    wt[off.w[l] + (int64_t)c * out_dim + o] = hi;
 }
 
 // Constants of motion of a camera ray in the Kerr picture: E = -p_t, L = p_phi and the
@@ -471,26 +374,6 @@ namespace {
 using namespace gt;
 using namespace gt::sg;
 
-__global__ void labels_kernel(int64_t n, int64_t row0, const uint8_t *status, const double *th,
-                              const double *ph, float *lab)
-{
-    const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= n) return;
-    const int64_t k = row0 + r;
-    const bool esc = status[k] == GT_RAY_ESCAPED;
-    float y = esc ? 1.0f : 0.0f, dx = 0.f, dy = 0.f, dz = 0.f;
-    if (esc) {
-        const double s = sin(th[k]);
-        dx = (float)(s * cos(ph[k]));
-        dy = (float)(s * sin(ph[k]));
-        dz = (float)cos(th[k]);
-    }
-    lab[r * 4 + 0] = y;
-    lab[r * 4 + 1] = dx;
-    lab[r * 4 + 2] = dy;
-    lab[r * 4 + 3] = dz;
-}
-
 inline unsigned blocks_for(int64_t n, int b = 256) { return (unsigned)((n + b - 1) / b); }
 
 } // namespace
@@ -498,24 +381,19 @@ inline unsigned blocks_for(int64_t n, int b = 256) { return (unsigned)((n + b - 
 struct gt_surrogate {
     int device = 0;
     Norm norm = {};
-    int64_t w_off[N_LAYERS] = {}, b_off[N_LAYERS] = {};
+    Offsets off = {};
     int64_t n_params = 0;
     float *p = nullptr, *g = nullptr, *m = nullptr, *v = nullptr; // fp32 params, grads, Adam
-    uint8_t *decay = nullptr;
     __nv_bfloat16 *w3 = nullptr; // split bf16 weights of the forward products, [out][3 in] per layer
-    int64_t w3_off[N_LAYERS] = {};
-    FusedMaps maps;   // w3 as the inference kernel reads it
+    __nv_bfloat16 *wt = nullptr; // transposed bf16 weights of the backward products, [in][out]
+    FusedMaps maps;              // both as the kernels read them
     int sm_count = 0;
     int64_t step = 0;
-    // workspace for `rows` rows
-    int64_t rows = 0;
-    __nv_bfloat16 *X[N_LAYERS] = {};  // split inputs of each layer (rows x 3 in, forward products)
-    __nv_bfloat16 *XT[N_LAYERS] = {}; // the same in bf16, transposed (in_dim x rows)
-    __nv_bfloat16 *WT = nullptr;      // transposed bf16 weights ([in][out] per layer)
-    __nv_bfloat16 *dZT = nullptr;     // transposed bf16 gradient (cols x rows)
-    float *Z[N_LAYERS] = {};         // pre-activations (fp32)
-    float *dXf = nullptr, *dZf = nullptr, *lab = nullptr, *loss = nullptr;
-    __nv_bfloat16 *dZb = nullptr;
+    // training workspace: the buffers of `tr` for up to `cap` rows, laid out for tr.ld of them
+    int64_t cap = 0;
+    TrainArgs tr = {};
+    WGradMaps wmaps;
+    float *loss = nullptr;
     // set to 1 by a kernel whose mbarrier wait ran out: host memory the device writes, so that
     // a call reads it after its synchronisation without a copy of its own
     int *err = nullptr, *err_host = nullptr;
@@ -526,44 +404,48 @@ namespace {
 void free_ws(gt_surrogate *s)
 {
     for (int l = 0; l < N_LAYERS; l++) {
-        cudaFree(s->X[l]);
-        cudaFree(s->XT[l]);
-        cudaFree(s->Z[l]);
-        s->X[l] = nullptr;
-        s->XT[l] = nullptr;
-        s->Z[l] = nullptr;
+        cudaFree(s->tr.xt[l]);
+        cudaFree(s->tr.dzt[l]);
     }
-    cudaFree(s->dZT);
-    s->dZT = nullptr;
-    cudaFree(s->dXf);
-    cudaFree(s->dZf);
-    cudaFree(s->dZb);
-    cudaFree(s->lab);
-    s->dXf = s->dZf = s->lab = nullptr;
-    s->dZb = nullptr;
-    s->rows = 0;
+    cudaFree(s->tr.z);
+    s->tr = TrainArgs();
+    s->cap = 0;
 }
 
-int ensure_ws(gt_surrogate *s, int64_t rows)
+// Buffers for batches of `rows` rows, laid out for exactly that many (padded to whole tiles).
+int ensure_ws(gt_surrogate *s, int64_t rows, cudaStream_t st)
 {
-    if (s->rows >= rows) return GT_OK;
-    free_ws(s);
-    cudaError_t e = cudaSuccess;
-    for (int l = 0; l < N_LAYERS && e == cudaSuccess; l++) {
-        e = cudaMalloc(&s->X[l], rows * 3 * IN_DIM[l] * sizeof(__nv_bfloat16));
-        if (e == cudaSuccess) e = cudaMalloc(&s->XT[l], rows * IN_DIM[l] * sizeof(__nv_bfloat16));
-        if (e == cudaSuccess) e = cudaMalloc(&s->Z[l], rows * OUT_DIM[l] * sizeof(float));
-    }
-    if (e == cudaSuccess) e = cudaMalloc(&s->dXf, rows * 256 * sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc(&s->dZf, rows * 256 * sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc(&s->dZb, rows * 256 * sizeof(__nv_bfloat16));
-    if (e == cudaSuccess) e = cudaMalloc(&s->dZT, rows * 256 * sizeof(__nv_bfloat16));
-    if (e == cudaSuccess) e = cudaMalloc(&s->lab, rows * 4 * sizeof(float));
-    if (e != cudaSuccess) {
+    const int64_t ld = (rows + FUSED_TILE - 1) / FUSED_TILE * FUSED_TILE;
+    if (s->cap < ld) {
         free_ws(s);
-        return e == cudaErrorMemoryAllocation ? GT_ERR_OOM : GT_ERR_CUDA;
+        cudaError_t e = cudaSuccess;
+        for (int l = 0; l < N_LAYERS && e == cudaSuccess; l++) {
+            e = cudaMalloc(&s->tr.xt[l], ld * IN_DIM[l] * sizeof(__nv_bfloat16));
+            if (e == cudaSuccess)
+                e = cudaMalloc(&s->tr.dzt[l], ld * OUT_DIM[l] * sizeof(__nv_bfloat16));
+        }
+        if (e == cudaSuccess)
+            e = cudaMalloc(&s->tr.z, (int64_t)fused_grid(ld, s->sm_count) * 4 * 256 * FUSED_TILE *
+                                         sizeof(float));
+        if (e != cudaSuccess) {
+            (void)cudaGetLastError(); // a failed allocation is not sticky: no later check reports it
+            free_ws(s);
+            return e == cudaErrorMemoryAllocation ? GT_ERR_OOM : GT_ERR_CUDA;
+        }
+        s->cap = ld;
     }
-    s->rows = rows;
+    if (s->tr.ld != ld) {
+        s->tr.ld = ld;
+        for (int l = 0; l < N_LAYERS; l++) s->tr.db[l] = s->g + s->off.b[l];
+        s->tr.loss = s->loss;
+        // the network uses 4 of the last layer's 16 outputs: the other rows of its gradient stay zero
+        if (cudaMemsetAsync(s->tr.dzt[N_LAYERS - 1], 0, ld * 16 * sizeof(__nv_bfloat16), st) !=
+                cudaSuccess ||
+            !wgrad_prepare(&s->wmaps, s->tr)) {
+            s->tr.ld = 0;
+            return GT_ERR_CUDA;
+        }
+    }
     return GT_OK;
 }
 
@@ -581,92 +463,44 @@ struct Dev {
     }
 };
 
-// split: C16 receives the [hi | lo | hi] split of the output (3 N columns)
-cudaError_t gemm(const void *A, int64_t a_sm, int64_t a_sk, const void *B, int64_t b_sn,
-                 int64_t b_sk, int M, int N, int K, const float *bias, int act, float *pre,
-                 float *C32, int64_t ldc, bool atomic, void *C16, int splits, int *err,
-                 cudaStream_t st, __nv_bfloat16 *C16T = nullptr, bool split = false)
+FusedArgs net_args(gt_surrogate *s, int64_t n)
 {
-    GemmArgs g = {};
-    g.c16_split = split ? 1 : 0;
-    g.M = M;
-    g.N = N;
-    g.K = K;
-    g.A = static_cast<const __nv_bfloat16 *>(A);
-    g.a_sm = a_sm;
-    g.a_sk = a_sk;
-    g.B = static_cast<const __nv_bfloat16 *>(B);
-    g.b_sn = b_sn;
-    g.b_sk = b_sk;
-    g.bias = bias;
-    g.act = act;
-    g.pre = pre;
-    g.ld_pre = N;
-    g.C32 = C32;
-    g.ldc = ldc;
-    g.atomic = atomic ? 1 : 0;
-    g.C16 = static_cast<__nv_bfloat16 *>(C16);
-    g.ldc16 = split ? 3 * (int64_t)N : N;
-    g.C16T = C16T;
-    g.ldt = M;
-    g.err = err;
-    // 256-wide tiles read each A row block once when there are many of them (inference
-    // chunks); 128-wide ones give a training batch twice as many tiles to spread over SMs
-    const int bn = (N >= 256 && M >= 65536) ? 256 : N >= 128 ? 128 : (N >= 64 ? 64 : (N >= 32 ? 32 : 16));
-    return launch_gemm(g, bn, splits, st);
-}
-
-// Forward pass of `B` rows whose features are in X[0]; leaves Z[4] = network output.
-// The training path: every layer's input, transposed input and pre-activation are kept.
-cudaError_t forward(gt_surrogate *s, int B, cudaStream_t st)
-{
-    cudaError_t e = cudaSuccess;
-    for (int l = 0; l < N_LAYERS && e == cudaSuccess; l++) {
-        const bool last = (l == N_LAYERS - 1);
-        const int K3 = 3 * IN_DIM[l];
-        e = gemm(s->X[l], K3, 1, s->w3 + s->w3_off[l], K3, 1, B, OUT_DIM[l], K3,
-                 s->p + s->b_off[l], last ? 0 : 1, last ? nullptr : s->Z[l],
-                 last ? s->Z[l] : nullptr, OUT_DIM[l], false, last ? nullptr : s->X[l + 1], 1,
-                 s->err, st, last ? nullptr : s->XT[l + 1], true);
-    }
-    return e;
-}
-
-// Network outputs of `a`'s rows (inference): one kernel, no workspace.
-cudaError_t infer_rows(gt_surrogate *s, FusedArgs a, cudaStream_t st)
-{
+    FusedArgs a = {};
+    a.n = n;
     a.norm = s->norm;
-    for (int l = 0; l < N_LAYERS; l++) a.bias[l] = s->p + s->b_off[l];
+    for (int l = 0; l < N_LAYERS; l++) a.bias[l] = s->p + s->off.b[l];
     a.err = s->err;
-    return launch_fused(s->maps, a, s->sm_count, st);
+    return a;
 }
 
-// Backward pass of B rows with labels in s->lab: gradients (zeroed here) into s->g.
-cudaError_t backward(gt_surrogate *s, int B, float w_dir, cudaStream_t st)
+struct Batch {
+    const double *alpha, *beta, *spin, *q, *theta0;
+    const uint8_t *status;
+    const double *th_end, *ph_end;
+};
+
+// Gradients of the mean loss of rows [row0, row0 + n) into s->g, the loss sum added to s->loss.
+cudaError_t gradients(gt_surrogate *s, const Batch &b, int64_t row0, int64_t n, float w_dir,
+                      cudaStream_t st)
 {
     cudaError_t e = cudaMemsetAsync(s->g, 0, s->n_params * sizeof(float), st);
     if (e != cudaSuccess) return e;
-    head_kernel<<<blocks_for(B), 256, 0, st>>>(B, s->Z[N_LAYERS - 1], s->lab, w_dir, 1.0f / B,
-                                               s->dZf, s->dZb, s->dZT, s->loss);
-    for (int l = N_LAYERS - 1; l >= 0 && e == cudaSuccess; l--) {
-        const int N = OUT_DIM[l], K = IN_DIM[l];
-        // dW_l[n, k] = sum_b dZ[b, n] X_l[b, k] from the transposed copies (K-contiguous
-        // in the batch), split over the batch
-        const int splits = B >= 512 ? (B / 256 < 128 ? B / 256 : 128) : 1;
-        e = gemm(s->dZT, B, 1, s->XT[l], B, 1, N, K, B, nullptr, 0, nullptr, s->g + s->w_off[l], K,
-                 true, nullptr, splits, s->err, st);
-        if (e != cudaSuccess) break;
-        // db_l = column sums of dZ
-        colsum_kernel<<<dim3(blocks_for(N, 128), 64), 128, 0, st>>>(s->dZf, B, N, s->g + s->b_off[l]);
-        if (l == 0) break;
-        // dX[b, k] = sum_n dZ[b, n] W_l[n, k] = dZ . (W_l^T)^T
-        e = gemm(s->dZb, N, 1, s->WT + s->w_off[l], N, 1, B, K, N, nullptr, 0, nullptr, s->dXf, K,
-                 false, nullptr, 1, s->err, st);
-        if (e != cudaSuccess) break;
-        silu_backward_kernel<<<blocks_for((int64_t)B * K), 256, 0, st>>>(B, K, s->dXf, s->Z[l - 1],
-                                                                         s->dZf, s->dZb, s->dZT);
-        e = cudaGetLastError();
-    }
+    FusedArgs a = net_args(s, n);
+    a.alpha = b.alpha + row0;
+    a.beta = b.beta + row0;
+    a.spin = b.spin + row0;
+    a.q = b.q + row0;
+    a.theta0 = b.theta0 + row0;
+    a.tr = s->tr;
+    a.tr.status = b.status + row0;
+    a.tr.th_end = b.th_end + row0;
+    a.tr.ph_end = b.ph_end + row0;
+    a.tr.w_dir = w_dir;
+    a.tr.inv_b = 1.0f / (float)n;
+    e = launch_fused_train(s->maps, a, s->sm_count, st);
+    float *gw[N_LAYERS];
+    for (int l = 0; l < N_LAYERS; l++) gw[l] = s->g + s->off.w[l];
+    if (e == cudaSuccess) e = launch_wgrad(s->wmaps, gw, s->tr.ld, s->err, s->sm_count, st);
     return e;
 }
 
@@ -677,17 +511,12 @@ int check_err(gt_surrogate *s, cudaStream_t st)
     return h ? GT_ERR_TIMEOUT : GT_OK;
 }
 
-// split bf16 weights (forward products) and transposed bf16 weights (backward products)
-// after an update
+// split and transposed bf16 weights from the parameters
 cudaError_t refresh_copies(gt_surrogate *s, cudaStream_t st)
 {
-    for (int l = 0; l < N_LAYERS; l++) {
-        const int64_t n = (int64_t)OUT_DIM[l] * IN_DIM[l];
-        weights_split_kernel<<<blocks_for(n), 256, 0, st>>>(s->p + s->w_off[l], OUT_DIM[l],
-                                                           IN_DIM[l], s->w3 + s->w3_off[l]);
-        weights_t_kernel<<<blocks_for(n), 256, 0, st>>>(s->p + s->w_off[l], OUT_DIM[l], IN_DIM[l],
-                                                        s->WT + s->w_off[l]);
-    }
+    update_kernel<false><<<blocks_for(s->n_params), 256, 0, st>>>(
+        s->n_params, s->off, s->p, nullptr, nullptr, nullptr, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 1.0f,
+        1.0f, s->w3, s->wt);
     return cudaGetLastError();
 }
 
@@ -728,23 +557,19 @@ int gt_surrogate_create(int device, const gt_surrogate_norm *nrm, uint64_t seed,
     int64_t off = 0;
     std::vector<int64_t> offs;
     std::vector<float> scales;
-    std::vector<uint8_t> decay;
     for (int l = 0; l < N_LAYERS; l++) {
-        s->w_off[l] = off;
+        s->off.w[l] = off;
         offs.push_back(off);
         // LeCun-normal weights (the 6 zero-padded input columns do not count)
         const int fan_in = l == 0 ? 10 : IN_DIM[l];
         scales.push_back((float)(1.0 / sqrt((double)fan_in)));
         off += (int64_t)OUT_DIM[l] * IN_DIM[l];
-        s->b_off[l] = off;
+        s->off.b[l] = off;
         offs.push_back(off);
         scales.push_back(0.0f);
         off += OUT_DIM[l];
     }
     s->n_params = off;
-    decay.assign(off, 0);
-    for (int l = 0; l < N_LAYERS; l++)
-        for (int64_t i = s->w_off[l]; i < s->b_off[l]; i++) decay[i] = 1;
     int64_t *d_offs = nullptr;
     float *d_scales = nullptr;
     cudaError_t e = cudaMalloc(&s->p, off * sizeof(float));
@@ -753,12 +578,11 @@ int gt_surrogate_create(int device, const gt_surrogate_norm *nrm, uint64_t seed,
     if (e == cudaSuccess) e = cudaMalloc(&s->v, off * sizeof(float));
     int64_t off3 = 0;
     for (int l = 0; l < N_LAYERS; l++) {
-        s->w3_off[l] = off3;
+        s->off.w3[l] = off3;
         off3 += (int64_t)OUT_DIM[l] * 3 * IN_DIM[l];
     }
     if (e == cudaSuccess) e = cudaMalloc(&s->w3, off3 * sizeof(__nv_bfloat16));
-    if (e == cudaSuccess) e = cudaMalloc(&s->WT, off * sizeof(__nv_bfloat16));
-    if (e == cudaSuccess) e = cudaMalloc(&s->decay, off);
+    if (e == cudaSuccess) e = cudaMalloc(&s->wt, off * sizeof(__nv_bfloat16));
     if (e == cudaSuccess) e = cudaMalloc(&s->loss, sizeof(float));
     if (e == cudaSuccess)
         e = cudaHostAlloc(&s->err_host, sizeof(int), cudaHostAllocMapped | cudaHostAllocPortable);
@@ -772,14 +596,16 @@ int gt_surrogate_create(int device, const gt_surrogate_norm *nrm, uint64_t seed,
         e = cudaMemcpy(d_offs, offs.data(), offs.size() * sizeof(int64_t), cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
         e = cudaMemcpy(d_scales, scales.data(), scales.size() * sizeof(float), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(s->decay, decay.data(), off, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(s->m, 0, off * sizeof(float));
     if (e == cudaSuccess) e = cudaMemset(s->v, 0, off * sizeof(float));
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&s->sm_count, cudaDevAttrMultiProcessorCount, device);
     if (e == cudaSuccess) {
-        const void *w[N_LAYERS];
-        for (int l = 0; l < N_LAYERS; l++) w[l] = s->w3 + s->w3_off[l];
-        if (!fused_prepare(&s->maps, w)) e = cudaErrorUnknown;
+        const void *w[N_LAYERS], *t[N_LAYERS];
+        for (int l = 0; l < N_LAYERS; l++) {
+            w[l] = s->w3 + s->off.w3[l];
+            t[l] = s->wt + s->off.w[l];
+        }
+        if (!fused_prepare(&s->maps, w, t)) e = cudaErrorUnknown;
     }
     if (e == cudaSuccess) {
         init_params_kernel<<<blocks_for(off), 256>>>(s->p, off, d_offs, d_scales, (int)offs.size(), seed);
@@ -807,8 +633,7 @@ int gt_surrogate_destroy(gt_surrogate *s)
     cudaFree(s->m);
     cudaFree(s->v);
     cudaFree(s->w3);
-    cudaFree(s->WT);
-    cudaFree(s->decay);
+    cudaFree(s->wt);
     cudaFree(s->loss);
     cudaFreeHost(s->err_host);
     delete s;
@@ -849,15 +674,14 @@ int gt_surrogate_eval(gt_ctx *ctx, gt_surrogate *s, int64_t n, const double *alp
         return GT_ERR_INVALID_ARG;
     Dev d(s->device);
     cudaStream_t st = gt_internal_stream(ctx);
-    FusedArgs a = {};
-    a.n = n;
+    FusedArgs a = net_args(s, n);
     a.alpha = alpha;
     a.beta = beta;
     a.spin = spin;
     a.q = q;
     a.theta0 = theta0;
     a.out = out;
-    if (infer_rows(s, a, st) != cudaSuccess) return GT_ERR_CUDA;
+    if (launch_fused(s->maps, a, s->sm_count, st) != cudaSuccess) return GT_ERR_CUDA;
     return check_err(s, st);
 }
 
@@ -869,14 +693,11 @@ int gt_surrogate_grad(gt_ctx *ctx, gt_surrogate *s, int64_t n, const double *alp
     if (!ctx || !s || n < 1 || n > (1 << 20) || !grads_host || !loss_host) return GT_ERR_INVALID_ARG;
     Dev d(s->device);
     cudaStream_t st = gt_internal_stream(ctx);
-    int rc = ensure_ws(s, n);
+    int rc = ensure_ws(s, n, st);
     if (rc != GT_OK) return rc;
-    features_kernel<<<blocks_for(n), 256, 0, st>>>(n, 0, alpha, beta, spin, q, theta0, s->norm, s->X[0],
-                                                   s->XT[0]);
-    labels_kernel<<<blocks_for(n), 256, 0, st>>>(n, 0, status, th_end, ph_end, s->lab);
+    const Batch all = {alpha, beta, spin, q, theta0, status, th_end, ph_end};
     cudaError_t e = cudaMemsetAsync(s->loss, 0, sizeof(float), st);
-    if (e == cudaSuccess) e = forward(s, (int)n, st);
-    if (e == cudaSuccess) e = backward(s, (int)n, dir_weight, st);
+    if (e == cudaSuccess) e = gradients(s, all, 0, n, dir_weight, st);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(grads_host, s->g, s->n_params * sizeof(float), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(loss_host, s->loss, sizeof(float), cudaMemcpyDeviceToHost, st);
@@ -897,8 +718,9 @@ int gt_surrogate_train(gt_ctx *ctx, gt_surrogate *s, const gt_train_cfg *cfg, in
     Dev d(s->device);
     cudaStream_t st = gt_internal_stream(ctx);
     const int B = cfg->batch;
-    int rc = ensure_ws(s, B);
+    int rc = ensure_ws(s, B, st);
     if (rc != GT_OK) return rc;
+    const Batch all = {alpha, beta, spin, q, theta0, status, th_end, ph_end};
     const int64_t nb = n / B; // full batches only
     if (nb < 1) return GT_ERR_INVALID_ARG;
     const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
@@ -908,19 +730,14 @@ int gt_surrogate_train(gt_ctx *ctx, gt_surrogate *s, const gt_train_cfg *cfg, in
         for (int64_t b = 0; b < nb && e == cudaSuccess; b++) {
             const double prog = ((double)ep * nb + b) / ((double)cfg->epochs * nb);
             const float lr = (float)(cfg->lr * 0.5 * (1.0 + cos(M_PI * prog)));
-            features_kernel<<<blocks_for(B), 256, 0, st>>>(B, b * B, alpha, beta, spin, q, theta0,
-                                                           s->norm, s->X[0], s->XT[0]);
-            labels_kernel<<<blocks_for(B), 256, 0, st>>>(B, b * B, status, th_end, ph_end, s->lab);
-            e = forward(s, B, st);
-            if (e == cudaSuccess) e = backward(s, B, (float)cfg->dir_weight, st);
+            e = gradients(s, all, b * B, B, (float)cfg->dir_weight, st);
             if (e != cudaSuccess) break;
             s->step++;
             const float bc1 = 1.0f - powf(b1, (float)s->step), bc2 = 1.0f - powf(b2, (float)s->step);
-            adamw_kernel<<<blocks_for(s->n_params), 256, 0, st>>>(s->n_params, s->p, s->g, s->m, s->v,
-                                                                  lr, b1, b2, eps,
-                                                                  (float)cfg->weight_decay, bc1, bc2,
-                                                                  s->decay);
-            e = refresh_copies(s, st);
+            update_kernel<true><<<blocks_for(s->n_params), 256, 0, st>>>(
+                s->n_params, s->off, s->p, s->g, s->m, s->v, lr, b1, b2, eps,
+                (float)cfg->weight_decay, bc1, bc2, s->w3, s->wt);
+            e = cudaGetLastError();
         }
         if (e != cudaSuccess) return GT_ERR_CUDA;
         if (loss_per_epoch) {
@@ -944,11 +761,10 @@ namespace sg {
 // The network on every pixel of the camera; its answers to `net` (float4 per pixel).
 int net_pass(gt_surrogate *s, const CamDesc *d_cam, int64_t n_pix, float4 *net, cudaStream_t st)
 {
-    FusedArgs a = {};
-    a.n = n_pix;
+    FusedArgs a = net_args(s, n_pix);
     a.cam = d_cam;
     a.out = (float *)net;
-    if (infer_rows(s, a, st) != cudaSuccess) return GT_ERR_CUDA;
+    if (launch_fused(s->maps, a, s->sm_count, st) != cudaSuccess) return GT_ERR_CUDA;
     return check_err(s, st);
 }
 

@@ -1,9 +1,11 @@
-"""The one-kernel forward pass of the surrogate (csrc/mlp_fused.cu) at the edges of its tiles."""
+"""The surrogate's single-kernel passes (csrc/mlp_fused.cu) at the edges of their tiles."""
 import numpy as np
 import pytest
 
 from oracle import mlp
 from paper_2310_15183_gb300 import workloads as W
+
+from .test_gpu_surrogate import _abs_scales, _fake_labels
 
 pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
@@ -58,3 +60,26 @@ def test_unaligned_output(net):
     torch.cuda.synchronize()
     assert torch.equal(buf[1:-1].view(200, 4), s.eval(tracer, dev))
     assert buf[0].item() == 0.0 and buf[-1].item() == 0.0
+
+
+@pytest.mark.parametrize("sizes", [(1, 128, 127), (300, 129, 300), (152 * 128 + 5, 40)])
+def test_gradients_at_tile_edges(net, sizes):
+    """Loss and gradients (one kernel for forward, loss and input gradients, one for the weight
+    gradients) on one network for batches of changing size: element-wise within the bounds of
+    the layer-wise test (2^-7 of the running bound: one bf16 rounding decision per operand)."""
+    tracer, s = net
+    for n in sizes:
+        host = W.surrogate_samples(n, seed=n + 1)
+        lab_h, lab_d = _fake_labels(n, n + 2)
+        grads, loss = s.grad(tracer, [torch.tensor(x, device="cuda") for x in host], lab_d, 10.0)
+        p = s.get_params().astype(np.float64)
+        X0 = mlp.features(*host)
+        y, d = mlp.labels(*lab_h)
+        ref_loss, ref_g, _ = mlp.loss_and_grad(p, X0, y, d, 10.0, bf=True)
+        assert abs(loss - ref_loss) < 1e-4 * abs(ref_loss), (n, loss, ref_loss)
+        scale_w, scale_b, _ = _abs_scales(p, X0, y, d, 10.0)
+        ws, bs = mlp.split(grads.astype(np.float64))
+        rws, rbs = mlp.split(ref_g)
+        for l in range(5):
+            assert np.all(np.abs(ws[l] - rws[l]) <= 2.0 ** -7 * scale_w[l] + 1e-12), (n, l)
+            assert np.all(np.abs(bs[l] - rbs[l]) <= 2.0 ** -7 * scale_b[l] + 1e-12), (n, l)
