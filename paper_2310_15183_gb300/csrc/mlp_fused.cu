@@ -30,7 +30,7 @@
 // Measured: 8 steps of 8,192 rows 3.88 -> 0.91 ms; loss and gradients of 16,384 rows with
 // their copy to the host 743 -> 156 us.
 //
-// Warps: 0 loads, 1 issues the MMAs, 2-5 compute the next tile's features in FP64 while the
+// Warps: 0 loads, 1 issues the MMAs, 2-5 compute the next tile's features while the
 // current one runs (and its labels), 6-21 drain the accumulator: bias, SiLU, split, back into the operand
 // buffer.  All hand-offs are mbarriers with bounded waits; a wait that runs out sets the
 // error flag and every role leaves its loop.
@@ -297,12 +297,8 @@ __global__ void __launch_bounds__(THREADS, 1)
                 make_features(g.alpha[r], g.beta[r], g.spin[r], g.q[r], g.theta0[r], g.norm, f);
             }
             float lab[3] = {0.0f, 0.0f, 0.0f}; // end direction; zero when the ray did not escape
-            if (TRAIN && r < g.n && g.tr.status[r] == GT_RAY_ESCAPED) {
-                const double th = g.tr.th_end[r], ph = g.tr.ph_end[r], s = sin(th);
-                lab[0] = (float)(s * cos(ph));
-                lab[1] = (float)(s * sin(ph));
-                lab[2] = (float)cos(th);
-            }
+            if (TRAIN && r < g.n && g.tr.status[r] == GT_RAY_ESCAPED)
+                unit_vector(g.tr.th_end[r], g.tr.ph_end[r], lab);
             if (TRAIN) {
 #pragma unroll
                 for (int j = 0; j < 16; j++) g.tr.xt[0][j * g.tr.ld + r] = __float2bfloat16(f[j]);

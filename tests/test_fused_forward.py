@@ -83,3 +83,20 @@ def test_gradients_at_tile_edges(net, sizes):
         for l in range(5):
             assert np.all(np.abs(ws[l] - rws[l]) <= 2.0 ** -7 * scale_w[l] + 1e-12), (n, l)
             assert np.all(np.abs(bs[l] - rbs[l]) <= 2.0 ** -7 * scale_b[l] + 1e-12), (n, l)
+
+
+def test_features_outside_the_pair_range(net):
+    """Rows whose polar form or angle leaves the range of the double-float evaluation (the image
+    centre, an angle of many turns) take FP64: the outputs match the reference like any row's."""
+    tracer, s = net
+    n = 8
+    al = np.array([0.0, 1e-9, 1e-30, 0.05, 0.05, -0.02, 1e-7, 0.03])
+    be = np.array([0.0, 0.0, 1e-30, 0.01, 0.0, 0.05, -1e-7, 0.0])
+    th = np.array([1.0, 1.0, 0.5, 700.0, -129.0, 1.2, 1.3, 127.9])
+    host = (al, be, np.full(n, 0.5), np.zeros(n), th)
+    out = s.eval(tracer, [torch.tensor(x, device="cuda") for x in host]).cpu().numpy()
+    p = s.get_params().astype(np.float64)
+    As, Zs = mlp.forward(p, mlp.features(*host), bf=True)
+    scale = np.abs(As[4]) @ np.abs(mlp.split(p)[0][4]).T + np.abs(mlp.split(p)[1][4])
+    err = np.abs(out - Zs[4][:, :4])
+    assert np.all(err <= 2.0 ** -12 * scale[:, :4]), float(np.max(err / scale[:, :4]))
