@@ -33,7 +33,7 @@ struct gt_ctx {
     int cam_valid = 0;
     int cam_flags = -1;
     double cam_rsw = -2.0;
-    gt::PairSpacetime cam_pair = {}; // the camera's double-float constants as set up on the device
+    CamDesc cam = {}; // the descriptor as set up on the device
     // batch descriptors (device)
     CamDesc *d_batch = nullptr;
     int batch_cap = 0;
@@ -169,7 +169,7 @@ int prepare_camera(gt_ctx *c)
     if (err == cudaSuccess) err = cudaStreamSynchronize(c->stream);
     if (err != cudaSuccess) return cuda_code(err);
     c->cam_valid = d.valid;
-    c->cam_pair = d.pair;
+    c->cam = d;
     c->cam_dirty = false;
     c->cam_flags = e.flags;
     c->cam_rsw = e.r_switch;
@@ -381,7 +381,7 @@ int run_trace(gt_ctx *c, const CamDesc *d_cams, int n_cams, int kind_hint, int64
               double *th, double *ph, uint8_t *status, uint32_t *nsteps,
               const int64_t *fresh_ids = nullptr, const gt::RayParams *d_rays = nullptr,
               bool compact_out = false, const Extra &x = Extra(), bool range_ok = true,
-              const gt::PairSpacetime *pair = nullptr)
+              const CamDesc *one = nullptr)
 {
     const gt_options e = effective(c->opts);
     if ((e.flags & PAPER_FLAGS) && mode != GT_MODE_FP64) return GT_ERR_INVALID_ARG;
@@ -416,9 +416,10 @@ int run_trace(gt_ctx *c, const CamDesc *d_cams, int n_cams, int kind_hint, int64
     a.disk = x.disk;
     a.z = x.z;
     a.states = x.states;
-    if (pair) {
-        a.pair = *pair;
-        a.pair_single = 1;
+    if (one) {
+        a.pair = one->pair;
+        a.stf = gt::to_float(one->st);
+        a.single = 1;
     }
     cudaError_t err =
         cudaMemsetAsync(c->d_scratch, 0, gt::SCR_WORDS * sizeof(unsigned long long), c->stream);
@@ -662,7 +663,7 @@ int gt_trace_range(gt_ctx *c, int64_t first, int64_t count, int64_t n_steps, dou
     const int kind = (c->Q != 0.0) ? gt::KIND_MN : gt::KIND_KERR;
     return run_trace(c, c->d_cam, 1, kind, first, count, n_steps, sp, mode, t, r, th, ph, status,
                      nsteps, nullptr, nullptr, false, Extra(), gt::pair_range(c->M, c->r0),
-                     &c->cam_pair);
+                     &c->cam);
 }
 
 int gt_trace_pixels(gt_ctx *c, const int64_t *pixels, int64_t n, int64_t n_steps, double sp,
@@ -683,7 +684,7 @@ int gt_trace_pixels(gt_ctx *c, const int64_t *pixels, int64_t n, int64_t n_steps
     const int kind = (c->Q != 0.0) ? gt::KIND_MN : gt::KIND_KERR;
     return run_trace(c, c->d_cam, 1, kind, 0, n, n_steps, sp, mode, t, r, th, ph, status, nsteps,
                      pixels, nullptr, true, Extra(), gt::pair_range(c->M, c->r0),
-                     &c->cam_pair);
+                     &c->cam);
 }
 
 int gt_trace_disk(gt_ctx *c, double r_in, double r_out, double half_thickness, int64_t n_steps,
@@ -711,7 +712,7 @@ int gt_trace_disk(gt_ctx *c, double r_in, double r_out, double half_thickness, i
     x.z = z;
     const int kind = (c->Q != 0.0) ? gt::KIND_MN : gt::KIND_KERR;
     return run_trace(c, c->d_cam, 1, kind, 0, (int64_t)c->res_x * c->res_y, n_steps, sp, mode, t,
-                     r, th, ph, status, nsteps, nullptr, nullptr, false, x, true, &c->cam_pair);
+                     r, th, ph, status, nsteps, nullptr, nullptr, false, x, true, &c->cam);
 }
 
 int gt_trace_states(gt_ctx *c, int64_t n, double *t, double *r, double *th, double *ph,
@@ -845,7 +846,7 @@ int gt_trace_batch(gt_ctx *c, const gt_camera_desc *cams, int n_cams, int64_t n_
     const int kind = any_mn && any_kerr ? 2 : (any_mn ? gt::KIND_MN : gt::KIND_KERR);
     return run_trace(c, c->d_batch, n_cams, kind, 0, off, n_steps, sp, mode, t, r, th, ph, status,
                      nsteps, nullptr, nullptr, false, Extra(), range_ok,
-                     n_cams == 1 ? &h[0].pair : nullptr);
+                     n_cams == 1 ? &h[0] : nullptr);
 }
 
 int gt_trace_rays(gt_ctx *c, int64_t n, const double *alpha, const double *beta,
@@ -959,7 +960,7 @@ int gt_surrogate_infer(gt_ctx *c, gt_surrogate *s, const gt_gate_cfg *gate, int6
     if (rc == GT_OK && n1 > 0)
         rc = run_trace(c, c->d_cam, 1, kind, 0, n1, n_steps, sp, mode, t, r, th, ph, status,
                        nsteps, list, nullptr, false, Extra(), gt::pair_range(c->M, c->r0),
-                     &c->cam_pair);
+                     &c->cam);
     if (rc != GT_OK) return rc;
     // 3. probe records from the traced probes
     if (pg.stride > 0) {
@@ -977,7 +978,7 @@ int gt_surrogate_infer(gt_ctx *c, gt_surrogate *s, const gt_gate_cfg *gate, int6
     if (rc == GT_OK && n2 > 0)
         rc = run_trace(c, c->d_cam, 1, kind, 0, n2, n_steps, sp, mode, t, r, th, ph, status,
                        nsteps, list, nullptr, false, Extra(), gt::pair_range(c->M, c->r0),
-                     &c->cam_pair);
+                     &c->cam);
     if (rc != GT_OK) return rc;
     if (n_fallback) *n_fallback = n1 - np + n2;
     if (n_probes) *n_probes = np;

@@ -129,10 +129,12 @@ struct TraceArgs {
     StateArrays states; // with states.t != null fresh rays start from these arrays and the
                         // end states (all 8 components) are written back to them
     int zone_df;        // FP32-mixed: the zone's Manko-Novikov field in double-float
-    // constants of the double-float step when the launch has one camera (pair_single): kernel
-    // parameters are read as instruction operands, descriptors in memory through registers
+    // constants of the double-float and of the FP32 step when the launch has one camera
+    // (`single`): kernel parameters are read as instruction operands, descriptors in memory
+    // through registers
     PairSpacetime pair;
-    int pair_single;
+    SpacetimeF stf;
+    int single;
 };
 
 // Host-side validation shared by every entry point that takes a spacetime or a camera

@@ -145,7 +145,8 @@ extern "C" int gt_trace_batch_noalloc(int device, void *cuda_stream, const gt_ca
     a.zone_df = 1; // the context's default zone (double-float Manko-Novikov field)
     if (n_cams == 1) {
         a.pair = h[0].pair;
-        a.pair_single = 1;
+        a.stf = gt::to_float(h[0].st);
+        a.single = 1;
     }
     const int kind = any_mn && any_kerr ? 2 : (any_mn ? gt::KIND_MN : gt::KIND_KERR);
     const int block = 128;

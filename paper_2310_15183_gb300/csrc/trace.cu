@@ -629,6 +629,66 @@ __device__ __forceinline__ float rk4_step32(const SpacetimeF &st, RayMixed &m, f
     return h;
 }
 
+// The same step out of line, for the rays whose stage angles the fast step below does not take.
+template <int KIND, bool PRECISE>
+__device__ __noinline__ float rk4_step32_call(const SpacetimeF &st, RayMixed &m, float sp, float w6)
+{
+    return rk4_step32<KIND, PRECISE>(st, m, sp, w6);
+}
+
+// rk4_step32 without a branch between its stages: the rotation of sin/cos by the series alone,
+// `turn` receiving the largest stage angle -- beyond 1/4 (not met in practice) the result is
+// not rk4_step32's and the caller repeats the step out of line.  The fused multiply-adds of the
+// sums are written out as the compiler forms them across rk4_step32's basic blocks, so that
+// both give the same bits.
+__device__ __forceinline__ void rotate_series(float s, float c, float d, float *s2, float *c2)
+{
+    const float d2 = d * d;
+    const float sd = fmaf(d * d2, fmaf(d2, fmaf(d2, -1.0f / 5040.0f, 1.0f / 120.0f), -1.0f / 6.0f), d);
+    const float cd = fmaf(d2, fmaf(d2, fmaf(d2, -1.0f / 720.0f, 1.0f / 24.0f), -0.5f), 1.0f);
+    *s2 = fmaf(s, cd, c * sd);
+    *c2 = fmaf(c, cd, -(s * sd));
+}
+
+__device__ __forceinline__ float stage_sum(float k1, float k2, float k3, float k4)
+{
+    return __fmaf_rn(2.0f, k3, __fmaf_rn(2.0f, k2, k1)) + k4;
+}
+
+template <int KIND, bool PRECISE = false>
+__device__ __forceinline__ float rk4_step32_fast(const SpacetimeF &st, RayMixed &m, float sp,
+                                                 float w6, float &turn)
+{
+    Rates<float> k1, k2, k3, k4;
+    const float r = m.r.hi, th = m.th.hi, pr = m.pr.hi, pth = m.pth.hi;
+    float s1, c1, s, c;
+    sincosf(th, &s1, &c1);
+    rates_f32<KIND, PRECISE>(st, r, s1, c1, pr, pth, m.ptf, m.pphf, k1);
+    const float h = fabsf(sp / k1.dt);
+    const float hh = 0.5f * h;
+    const float d1 = __fmul_rn(hh, k1.dth);
+    rotate_series(s1, c1, d1, &s, &c);
+    rates_f32<KIND, PRECISE>(st, fmaf(hh, k1.dr, r), s, c, fmaf(hh, k1.dpr, pr),
+                             fmaf(hh, k1.dpth, pth), m.ptf, m.pphf, k2);
+    const float d2 = __fmul_rn(hh, k2.dth);
+    rotate_series(s1, c1, d2, &s, &c);
+    rates_f32<KIND, PRECISE>(st, fmaf(hh, k2.dr, r), s, c, fmaf(hh, k2.dpr, pr),
+                             fmaf(hh, k2.dpth, pth), m.ptf, m.pphf, k3);
+    const float d3 = __fmul_rn(h, k3.dth);
+    rotate_series(s1, c1, d3, &s, &c);
+    rates_f32<KIND, PRECISE>(st, fmaf(h, k3.dr, r), s, c, fmaf(h, k3.dpr, pr),
+                             fmaf(h, k3.dpth, pth), m.ptf, m.pphf, k4);
+    turn = fmaxf(fmaxf(fabsf(d1), fabsf(d2)), fabsf(d3));
+    const float hw = h * w6;
+    f2_add(m.t, hw * stage_sum(k1.dt, k2.dt, k3.dt, k4.dt));
+    f2_add(m.r, hw * stage_sum(k1.dr, k2.dr, k3.dr, k4.dr));
+    f2_add(m.th, hw * stage_sum(k1.dth, k2.dth, k3.dth, k4.dth));
+    f2_add(m.ph, hw * stage_sum(k1.dph, k2.dph, k3.dph, k4.dph));
+    f2_add(m.pr, hw * stage_sum(k1.dpr, k2.dpr, k3.dpr, k4.dpr));
+    f2_add(m.pth, hw * stage_sum(k1.dpth, k2.dpth, k3.dpth, k4.dpth));
+    return h;
+}
+
 // H = 0 re-projection in FP64 (mixed mode): solve g^rr p_r^2 = -(rest) for |p_r|,
 // keeping the sign of p_r.  Skipped near radial turning points, where the radial
 // term is small against the rest and the square root is ill-conditioned.
@@ -683,13 +743,13 @@ __device__ __forceinline__ void park(const TraceArgs &A, int64_t id, uint32_t n,
     *ok = true;
 }
 
-template <int MODE, int KIND, bool PRECISE>
+// SINGLE: one camera, its constants in the kernel's parameters (A.pair, A.stf).
+template <int MODE, int KIND, bool PRECISE, bool SINGLE>
 __device__ __forceinline__ void trace_body(const TraceArgs &A, int one_shot)
 {
     constexpr bool ZONE = MODE == 3 || MODE == 4;  // zone rays, parked when they leave
     constexpr bool PAIR = MODE == 4 || MODE == 5;  // three-float state, double-float step
     constexpr bool TABLES = PAIR || MODE == 1;
-    constexpr bool SINGLE = PAIR && PRECISE;       // one camera, its constants in A.pair
     // per-ray spacetimes come with KIND_ANY only, and never to the double-float MODE 5
     const RayParams *const rays = KIND == KIND_ANY && MODE != 5 ? A.rays : nullptr;
     __shared__ PairTables tab_s[1];
@@ -729,6 +789,7 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A, int one_shot)
     double r_sw = cams[0].r_switch;
     const float spf = A.sp_f, w6f = A.w6_f;
     const float h_thr_f = A.h_thr_f;
+    const uint32_t n_last = (uint32_t)A.n_steps; // n_steps <= 2^32 - 1
     F2 r_esc_f = f2_from(r_esc);
     float r_sw_f = (float)r_sw;
     TF r_esc_t = tf_from(r_esc), r_out_t = tf_from(1.25 * r_sw);
@@ -877,12 +938,13 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A, int one_shot)
                 }
             }
         }
-        if (!__any_sync(FULL_MASK, active)) {
+        const unsigned live = __ballot_sync(FULL_MASK, active);
+        if (!live) {
             if (drained) break;
             continue;
         }
         // ---- watchdog: stop every lane with status TIMEOUT
-        if (A.timeout_ns && (it & 127u) == 0u) {
+        if (A.timeout_ns && (MODE == 2 || (it & 127u) == 0u)) {
             int stop = 0;
             if (lane == 0) {
                 if (*tflag) {
@@ -1056,9 +1118,38 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A, int one_shot)
                 }
             }
         } else { // MODE 2: FP32 steps only, exit tests in FP32
-            RayMixed keep = m;
-            const float h = rk4_step32<KIND, PRECISE>(stf, m, spf, w6f);
-            ++n;
+            // What bounds it: issue slots with four warps a scheduler (the FP32 pipe is busy 70 to
+            // 73 % of the cycles, a slot used in 82 to 84 %), the dependent chain of a step with
+            // fewer -- and a terminating image ends on its longest rays, 450,000 steps of a lone
+            // warp where the mean is 250,000.  Votes, refills and exit tests per step, three
+            // branches around the stage rotations and the spacetime's constants in registers
+            // cost both: a step is 417 instructions (Kerr; 482 before) and 1,261 (Manko-
+            // Novikov; 1,318), a lone Kerr warp takes 764 cycles a step (1,284), a full chip 505 a
+            // warp (641); Manko-Novikov 1,880 (2,550) and 1,470 (1,676).
+            // Steps back to back until some lane of the warp has something to do: an exit, the
+            // zone, a re-projection, a stage angle the fast step does not take.  One test covers
+            // them all (the sum is finite only if every coordinate is; r within [r_switch,
+            // r_escape) and h at or above the horizon's step are false for NaN); the exact tests
+            // below decide.  128 steps at most, for the watchdog.
+            const uint32_t n_event = rp_next < n_last ? rp_next : n_last;
+            const SpacetimeF &sf = SINGLE ? A.stf : stf;
+            RayMixed keep;
+            float h, turn;
+            bool event;
+            for (int q = 0;;) {
+                keep = m;
+                h = rk4_step32_fast<KIND, PRECISE>(sf, m, spf, w6f, turn);
+                ++n;
+                const float sum = ((m.t.hi + m.th.hi) + (m.ph.hi + m.pr.hi)) + m.pth.hi;
+                event = !(m.r.hi < r_esc_f.hi && m.r.hi >= r_sw_f && h >= h_thr_f &&
+                          turn <= 0.25f && fabsf(sum) <= 3.4028234e38f && n != n_event);
+                if (__any_sync(live, event || A.disk.on) || ++q == 128) break;
+            }
+            if (!event && !A.disk.on) continue;
+            if (!(turn <= 0.25f)) {
+                m = keep;
+                h = rk4_step32_call<KIND, PRECISE>(sf, m, spf, w6f);
+            }
             const bool ok = isfinite(h) && isfinite(m.t.hi) && isfinite(m.r.hi) &&
                             isfinite(m.th.hi) && isfinite(m.ph.hi) && isfinite(m.pr.hi) &&
                             isfinite(m.pth.hi);
@@ -1119,10 +1210,11 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A, int one_shot)
 
 // The FP32 rounds kernel (MODE 2) is held to 128 registers: four resident blocks of 128
 // threads per SM, also with PRECISE (GT_FLAG_PRECISE_MN), which needs a few more.
-template <int MODE, int KIND, bool PRECISE = false>
-__global__ void __launch_bounds__(256, MODE == 2 ? 2 : 1) trace_kernel(TraceArgs A, int one_shot)
+template <int MODE, int KIND, bool PRECISE = false, bool SINGLE = false>
+__global__ void __launch_bounds__(256, MODE == 2 ? 2 : 1)
+    trace_kernel(const __grid_constant__ TraceArgs A, int one_shot)
 {
-    trace_body<MODE, KIND, PRECISE>(A, one_shot);
+    trace_body<MODE, KIND, PRECISE, SINGLE>(A, one_shot);
 }
 
 // The double-float kernels: 168 registers, 12 warps an SM.  The Manko-Novikov sweep spills
@@ -1134,7 +1226,7 @@ template <int MODE, int KIND, bool SINGLE>
 __global__ void __maxnreg__(KIND == KIND_ANY ? 255 : 168)
     pair_kernel(const __grid_constant__ TraceArgs A, int one_shot)
 {
-    trace_body<MODE, KIND, SINGLE>(A, one_shot);
+    trace_body<MODE, KIND, false, SINGLE>(A, one_shot);
 }
 
 // ------------------------------------------------------------------ two rays per thread
@@ -1339,22 +1431,31 @@ cudaError_t launch_set_condition(cudaGraphConditionalHandle h, const unsigned lo
     return cudaGetLastError();
 }
 
+template <int MODE, int KIND, bool SINGLE>
+static void launch_kernel(const TraceArgs &a, int block, int grid, int one_shot, cudaStream_t s)
+{
+    if constexpr (MODE >= 4) {
+        pair_kernel<MODE, KIND, SINGLE><<<grid, block, 0, s>>>(a, one_shot);
+    } else if constexpr (MODE == 2) {
+        if (KIND != KIND_KERR && (a.flags & GT_FLAG_PRECISE_MN))
+            trace_kernel<MODE, KIND, KIND != KIND_KERR, SINGLE><<<grid, block, 0, s>>>(a, one_shot);
+        else
+            trace_kernel<MODE, KIND, false, SINGLE><<<grid, block, 0, s>>>(a, one_shot);
+    } else {
+        trace_kernel<MODE, KIND><<<grid, block, 0, s>>>(a, one_shot);
+    }
+}
+
 template <int MODE, int KIND>
 static cudaError_t launch_one(const TraceArgs &a, int block, int grid, bool one_shot, cudaStream_t s)
 {
-    if constexpr (MODE == 2 && KIND != KIND_KERR) {
-        if (a.flags & GT_FLAG_PRECISE_MN) {
-            trace_kernel<MODE, KIND, true><<<grid, block, 0, s>>>(a, one_shot ? 1 : 0);
-            return cudaGetLastError();
-        }
-    }
-    if constexpr (MODE >= 4) {
-        if (KIND < KIND_ANY && a.pair_single)
-            pair_kernel<MODE, KIND, KIND < KIND_ANY><<<grid, block, 0, s>>>(a, one_shot ? 1 : 0);
-        else
-            pair_kernel<MODE, KIND, false><<<grid, block, 0, s>>>(a, one_shot ? 1 : 0);
-    } else
-        trace_kernel<MODE, KIND><<<grid, block, 0, s>>>(a, one_shot ? 1 : 0);
+    // (Kerr's FP32 step gains nothing from it, and compiles to other fused multiply-adds)
+    constexpr bool CAN_SINGLE =
+        (MODE == 2 && KIND == KIND_MN) || (MODE >= 4 && KIND < KIND_ANY);
+    if (CAN_SINGLE && a.single)
+        launch_kernel<MODE, KIND, CAN_SINGLE>(a, block, grid, one_shot ? 1 : 0, s);
+    else
+        launch_kernel<MODE, KIND, false>(a, block, grid, one_shot ? 1 : 0, s);
     return cudaGetLastError();
 }
 
@@ -1398,7 +1499,8 @@ static int occupancy_one(int block)
     int n = 0;
     cudaError_t e;
     if constexpr (MODE >= 4)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, pair_kernel<MODE, KIND, (KIND < KIND_ANY)>, block, 0);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+            &n, pair_kernel<MODE, KIND, (KIND < KIND_ANY)>, block, 0);
     else
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, trace_kernel<MODE, KIND>, block, 0);
     if (e != cudaSuccess) return 1;
