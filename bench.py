@@ -100,8 +100,8 @@ class ClockSampler:
 
 # ------------------------------------------------------------------ ncu traffic record
 # sources that define the ray-tracing kernels (a traffic record stays valid while they do)
-TRACE_SOURCES = ("trace.cu", "spacetime.cuh", "internal.cuh", "camera.cuh", "compensated.cuh",
-                 "df.cuh", "zone_df.cuh")
+TRACE_SOURCES = ("trace.cu", "trace_fp32.cu", "trace_body.cuh", "spacetime.cuh", "internal.cuh",
+                 "camera.cuh", "compensated.cuh", "df.cuh", "pair.cuh")
 
 
 def source_sha1() -> str:

@@ -21,6 +21,8 @@ INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xptxas", "-v",
          "-I" + INCLUDE]
+# flags of one translation unit (trace_fp32.cu says why)
+FILE_FLAGS = {"trace_fp32.cu": ["-ftz=true"]}
 
 
 def nvcc() -> str:
@@ -49,6 +51,7 @@ def _stale() -> bool:
 def _compile(src: str) -> tuple:
     obj = os.path.join(BUILD, os.path.basename(src)[:-3] + ".o")
     extra = os.environ.get("GT_NVCC_EXTRA", "").split()  # e.g. -DGT_FIELD_NOINLINE
+    extra = FILE_FLAGS.get(os.path.basename(src), []) + extra
     cmd = [nvcc()] + ARCH + FLAGS + extra + ["-c", src, "-o", obj]
     p = subprocess.run(cmd, capture_output=True, text=True)
     if p.returncode != 0:

@@ -380,7 +380,7 @@ int run_trace(gt_ctx *c, const CamDesc *d_cams, int n_cams, int kind_hint, int64
               int64_t n_rays, int64_t n_steps, double sp, int mode, double *t, double *r,
               double *th, double *ph, uint8_t *status, uint32_t *nsteps,
               const int64_t *fresh_ids = nullptr, const gt::RayParams *d_rays = nullptr,
-              bool compact_out = false, const Extra &x = Extra(), bool range_ok = true,
+              bool compact_out = false, const Extra &x = Extra(), bool range_ok = false,
               const CamDesc *one = nullptr)
 {
     const gt_options e = effective(c->opts);
@@ -416,6 +416,7 @@ int run_trace(gt_ctx *c, const CamDesc *d_cams, int n_cams, int kind_hint, int64
     a.disk = x.disk;
     a.z = x.z;
     a.states = x.states;
+    a.range_ok = range_ok ? 1 : 0;
     if (one) {
         a.pair = one->pair;
         a.stf = gt::to_float(one->st);
@@ -425,7 +426,7 @@ int run_trace(gt_ctx *c, const CamDesc *d_cams, int n_cams, int kind_hint, int64
         cudaMemsetAsync(c->d_scratch, 0, gt::SCR_WORDS * sizeof(unsigned long long), c->stream);
     if (err != cudaSuccess) return cuda_code(err);
     const bool one_shot = (e.flags & GT_FLAG_ONE_SHOT) != 0;
-    const int kmode64 = gt::fp64_kmode(a, kind_hint, range_ok);
+    const int kmode64 = gt::fp64_kmode(a, kind_hint);
     int rc;
     if (e.flags & GT_FLAG_GRAPH) {
         // the launch replayed from a CUDA graph, captured once per distinct launch and
@@ -712,7 +713,8 @@ int gt_trace_disk(gt_ctx *c, double r_in, double r_out, double half_thickness, i
     x.z = z;
     const int kind = (c->Q != 0.0) ? gt::KIND_MN : gt::KIND_KERR;
     return run_trace(c, c->d_cam, 1, kind, 0, (int64_t)c->res_x * c->res_y, n_steps, sp, mode, t,
-                     r, th, ph, status, nsteps, nullptr, nullptr, false, x, true, &c->cam);
+                     r, th, ph, status, nsteps, nullptr, nullptr, false, x,
+                     gt::pair_range(c->M, c->r0), &c->cam);
 }
 
 int gt_trace_states(gt_ctx *c, int64_t n, double *t, double *r, double *th, double *ph,
@@ -881,7 +883,7 @@ int gt_trace_rays(gt_ctx *c, int64_t n, const double *alpha, const double *beta,
     if (err != cudaSuccess) return cuda_code(err);
     // the kernel reads descriptor 0 before the per-ray set-up replaces it
     return run_trace(c, c->d_cam, 1, 2, 0, n, n_steps, sp, mode, t, r, th, ph, status, nsteps,
-                     nullptr, c->d_rays);
+                     nullptr, c->d_rays, false, Extra(), gt::pair_range(M, r0));
 }
 
 int gt_surrogate_infer(gt_ctx *c, gt_surrogate *s, const gt_gate_cfg *gate, int64_t n_steps,

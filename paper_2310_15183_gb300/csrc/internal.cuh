@@ -135,6 +135,7 @@ struct TraceArgs {
     PairSpacetime pair;
     SpacetimeF stf;
     int single;
+    int range_ok; // pair_range() of every camera of the launch
 };
 
 // Host-side validation shared by every entry point that takes a spacetime or a camera
@@ -176,12 +177,12 @@ inline void fill_desc(CamDesc &d, double M, double S, double Q, double r0, doubl
 // Kernel mode of a GT_MODE_FP64 launch: the double-float step for camera rays with exact
 // derivatives under RK4, whose scales stay well inside the float range; FP64 arithmetic for
 // the listing's numerics, the ring, caller states, per-ray spacetimes (a set-up per ray) and
-// other scales.  `range_ok` is pair_range() over the launch's cameras.
+// other scales.
 inline bool pair_range(double M, double r0) { return M >= 1e-3 && M <= 1e3 && r0 <= 1e5; }
 
-inline int fp64_kmode(const TraceArgs &a, int kind_hint, bool range_ok)
+inline int fp64_kmode(const TraceArgs &a, int kind_hint)
 {
-    return range_ok && a.sp >= 1e-9 && a.sp <= 1.0 && kind_hint != KIND_FD && !a.euler &&
+    return a.range_ok && a.sp >= 1e-9 && a.sp <= 1.0 && kind_hint != KIND_FD && !a.euler &&
                    !a.f32_io && !a.disk.on && !a.states.t && !a.rays
                ? KMODE_FP64_PAIR
                : KMODE_FP64;
@@ -197,6 +198,10 @@ cudaError_t launch_set_condition(cudaGraphConditionalHandle h, const unsigned lo
 int max_blocks_per_sm(int kmode, int kind_hint, int block);
 cudaError_t launch_trace(const TraceArgs &a, int kmode, int kind_hint, int block, int grid,
                          bool one_shot, cudaStream_t s);
+// The FP32 rounds kernel (trace_fp32.cu), for launches with a.range_ok.
+cudaError_t launch_trace_fp32(const TraceArgs &a, int kind_hint, int block, int grid, bool one_shot,
+                              cudaStream_t s);
+int max_blocks_per_sm_fp32(int kind_hint, int block);
 // The FP32 rounds kernel with two rays per thread (persistent launch only), when the
 // launch allows it (one camera of one spacetime kind; no watchdog, per-ray parameters,
 // state arrays or ring).

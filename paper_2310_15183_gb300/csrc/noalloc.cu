@@ -142,6 +142,7 @@ extern "C" int gt_trace_batch_noalloc(int device, void *cuda_stream, const gt_ca
     a.status = status;
     a.nsteps = nsteps;
     a.scratch = words;
+    a.range_ok = range_ok ? 1 : 0;
     a.zone_df = 1; // the context's default zone (double-float Manko-Novikov field)
     if (n_cams == 1) {
         a.pair = h[0].pair;
@@ -151,7 +152,7 @@ extern "C" int gt_trace_batch_noalloc(int device, void *cuda_stream, const gt_ca
     const int kind = any_mn && any_kerr ? 2 : (any_mn ? gt::KIND_MN : gt::KIND_KERR);
     const int block = 128;
     const int kmode =
-        mode == GT_MODE_FP64 ? gt::fp64_kmode(a, kind, range_ok) : gt::KMODE_MIXED_INLINE;
+        mode == GT_MODE_FP64 ? gt::fp64_kmode(a, kind) : gt::KMODE_MIXED_INLINE;
     const int fit = gt::max_blocks_per_sm(kmode, kind, block);
     const int grid = (fit < 4 ? fit : 4) * sms;
     // FP32-mixed runs its zone inline here: the park lists of the context path

@@ -8,7 +8,7 @@ import pytest
 
 from paper_2310_15183_gb300 import workloads as W
 
-from .parity import to_numpy
+from .parity import mixed_report, neighbour_band, to_numpy
 
 pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
@@ -85,3 +85,24 @@ def test_watchdog_stops_the_step_loop(tracer):
     tracer.set_options()
     tracer.set_camera(15.0, 1.2, 75.0, 8, 8)
     assert np.all(to_numpy(tracer.trace(100, 1.5e-4, 1))["nsteps"] == 100)
+
+
+
+
+@pytest.mark.parametrize("exponent", [-20, -9, 9, 11, 20])
+@pytest.mark.parametrize("Q", [0.0, 2.0])
+def test_units_of_length_on_both_sides_of_the_range(tracer, Q, exponent):
+    """Camera rays of ordinary scale run the flush-to-zero build of the FP32 kernel, other units
+    of length the one that keeps denormals (the line lies at M = 1e-3 and 1e3): frames of
+    either against the FP64 mode by the mixed mode's criteria, statuses of 99.9 % and end angles
+    within 1e-3 rad away from the shadow's edge.  (The pixel grid is not the same in every unit:
+    at 2^-11 its rays pass through the axis, where the two modes part.)"""
+    u = 2.0 ** exponent
+    nx, ny = 24, 18
+    tracer.set_spacetime(u, 0.48 * u * u, Q)  # S is an area, Q a pure number
+    tracer.set_camera(20.0 * u, 1.2, 60.0, nx, ny)
+    tracer.set_options()
+    ref, got = [to_numpy(tracer.trace(4000, 2e-2 * u, mode)) for mode in (0, 1)]
+    band = neighbour_band(ref["status"], nx, ny) | (ref["r"] < 4.0 * u)
+    rep = mixed_report(got, ref, exclude=band)
+    assert rep["n"] > 100 and rep["agree"] >= 0.999 and rep["max_angle"] <= 1e-3, rep
