@@ -288,6 +288,23 @@ GT_HD void p_sincos(DF th, float th2, const PairTables *__restrict__ tab, DF *so
     *co = p_add3(p_fma(C, cd, p_neg(p_mul(S, sd))), C3);
 }
 
+// sin and cos of th + d from s = sin th, c = cos th for the small angle of an RK4 stage,
+// |d| <= 2^-9: sin d = d - d^3/6 and cos d - 1 = -d^2/2 + d^4/24, each beyond d itself below
+// 2^-18 of the result, so in float; a third of p_sincos's instructions.  One table look-up a
+// step instead of four: the 256 x 256 Manko-Novikov FP64 frame 39.8 -> 38.6 ms, the 64 x 64
+// Schwarzschild one 4.26 -> 4.14 ms; frames of the zone as before (77.9 ms).
+GT_HD void p_rotate(DF s, DF c, DF d, DF *so, DF *co)
+{
+    const float t = GT_P_MUL(d.hi, d.hi);
+    const float s3 = GT_P_MUL(GT_P_MUL(t, d.hi), -1.0f / 6.0f);
+    // -(d.hi + d.lo)^2 / 2 with the product's error: t is 2^-18, its rounding 2^-43
+    const float te = fmaf(GT_P_ADD(d.hi, d.hi), d.lo, fmaf(d.hi, d.hi, -t));
+    const DF sd(d.hi, GT_P_ADD(d.lo, s3));
+    const DF cd(GT_P_MUL(-0.5f, t), fmaf(GT_P_MUL(t, t), 1.0f / 24.0f, GT_P_MUL(-0.5f, te)));
+    *so = p_add(p_fma(s, cd, p_mul(c, sd)), s);
+    *co = p_add(p_fma(c, cd, p_neg(p_mul(s, sd))), c);
+}
+
 // ------------------------------------------------------------------ coordinates
 // the leading pair, and the sum with a pair as a pair
 GT_HD DF tf_pair(TF t) { return DF(t.a, t.b); }

@@ -339,14 +339,14 @@ __device__ __forceinline__ bool pair_step(const PairSpacetime &c, const PairTabl
                                           TF sp, TF w6, DF &h_out)
 {
     const DF rp0 = tf_diff(x.r, c.r_plus);
-    DF rp = rp0, pr = tf_pair(x.pr), pth = tf_pair(x.pth), th = tf_pair(x.th);
+    DF rp = rp0, pr = tf_pair(x.pr), pth = tf_pair(x.pth), s1, c1;
+    p_sincos(tf_pair(x.th), x.th.c, tab, &s1, &c1);
+    DF s = s1, cs = c1;
     Rates<DF> k, acc;
     DF h(0.0f, 0.0f);
-    bool ok = fabsf(x.th.a) <= 128.0f;
+    bool ok = fabsf(x.th.a) <= 128.0f && fabsf(s1.hi) >= 1e-6f;
 #pragma unroll 1
     for (int stage = 0; stage < 4; stage++) {
-        DF s, cs;
-        p_sincos(th, x.th.c, tab, &s, &cs);
         if (KIND == KIND_MN || (KIND == KIND_ANY && c.kind == KIND_MN)) {
             float ex[4];
             mn_rates_pair(c, rp, s, cs, pr, pth, x.pt, x.pph, PairExp{tab}, k, ex);
@@ -355,7 +355,6 @@ __device__ __forceinline__ bool pair_step(const PairSpacetime &c, const PairTabl
         } else {
             kerr_rates_pair(c, rp, s, cs, pr, pth, x.pt, x.pph, k);
         }
-        ok = ok && fabsf(s.hi) >= 1e-6f;
         if (stage == 0) {
             h = p_norm(p_mul3(p_rcp(k.dt), sp));
             if (h.hi < 0.0f) h = p_neg(h);
@@ -372,9 +371,17 @@ __device__ __forceinline__ bool pair_step(const PairSpacetime &c, const PairTabl
         if (stage < 3) {
             const DF d = p_scale(h, stage < 2 ? 0.5f : 1.0f);
             rp = p_norm(p_fma(d, k.dr, rp0));
-            pr = p_norm(p_fma(d, k.dpr, tf_pair(x.pr)));
-            pth = p_norm(p_fma(d, k.dpth, tf_pair(x.pth)));
-            th = p_norm(p_fma(d, k.dth, tf_pair(x.th)));
+            pr = p_fma(d, k.dpr, tf_pair(x.pr));
+            pth = p_fma(d, k.dpth, tf_pair(x.pth));
+            const DF dth = p_norm(p_mul(d, k.dth));
+            if (fabsf(dth.hi) <= 0.001953125f) {
+                p_rotate(s1, c1, dth, &s, &cs);
+            } else { // a step of a radian's order
+                const DF th = p_norm(p_add(tf_pair(x.th), dth));
+                ok = ok && fabsf(th.hi) <= 128.0f;
+                p_sincos(th, x.th.c, tab, &s, &cs);
+            }
+            ok = ok && fabsf(s.hi) >= 1e-6f;
         }
     }
     // the sums of the stages are finite only if every rate was

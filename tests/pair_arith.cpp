@@ -189,11 +189,11 @@ struct StateTF {
 static void rk4_pair(const PairSpacetime &c, StateTF &x, TF sp, TF w6)
 { // the stages of the kernels' pair_step
     const DF rp0 = tf_diff(x.r, c.r_plus);
-    DF rp = rp0, pr = tf_pair(x.pr), pth = tf_pair(x.pth), th = tf_pair(x.th), h(0, 0);
+    DF rp = rp0, pr = tf_pair(x.pr), pth = tf_pair(x.pth), h(0, 0), s1, c1;
+    p_sincos(tf_pair(x.th), x.th.c, &TAB, &s1, &c1);
+    DF s = s1, cs = c1;
     Rates<DF> k, acc;
     for (int i = 0; i < 4; i++) {
-        DF s, cs;
-        p_sincos(th, x.th.c, &TAB, &s, &cs);
         rates_pair(c, rp, s, cs, pr, pth, x.pt, x.pph, k);
         if (i == 0) {
             h = p_norm(p_mul3(p_rcp(k.dt), sp));
@@ -212,9 +212,9 @@ static void rk4_pair(const PairSpacetime &c, StateTF &x, TF sp, TF w6)
         if (i < 3) {
             const DF d = p_scale(h, i < 2 ? 0.5f : 1.0f);
             rp = p_norm(p_fma(d, k.dr, rp0));
-            pr = p_norm(p_fma(d, k.dpr, tf_pair(x.pr)));
-            pth = p_norm(p_fma(d, k.dpth, tf_pair(x.pth)));
-            th = p_norm(p_fma(d, k.dth, tf_pair(x.th)));
+            pr = p_fma(d, k.dpr, tf_pair(x.pr));
+            pth = p_fma(d, k.dpth, tf_pair(x.pth));
+            p_rotate(s1, c1, p_norm(p_mul(d, k.dth)), &s, &cs);
         }
     }
     const DF w = p_norm(p_mul3(h, w6));
@@ -321,7 +321,7 @@ static void rates(double M, double S, double Q, double lo, double hi, const char
 
 int main()
 {
-    LD w[8] = {};
+    LD w[9] = {};
     for (int i = 0; i < 200000; i++) {
         const DF a = rnd(), b = rnd(), c = rnd();
         auto rel = [](LD got, LD want, LD scale) { return fabsl(got - want) / scale; };
@@ -338,14 +338,19 @@ int main()
         DF s, cs;
         p_sincos(tf_pair(th), th.c, &TAB, &s, &cs);
         w[6] = fmaxl(w[6], fmaxl(fabsl(ld(s) - sinl(ld(th))), fabsl(ld(cs) - cosl(ld(th)))));
+        const double d0 = uni(-1, 1) * ldexp(1.0, -(int)uni(9, 40));
+        const LD a0 = atan2l(ld(s), ld(cs)) + (LD)(float)d0; // the angle of the pair, turned
+        DF s2, c2;
+        p_rotate(s, cs, DF((float)d0, 0.0f), &s2, &c2);
+        w[8] = fmaxl(w[8], fmaxl(fabsl(ld(s2) - sinl(a0)), fabsl(ld(c2) - cosl(a0))));
         const TF t = tf((LD)uni(-20, 20) + uni(-1, 1) * 1e-18L);
         const DF d(uni(-1, 1) * ldexp(1.0, -(int)uni(0, 40)));
         if (fabsl(ld(t)) > 1e-3) w[7] = fmaxl(w[7], rel(ld(tf_add(t, d)), ld(t) + ld(d), fabsl(ld(t)) + fabsl(ld(d))));
     }
     printf("{\"mul\": %.2e, \"add\": %.2e, \"fma\": %.2e, \"rcp\": %.2e, \"rsqrt\": %.2e, \"exp\": %.2e, "
-           "\"sincos\": %.2e, \"tf_add\": %.2e, ",
+           "\"sincos\": %.2e, \"tf_add\": %.2e, \"rotate\": %.2e, ",
            (double)w[0], (double)w[1], (double)w[2], (double)w[3], (double)w[4], (double)w[5],
-           (double)w[6], (double)w[7]);
+           (double)w[6], (double)w[7], (double)w[8]);
     printf("\"rates\": {");
     rates(1, 0.9, 0, 1e-4, 0.1, "kerr near r_+");
     rates(1, 0.9, 0, 0.1, 20, "kerr");

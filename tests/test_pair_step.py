@@ -35,6 +35,7 @@ def test_pair_arithmetic_rates_and_trajectories(tmp_path):
     assert res["rcp"] <= 8 * u2 and res["rsqrt"] <= 12 * u2, res
     assert res["exp"] <= 2.0 ** -44 and res["sincos"] <= 2.0 ** -46, res
     assert res["tf_add"] <= 2.0 ** -61, res
+    assert res["rotate"] <= 2.0 ** -46, res  # absolute, as sincos: a handful of u^2
     for name, r in res["rates"].items():
         if name:
             assert r["n"] >= 5000, (name, r)
