@@ -200,7 +200,9 @@ GT_HD void mkvar(V1<T> &o, T v, T, T) { o = {v}; }
 // The rate functions take theta through s = sin(theta) and cs = cos(theta) (the *_sc
 // forms), so that a caller that already has them -- the FP32 RK4 step rotates the first
 // stage's pair to the later stages -- need not evaluate them again.
-template <class T>
+// OWN: the product a p_t inside the fused difference of d p_theta, the form the compiler takes
+// where the kind of spacetime is the ray's own (its default elsewhere differs by the last bit).
+template <class T, bool OWN = false>
 GT_HD void kerr_rates_sc(const SpacetimeT<T> &c, T r, T s, T cs, T pr, T pth, T pt, T pph,
                          Rates<T> &o)
 {
@@ -223,7 +225,8 @@ GT_HD void kerr_rates_sc(const SpacetimeT<T> &c, T r, T s, T cs, T pr, T pth, T 
     o.dt = (a * V * s - ra2 * WiD) * iSigma;
     o.dph = (V * is - a * WiD) * iSigma;
     const T Kr = T(2) * (r - M) * fma_t(pr, pr, WiD * WiD) - T(4) * r * pt * WiD;
-    const T Kth = T(2) * V * cs * (a * pt - pph * is2);
+    const T ap = OWN ? fma_t(a, pt, -(pph * is2)) : a * pt - pph * is2;
+    const T Kth = T(2) * V * cs * ap;
     const T KiS = K * iSigma;
     o.dpr = T(-0.5) * (Kr - T(2) * r * KiS) * iSigma;
     o.dpth = T(-0.5) * fma_t(T(2) * a2 * s * cs, KiS, Kth) * iSigma;

@@ -580,13 +580,13 @@ __device__ __forceinline__ void mixed_to64(const RayMixed &m, Ray64 &x)
 #define GT_FIELD_ATTR __forceinline__
 #endif
 
-template <int KIND, bool PRECISE>
+template <int KIND, bool PRECISE, bool OWN = false>
 __device__ GT_FIELD_ATTR void rates_f32(const SpacetimeF &st, float r, float s, float cs,
                                           float pr, float pth, float pt, float pph,
                                           Rates<float> &o)
 {
     if (KIND == KIND_KERR || (KIND == 2 && st.kind == KIND_KERR))
-        kerr_rates_sc<float>(st, r, s, cs, pr, pth, pt, pph, o);
+        kerr_rates_sc<float, OWN>(st, r, s, cs, pr, pth, pt, pph, o);
     else
         mn_rates_sc<float, PRECISE>(st, r, s, cs, pr, pth, pt, pph, o);
 }
@@ -643,12 +643,16 @@ __device__ __forceinline__ void rotate_series(float s, float c, float d, float *
     *c2 = fmaf(c, cd, -(s * sd));
 }
 
+// OWN: the bits of a field behind a branch on the ray's own kind of spacetime -- the rates rounded
+// before they are summed, except theta's.
+template <bool OWN>
 __device__ __forceinline__ float stage_sum(float k1, float k2, float k3, float k4)
 {
-    return __fmaf_rn(2.0f, k3, __fmaf_rn(2.0f, k2, k1)) + k4;
+    const float s = __fmaf_rn(2.0f, k3, __fmaf_rn(2.0f, k2, k1));
+    return OWN ? __fadd_rn(s, k4) : s + k4;
 }
 
-template <int KIND, bool PRECISE = false>
+template <int KIND, bool PRECISE = false, bool OWN = false>
 __device__ __forceinline__ float rk4_step32_fast(const SpacetimeF &st, RayMixed &m, float sp,
                                                  float w6, float &turn)
 {
@@ -656,29 +660,29 @@ __device__ __forceinline__ float rk4_step32_fast(const SpacetimeF &st, RayMixed 
     const float r = m.r.hi, th = m.th.hi, pr = m.pr.hi, pth = m.pth.hi;
     float s1, c1, s, c;
     sincosf(th, &s1, &c1);
-    rates_f32<KIND, PRECISE>(st, r, s1, c1, pr, pth, m.ptf, m.pphf, k1);
+    rates_f32<KIND, PRECISE, OWN>(st, r, s1, c1, pr, pth, m.ptf, m.pphf, k1);
     const float h = fabsf(sp / k1.dt);
     const float hh = 0.5f * h;
     const float d1 = __fmul_rn(hh, k1.dth);
     rotate_series(s1, c1, d1, &s, &c);
-    rates_f32<KIND, PRECISE>(st, fmaf(hh, k1.dr, r), s, c, fmaf(hh, k1.dpr, pr),
+    rates_f32<KIND, PRECISE, OWN>(st, fmaf(hh, k1.dr, r), s, c, fmaf(hh, k1.dpr, pr),
                              fmaf(hh, k1.dpth, pth), m.ptf, m.pphf, k2);
     const float d2 = __fmul_rn(hh, k2.dth);
     rotate_series(s1, c1, d2, &s, &c);
-    rates_f32<KIND, PRECISE>(st, fmaf(hh, k2.dr, r), s, c, fmaf(hh, k2.dpr, pr),
+    rates_f32<KIND, PRECISE, OWN>(st, fmaf(hh, k2.dr, r), s, c, fmaf(hh, k2.dpr, pr),
                              fmaf(hh, k2.dpth, pth), m.ptf, m.pphf, k3);
     const float d3 = __fmul_rn(h, k3.dth);
     rotate_series(s1, c1, d3, &s, &c);
-    rates_f32<KIND, PRECISE>(st, fmaf(h, k3.dr, r), s, c, fmaf(h, k3.dpr, pr),
+    rates_f32<KIND, PRECISE, OWN>(st, fmaf(h, k3.dr, r), s, c, fmaf(h, k3.dpr, pr),
                              fmaf(h, k3.dpth, pth), m.ptf, m.pphf, k4);
     turn = fmaxf(fmaxf(fabsf(d1), fabsf(d2)), fabsf(d3));
     const float hw = h * w6;
-    f2_add(m.t, hw * stage_sum(k1.dt, k2.dt, k3.dt, k4.dt));
-    f2_add(m.r, hw * stage_sum(k1.dr, k2.dr, k3.dr, k4.dr));
-    f2_add(m.th, hw * stage_sum(k1.dth, k2.dth, k3.dth, k4.dth));
-    f2_add(m.ph, hw * stage_sum(k1.dph, k2.dph, k3.dph, k4.dph));
-    f2_add(m.pr, hw * stage_sum(k1.dpr, k2.dpr, k3.dpr, k4.dpr));
-    f2_add(m.pth, hw * stage_sum(k1.dpth, k2.dpth, k3.dpth, k4.dpth));
+    f2_add(m.t, hw * stage_sum<OWN>(k1.dt, k2.dt, k3.dt, k4.dt));
+    f2_add(m.r, hw * stage_sum<OWN>(k1.dr, k2.dr, k3.dr, k4.dr));
+    f2_add(m.th, hw * stage_sum<false>(k1.dth, k2.dth, k3.dth, k4.dth));
+    f2_add(m.ph, hw * stage_sum<OWN>(k1.dph, k2.dph, k3.dph, k4.dph));
+    f2_add(m.pr, hw * stage_sum<OWN>(k1.dpr, k2.dpr, k3.dpr, k4.dpr));
+    f2_add(m.pth, hw * stage_sum<OWN>(k1.dpth, k2.dpth, k3.dpth, k4.dpth));
     return h;
 }
 
@@ -1131,7 +1135,14 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A, int one_shot)
             bool event;
             for (int q = 0;;) {
                 keep = m;
-                h = rk4_step32_fast<KIND, PRECISE>(sf, m, spf, w6f, turn);
+                if (KIND != KIND_ANY)
+                    h = rk4_step32_fast<KIND, PRECISE>(sf, m, spf, w6f, turn);
+                // one branch a step, none between its stages: a lone warp of Kerr rays with
+                // spacetimes of their own takes 374 ns a step (499 with a branch a stage)
+                else if (sf.kind == KIND_KERR)
+                    h = rk4_step32_fast<KIND_KERR, PRECISE, true>(sf, m, spf, w6f, turn);
+                else
+                    h = rk4_step32_fast<KIND_MN, PRECISE, true>(sf, m, spf, w6f, turn);
                 ++n;
                 const float sum = ((m.t.hi + m.th.hi) + (m.ph.hi + m.pr.hi)) + m.pth.hi;
                 event = !(m.r.hi < r_esc_f.hi && m.r.hi >= r_sw_f && h >= h_thr_f &&

@@ -87,6 +87,28 @@ def test_watchdog_stops_the_step_loop(tracer):
     assert np.all(to_numpy(tracer.trace(100, 1.5e-4, 1))["nsteps"] == 100)
 
 
+@pytest.mark.parametrize("flags", [0, 16])
+@pytest.mark.parametrize("n", [1, 33, 200])
+def test_rays_of_either_kind_with_their_own_spacetimes(tracer, n, flags):
+    """Kerr and Manko-Novikov rays side by side in a warp: the bits of each ray in a launch of
+    its own, and the FP64 mode by the mixed mode's criterion of 1e-3 rad."""
+    a = list(W.surrogate_samples(n, seed=3, q_max=2.0))
+    a[3] = np.where(np.arange(n) % 3 == 0, 0.0, a[3])
+    dev = [torch.tensor(v, device="cuda") for v in a]
+    tracer.set_options(flags=flags)
+
+    def rays(sel, mode):
+        return to_numpy(tracer.trace_rays(*[d[sel].contiguous() for d in dev], M=0.5, r0=15.0,
+                                          n_steps=600, step_precision=2e-2, mode=mode))
+
+    full, ref = rays(slice(None), 1), rays(slice(None), 0)
+    for k in range(0, n, max(1, n // 9)):
+        one = rays(slice(k, k + 1), 1)
+        for key in KEYS:
+            assert np.array_equal(one[key], full[key][k:k + 1], equal_nan=True), (k, key)
+    far = ref["r"] > 4.0
+    rep = mixed_report({k: v[far] for k, v in full.items()}, {k: v[far] for k, v in ref.items()})
+    assert far.sum() >= 0.8 * n and rep["agree"] >= 0.999 and rep["max_angle"] <= 1e-3, rep
 
 
 @pytest.mark.parametrize("exponent", [-20, -9, 9, 11, 20])
