@@ -1,11 +1,9 @@
-// mlp.cu -- tensor-core GEMM on tcgen05 (TMEM accumulators) for the surrogate network's
-// forward and backward passes.
+// mlp.cu -- tensor-core GEMM on tcgen05 (TMEM accumulators), the library call gt_gemm_bf16.
 //
 // gemm:  C[m, n] = sum_k A[m, k] B[n, k]  (+ bias[n]) (then SiLU)
 //   A element (m, k) at A[m * a_sm + k * a_sk], B element (n, k) at B[n * b_sn + k * b_sk]
-//   (bf16, or fp16 for both; any strides, so transposed operands need no copy), FP32
-//   accumulation in TMEM; outputs any of: FP32 C (stored, or added for split-K), the FP32
-//   pre-activation, a 16-bit copy and a transposed bf16 copy.
+//   (bf16, any strides, so transposed operands need no copy), FP32 accumulation in TMEM;
+//   FP32 C stored, or added (split-K, accumulation).
 //
 // Three kernels, chosen by operand layout:
 //  * tc_gemm_ws_kernel (K-contiguous operands with encodable TMA tensor maps): persistent,
@@ -19,7 +17,6 @@
 //  * tc_gemm_kernel (any strides): the same tile with register-staged loads.
 #include <cuda.h>
 #include <cuda_bf16.h>
-#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <cudaTypedefs.h>
 #include <stdint.h>
@@ -28,13 +25,26 @@
 #include <string.h>
 
 #include "../../include/geotrace.h"
-#include "mlp.cuh"
 #include "tc_gemm.cuh"
 #include "tma_map.cuh"
 
 namespace gt {
 
 namespace {
+
+struct GemmArgs {
+    int M, N, K;
+    const __nv_bfloat16 *A; // (m, k) at A[m * a_sm + k * a_sk]
+    int64_t a_sm, a_sk;
+    const __nv_bfloat16 *B; // (n, k) at B[n * b_sn + k * b_sk]
+    int64_t b_sn, b_sk;
+    const float *bias; // [N] or null
+    int act;           // 0 identity, 1 SiLU
+    float *C;          // fp32 output (ldc)
+    int64_t ldc;
+    int atomic;        // accumulate into C (split-K)
+    int *err;          // set to 1 when an mbarrier wait ran out
+};
 
 constexpr int BM = 128;
 constexpr int BK = 64;
@@ -93,57 +103,13 @@ __device__ __forceinline__ void stage_tile(uint8_t *sm, const __nv_bfloat16 *__r
 
 __device__ __forceinline__ float silu(float z) { return __fdividef(z, 1.0f + __expf(-z)); }
 
-// 16-bit output element (bf16, or fp16 bits stored in the same slot) and a packed pair
-__device__ __forceinline__ __nv_bfloat16 to_c16(float y, int f16)
-{
-    if (f16) {
-        const __half h = __float2half_rn(y);
-        return __ushort_as_bfloat16(__half_as_ushort(h));
-    }
-    return __float2bfloat16(y);
-}
-__device__ __forceinline__ uint32_t pack_c16(float lo, float hi, int f16)
-{
-    if (f16) {
-        const __half2 h = __floats2half2_rn(lo, hi);
-        return *reinterpret_cast<const uint32_t *>(&h);
-    }
-    const __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
-    return *reinterpret_cast<const uint32_t *>(&h);
-}
-
-// bf16 pair of y: hi = bf16(y) and lo = bf16(y - hi) (y - hi is exact in FP32), so that
-// hi + lo carries y to about 2^-17 relative
-__device__ __forceinline__ void split_bf16(float y, __nv_bfloat16 *hi, __nv_bfloat16 *lo)
-{
-    *hi = __float2bfloat16(y);
-    *lo = __float2bfloat16(y - __bfloat162float(*hi));
-}
-
-// One 16-bit output value: plain, or split into [hi | lo | hi] columns (c16_split)
-__device__ __forceinline__ void store_c16(const GemmArgs &g, int64_t row, int col, float y)
-{
-    __nv_bfloat16 *p = g.C16 + row * g.ldc16 + col;
-    if (g.c16_split) {
-        __nv_bfloat16 hi, lo;
-        split_bf16(y, &hi, &lo);
-        p[0] = hi;
-        p[g.N] = lo;
-        p[2 * g.N] = hi;
-    } else {
-        *p = to_c16(y, g.c16_f16);
-    }
-}
-
 // Epilogue shared by both kernels: TMEM -> registers (thread = row) -> bias -> shared
 // memory tile (32 columns at a time) -> coalesced stores where each warp writes
-// 32 consecutive columns of one row.  The transposed bf16 copy is written straight from
-// the row owner (consecutive lanes = consecutive rows, already coalesced).
+// 32 consecutive columns of one row.
 __device__ __forceinline__ void gemm_epilogue(const GemmArgs &g, uint32_t tmem, int BN_, int m0,
                                               int n0, bool have_acc, float *stage /* 128 x 33 */)
 {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int row_own = m0 + warp * 32 + lane;
     for (int cc = 0; cc < BN_; cc += 32) {
         float v[32];
         if (have_acc) {
@@ -158,9 +124,6 @@ __device__ __forceinline__ void gemm_epilogue(const GemmArgs &g, uint32_t tmem, 
             float z = v[i];
             if (g.bias && blockIdx.z == 0 && col < g.N) z += g.bias[col];
             stage[(warp * 32 + lane) * 33 + i] = z;
-            if (g.C16T && row_own < g.M && col < g.N)
-                g.C16T[(int64_t)col * g.ldt + row_own] =
-                    __float2bfloat16(g.act == 1 ? silu(z) : z);
         }
         __syncthreads();
         // 128 rows x 32 columns: warp w writes rows w, w + 4, ..., lane = column
@@ -170,16 +133,12 @@ __device__ __forceinline__ void gemm_epilogue(const GemmArgs &g, uint32_t tmem, 
                 const int row = m0 + rr;
                 if (row >= g.M) break;
                 const float z = stage[rr * 33 + lane];
-                if (g.pre) g.pre[(int64_t)row * g.ld_pre + col] = z;
                 const float y = g.act == 1 ? silu(z) : z;
-                if (g.C32) {
-                    float *p = g.C32 + (int64_t)row * g.ldc + col;
-                    if (g.atomic)
-                        atomicAdd(p, y);
-                    else
-                        *p = y;
-                }
-                if (g.C16) store_c16(g, row, col, y);
+                float *p = g.C + (int64_t)row * g.ldc + col;
+                if (g.atomic)
+                    atomicAdd(p, y);
+                else
+                    *p = y;
             }
         }
         __syncthreads();
@@ -217,7 +176,7 @@ __global__ void __launch_bounds__(128) tc_gemm_kernel(GemmArgs g)
     bool ok = true;
     const bool a_vec = (g.a_sk == 1) && (g.a_sm % 8 == 0) && ((uintptr_t)g.A % 16 == 0);
     const bool b_vec = (g.b_sk == 1) && (g.b_sn % 8 == 0) && ((uintptr_t)g.B % 16 == 0);
-    const uint32_t idesc = tc::idesc_f16_f32(BM, BN, g.f16_in == 0);
+    const uint32_t idesc = tc::idesc_bf16_f32(BM, BN);
 
     for (int c = 0; c < nk; ++c) {
         const int s = c & 1;
@@ -324,7 +283,7 @@ __global__ void __launch_bounds__(128) tc_gemm_pipe_kernel(GemmArgs g)
     tc::fence_after_sync();
     const uint32_t tmem = *tmem_slot;
     const uint32_t sbase = tc::smem_u32(smem);
-    const uint32_t idesc = tc::idesc_f16_f32(BM, BN, g.f16_in == 0);
+    const uint32_t idesc = tc::idesc_bf16_f32(BM, BN);
 
     auto issue = [&](int c) {
         const uint32_t a_s = sbase + (c % STAGES) * L::STAGE;
@@ -408,9 +367,8 @@ constexpr int EPI_WARPS = 8;
 constexpr int WS_THREADS = 64 + 32 * EPI_WARPS;
 
 // Per-epilogue-warp staging of the TMA-store epilogue: a 32 x 32 FP32 box (128-byte
-// swizzle), a 32 x 32 bf16 box (64-byte swizzle), a 32 x 32 transposed bf16 box (no
 // swizzle) and 32 bias values.
-constexpr uint32_t STG_F32 = 0, STG_B16 = 4096, STG_B16T = 6144, STG_BIAS = 8192, STG_WARP = 9216;
+constexpr uint32_t STG_F32 = 0, STG_BIAS = 4096, STG_WARP = 5120;
 
 template <int BN, int S, bool TMA_OUT>
 struct WsSmem {
@@ -429,14 +387,10 @@ struct WsSmem {
     static_assert(STAGE % 1024 == 0, "stage size keeps the staging boxes 1024-byte aligned");
 };
 
-struct OutMaps {
-    CUtensorMap c32, pre, c16, c16t;
-};
-
 template <int BN, int S, bool TMA_OUT>
 __global__ void __launch_bounds__(WS_THREADS, 1)
     tc_gemm_ws_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                      const __grid_constant__ OutMaps om, GemmArgs g, int splits)
+                      const __grid_constant__ CUtensorMap tmC, GemmArgs g, int splits)
 {
     using L = WsSmem<BN, S, TMA_OUT>;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -502,7 +456,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
         }
     } else if (warp == 1) {
         if (lane == 0) { // ---- MMA issuer
-            const uint32_t idesc = tc::idesc_f16_f32(BM, BN, g.f16_in == 0);
+            const uint32_t idesc = tc::idesc_bf16_f32(BM, BN);
             uint32_t q = 0, tl = 0;
             for (int t = blockIdx.x; t < total && ok; t += gridDim.x, ++tl) {
                 const int ks = t / (m_tiles * n_tiles);
@@ -538,8 +492,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
     } else if (TMA_OUT) { // ---- epilogue warps 2..9 storing through TMA
         const int quarter = warp & 3, half = (warp - 2) >> 2;
         uint8_t *stg = smem + S * L::STAGE + (warp - 2) * STG_WARP;
-        const uint32_t s_f32 = tc::smem_u32(stg + STG_F32), s_b16 = tc::smem_u32(stg + STG_B16),
-                       s_b16t = tc::smem_u32(stg + STG_B16T);
+        const uint32_t s_f32 = tc::smem_u32(stg + STG_F32);
         float *sbias = reinterpret_cast<float *>(stg + STG_BIAS);
         uint32_t tl = 0;
         for (int t = blockIdx.x; t < total && ok; t += gridDim.x, ++tl) {
@@ -578,92 +531,23 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
                         v[i + 3] += bb.w;
                     }
                 }
-                // FP32 box, row = lane, 16-byte chunk c at c ^ (row % 8)
-                auto put_f32 = [&]() {
-#pragma unroll
-                    for (int c = 0; c < 8; c++)
-                        *reinterpret_cast<float4 *>(stg + STG_F32 + lane * 128 + ((c ^ (lane & 7)) << 4)) =
-                            make_float4(v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]);
-                    tc::fence_proxy_async();
-                    __syncwarp();
-                };
-                if (g.pre) {
-                    put_f32();
-                    if (lane == 0) {
-                        tc::tma_store_2d(&om.pre, n0 + cc, m0, s_f32);
-                        tc::bulk_commit();
-                    }
-                }
                 if (g.act == 1) {
 #pragma unroll
                     for (int i = 0; i < 32; i++) v[i] = silu(v[i]);
                 }
-                if (g.C32) {
-                    if (g.pre) {
-                        if (lane == 0) tc::bulk_wait_read();
-                        __syncwarp();
-                    }
-                    put_f32();
-                    if (lane == 0) {
-                        if (g.atomic)
-                            tc::tma_reduce_add_2d(&om.c32, n0 + cc, m0, s_f32);
-                        else
-                            tc::tma_store_2d(&om.c32, n0 + cc, m0, s_f32);
-                        tc::bulk_commit();
-                    }
-                }
-                // 16-bit box, row = lane (64 bytes), chunk c at c ^ ((row / 2) % 4); with
-                // c16_split the hi halves first (the lo halves follow below)
-                auto put_b16 = [&](bool lo_part) {
+                // FP32 box, row = lane, 16-byte chunk c at c ^ (row % 8)
 #pragma unroll
-                    for (int c = 0; c < 4; c++) {
-                        uint4 w;
-                        uint32_t *wp = &w.x;
-#pragma unroll
-                        for (int j = 0; j < 4; j++) {
-                            const float a = v[8 * c + 2 * j], b = v[8 * c + 2 * j + 1];
-                            if (g.c16_split) {
-                                __nv_bfloat16 ha, la, hb, lb;
-                                split_bf16(a, &ha, &la);
-                                split_bf16(b, &hb, &lb);
-                                const __nv_bfloat162 h2 = lo_part ? __halves2bfloat162(la, lb)
-                                                                  : __halves2bfloat162(ha, hb);
-                                wp[j] = *reinterpret_cast<const uint32_t *>(&h2);
-                            } else {
-                                wp[j] = pack_c16(a, b, g.c16_f16);
-                            }
-                        }
-                        *reinterpret_cast<uint4 *>(stg + STG_B16 + lane * 64 +
-                                                   ((c ^ ((lane >> 1) & 3)) << 4)) = w;
-                    }
-                };
-                if (g.C16) put_b16(false);
-                if (g.C16T) { // transposed bf16 box: row = column i, element = lane
-#pragma unroll
-                    for (int i = 0; i < 32; i++)
-                        reinterpret_cast<__nv_bfloat16 *>(stg + STG_B16T)[i * 32 + lane] =
-                            __float2bfloat16(v[i]);
-                }
-                if (g.C16 || g.C16T) {
-                    tc::fence_proxy_async();
-                    __syncwarp();
-                    if (lane == 0) {
-                        if (g.C16) tc::tma_store_2d(&om.c16, n0 + cc, m0, s_b16);
-                        if (g.C16 && g.c16_split) tc::tma_store_2d(&om.c16, 2 * g.N + n0 + cc, m0, s_b16);
-                        if (g.C16T) tc::tma_store_2d(&om.c16t, m0, n0 + cc, s_b16t);
-                        tc::bulk_commit();
-                    }
-                }
-                if (g.C16 && g.c16_split) { // the lo halves into the middle N columns
-                    if (lane == 0) tc::bulk_wait_read();
-                    __syncwarp();
-                    put_b16(true);
-                    tc::fence_proxy_async();
-                    __syncwarp();
-                    if (lane == 0) {
-                        tc::tma_store_2d(&om.c16, g.N + n0 + cc, m0, s_b16);
-                        tc::bulk_commit();
-                    }
+                for (int c = 0; c < 8; c++)
+                    *reinterpret_cast<float4 *>(stg + STG_F32 + lane * 128 + ((c ^ (lane & 7)) << 4)) =
+                        make_float4(v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]);
+                tc::fence_proxy_async();
+                __syncwarp();
+                if (lane == 0) {
+                    if (g.atomic)
+                        tc::tma_reduce_add_2d(&tmC, n0 + cc, m0, s_f32);
+                    else
+                        tc::tma_store_2d(&tmC, n0 + cc, m0, s_f32);
+                    tc::bulk_commit();
                 }
                 __syncwarp();
             }
@@ -684,7 +568,6 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
             if (!ok) break;
             tc::fence_after_sync();
             const int m0 = mt * BM + quarter * 32, n0 = nt * BN;
-            const int row_own = m0 + lane;
             for (int cc = 32 * half; cc < BN; cc += 64) {
                 float v[32];
                 tc::tmem_ld32(tmem + (uint32_t)(b * BN + cc) + ((uint32_t)(quarter * 32) << 16), v);
@@ -692,16 +575,6 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
                 const int col = n0 + cc + lane;
                 const bool col_ok = cc + lane < BN && col < g.N;
                 const float bias = (g.bias && ks == 0 && col_ok) ? g.bias[col] : 0.f;
-                if (g.C16T) { // transposed bf16 copy, written by the row owner
-#pragma unroll
-                    for (int i = 0; i < 32; i++) {
-                        const float z = v[i] + __shfl_sync(0xffffffffu, bias, i);
-                        const int c = n0 + cc + i;
-                        if (row_own < g.M && cc + i < BN && c < g.N)
-                            g.C16T[(int64_t)c * g.ldt + row_own] =
-                                __float2bfloat16(g.act == 1 ? silu(z) : z);
-                    }
-                }
 #pragma unroll
                 for (int i = 0; i < 32; i++) stg[lane * 33 + i] = v[i];
                 __syncwarp();
@@ -712,16 +585,12 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
                         if (rr < nrows) {
                             const int64_t row = m0 + rr;
                             const float z = stg[rr * 33 + lane] + bias;
-                            if (g.pre) g.pre[row * g.ld_pre + col] = z;
                             const float y = g.act == 1 ? silu(z) : z;
-                            if (g.C32) {
-                                float *p = g.C32 + row * g.ldc + col;
-                                if (g.atomic)
-                                    atomicAdd(p, y);
-                                else
-                                    *p = y;
-                            }
-                            if (g.C16) store_c16(g, row, col, y);
+                            float *p = g.C + row * g.ldc + col;
+                            if (g.atomic)
+                                atomicAdd(p, y);
+                            else
+                                *p = y;
                         }
                     }
                 }
@@ -741,29 +610,29 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
 
 int g_sm_count = 0;
 
-// Output tensor map (2-D, row stride `ld` elements) with 32 x 32 boxes.
-bool make_out_map(CUtensorMap *m, void *base, CUtensorMapDataType dt, int esize, uint64_t rows,
-                  uint64_t cols, uint64_t ld, CUtensorMapSwizzle sw)
+// Tensor map of C (2-D, row stride `ld` elements) with 32 x 32 boxes.
+bool make_out_map(CUtensorMap *m, float *base, uint64_t rows, uint64_t cols, uint64_t ld)
 {
     auto enc = tma::encoder();
-    if (!enc || rows == 0 || cols == 0 || ((uintptr_t)base & 15) || (ld * esize) % 16) return false;
+    if (!enc || rows == 0 || cols == 0 || ((uintptr_t)base & 15) || (ld * 4) % 16) return false;
     cuuint64_t dims[2] = {cols, rows};
-    cuuint64_t strides[1] = {ld * esize};
+    cuuint64_t strides[1] = {ld * 4};
     cuuint32_t box[2] = {32, 32};
     cuuint32_t estr[2] = {1, 1};
-    return enc(m, dt, 2, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, sw,
+    return enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, base, dims, strides, box, estr,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 template <int BN, int S, bool TMA_OUT>
-cudaError_t launch_ws_kernel(const CUtensorMap &ta, const CUtensorMap &tb, const OutMaps &om,
+cudaError_t launch_ws_kernel(const CUtensorMap &ta, const CUtensorMap &tb, const CUtensorMap &tc_out,
                              const GemmArgs &g, int splits, int grid, cudaStream_t s)
 {
     using L = WsSmem<BN, S, TMA_OUT>;
     cudaError_t e = cudaFuncSetAttribute(tc_gemm_ws_kernel<BN, S, TMA_OUT>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, L::TOTAL);
     if (e != cudaSuccess) return e;
-    tc_gemm_ws_kernel<BN, S, TMA_OUT><<<grid, WS_THREADS, L::TOTAL, s>>>(ta, tb, om, g, splits);
+    tc_gemm_ws_kernel<BN, S, TMA_OUT><<<grid, WS_THREADS, L::TOTAL, s>>>(ta, tb, tc_out, g, splits);
     return cudaGetLastError();
 }
 
@@ -775,24 +644,10 @@ cudaError_t launch_ws(const GemmArgs &g, int splits, cudaStream_t s, bool *used)
     if (!tma::make_map(&ta, g.A, (uint64_t)g.M, (uint64_t)g.K, (uint64_t)g.a_sm, BM) ||
         !tma::make_map(&tb, g.B, (uint64_t)g.N, (uint64_t)g.K, (uint64_t)g.b_sn, BN))
         return cudaSuccess; // caller falls back
-    // TMA-store epilogue when every requested output has an encodable map
-    OutMaps om;
-    memset(&om, 0, sizeof(om));
-    bool tma_out = BN >= 32;
-    if (tma_out && g.C32)
-        tma_out = make_out_map(&om.c32, g.C32, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, g.M, g.N, g.ldc,
-                               CU_TENSOR_MAP_SWIZZLE_128B);
-    if (tma_out && g.pre)
-        tma_out = make_out_map(&om.pre, g.pre, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, g.M, g.N,
-                               g.ld_pre, CU_TENSOR_MAP_SWIZZLE_128B);
-    if (tma_out && g.C16)
-        tma_out = make_out_map(&om.c16, g.C16,
-                               g.c16_f16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16,
-                               2, g.M, g.c16_split ? 3 * (uint64_t)g.N : (uint64_t)g.N,
-                               g.ldc16, CU_TENSOR_MAP_SWIZZLE_64B);
-    if (tma_out && g.C16T)
-        tma_out = make_out_map(&om.c16t, g.C16T, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, g.N, g.M, g.ldt,
-                               CU_TENSOR_MAP_SWIZZLE_NONE);
+    // TMA-store epilogue when C has an encodable map
+    CUtensorMap c_map;
+    memset(&c_map, 0, sizeof(c_map));
+    const bool tma_out = BN >= 32 && make_out_map(&c_map, g.C, g.M, g.N, g.ldc);
     if (g_sm_count == 0) {
         int dev = 0;
         cudaGetDevice(&dev);
@@ -805,8 +660,8 @@ cudaError_t launch_ws(const GemmArgs &g, int splits, cudaStream_t s, bool *used)
     const int grid = (int)(total < g_sm_count ? total : g_sm_count);
     constexpr int S = BN >= 256 ? 3 : 4;
     *used = true;
-    return tma_out ? launch_ws_kernel<BN, S, true>(ta, tb, om, g, splits, grid, s)
-                   : launch_ws_kernel<BN, S, false>(ta, tb, om, g, splits, grid, s);
+    return tma_out ? launch_ws_kernel<BN, S, true>(ta, tb, c_map, g, splits, grid, s)
+                   : launch_ws_kernel<BN, S, false>(ta, tb, c_map, g, splits, grid, s);
 }
 
 template <int BN>
@@ -821,12 +676,11 @@ cudaError_t launch_bn(const GemmArgs &g, int splits, cudaStream_t s)
     return cudaGetLastError();
 }
 
-} // namespace
-
 // The warp-specialised TMA kernel is the default for K-contiguous operands; setting
 // GT_GEMM_NO_TMA in the environment selects the cp.async pipeline instead.
-static const bool g_use_ws = getenv("GT_GEMM_NO_TMA") == nullptr;
+const bool g_use_ws = getenv("GT_GEMM_NO_TMA") == nullptr;
 
+// bn in {16, 32, 64, 128, 256}; splits = K splits (gridDim.z).
 cudaError_t launch_gemm(const GemmArgs &g, int bn, int splits, cudaStream_t s)
 {
     if (splits < 1) splits = 1;
@@ -865,6 +719,8 @@ cudaError_t launch_gemm(const GemmArgs &g, int bn, int splits, cudaStream_t s)
     }
 }
 
+} // namespace
+
 } // namespace gt
 
 extern "C" int gt_gemm_bf16(int device, void *cuda_stream, int M, int N, int K, const void *A,
@@ -891,7 +747,7 @@ extern "C" int gt_gemm_bf16(int device, void *cuda_stream, int M, int N, int K, 
     g.b_sk = b_sk;
     g.bias = bias;
     g.act = act;
-    g.C32 = C;
+    g.C = C;
     g.ldc = ldc;
     g.atomic = accumulate || splits > 1;
     cudaError_t e = gt::launch_gemm(g, bn, splits, (cudaStream_t)cuda_stream);

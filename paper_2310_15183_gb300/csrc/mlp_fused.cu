@@ -199,8 +199,8 @@ __global__ void __launch_bounds__(THREADS, 1)
         }
     } else if (warp == 1) {
         if (lane == 0) { // ---- MMA
-            const uint32_t id_h = tc::idesc_f16_f32(TILE, 256, true);
-            const uint32_t id_o = tc::idesc_f16_f32(TILE, 16, true);
+            const uint32_t id_h = tc::idesc_bf16_f32(TILE, 256);
+            const uint32_t id_o = tc::idesc_bf16_f32(TILE, 16);
             uint32_t q = 0, hid = 0, acc = 0, tl = 0;
             auto full = [&](uint32_t j) {
                 if (ok) ok = tc::mbar_wait(FULL(j % RING), (j / RING) & 1, WAIT_LIMIT);
@@ -578,7 +578,7 @@ __global__ void __launch_bounds__(64 + 32 * WG_EPI, 1)
         }
     } else if (warp == 1) {
         if (lane == 0) {
-            const uint32_t idesc = tc::idesc_f16_f32(128, n_cols, true);
+            const uint32_t idesc = tc::idesc_bf16_f32(128, n_cols);
             uint32_t q = 0;
             for (int c = c0; c < c1 && ok; c++, q++) {
                 const uint32_t s = q % WG_RING;

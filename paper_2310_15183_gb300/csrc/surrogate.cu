@@ -1,15 +1,14 @@
 // surrogate.cu -- the MLP surrogate of the ray tracer: per-pixel (alpha, beta, spin,
 // q, theta0) -> (escape logit, end direction), trained on rays the integrator itself
-// produces, evaluated with the tcgen05 GEMM, and backed by the integrator for
-// low-confidence and photon-ring pixels.
+// produces, evaluated and trained by the fused tcgen05 kernels of mlp_fused.cu, and backed
+// by the integrator for low-confidence and photon-ring pixels.
 //
 // Network: 16 (5 inputs and 5 columns derived from them, zero padded) -> 256 -> 256 ->
 // 256 -> 256 -> 16 (4 used: logit and the unit vector of the end direction, which unlike
 // (theta, phi) has no jump at phi = +-pi), SiLU between layers.  FP32 master weights and
 // AdamW state.  The forward products are split-precision BF16: each layer input x and
 // weight w is carried as a bf16 pair (hi, lo), hi = bf16(v), lo = bf16(v - hi), and the
-// product is x_hi w_hi + x_lo w_hi + x_hi w_lo -- one tcgen05 GEMM over K' = 3K with the
-// input laid out [x_hi | x_lo | x_hi] and the weights [w_hi | w_hi | w_lo] -- which carries
+// product is x_hi w_hi + x_lo w_hi + x_hi w_lo in one accumulator, which carries
 // the layer to about 2^-16 relative instead of bf16's 2^-8 (the dropped x_lo w_lo term is
 // 2^-16 of the product); the end direction is read from the last layer, and a single
 // 16-bit product leaves a rounding floor of 5e-4 (FP16) to 2e-3 rad (BF16) under it.  The
@@ -27,7 +26,6 @@
 
 #include "../../include/geotrace.h"
 #include "internal.cuh"
-#include "mlp.cuh"
 #include "mlp_fused.cuh"
 #include "camera.cuh"
 #include "features.cuh"

@@ -1,6 +1,6 @@
 // tc_gemm.cuh -- fifth-generation tensor-core (tcgen05) building blocks for sm_103a:
 // TMEM allocation, UMMA shared-memory / instruction descriptors, kind::f16 MMA with
-// BF16 or FP16 operands and FP32 accumulation in TMEM, commit to an mbarrier, TMEM
+// BF16 operands and FP32 accumulation in TMEM, commit to an mbarrier, TMEM
 // loads, and the TMA bulk-tensor loads, stores and reductions with their mbarriers.
 //
 // Two operand layouts in shared memory, both K-major:
@@ -44,14 +44,12 @@ __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t saddr)
 }
 
 // 32-bit instruction descriptor of kind::f16: D = F32 (bits 4-5 = 1), A and B both BF16
-// (bits 7-9 = 1, 10-12 = 1) or both FP16 (0), both K-major (bits 15, 16 = 0), N >> 3 at
-// 17, M >> 4 at 24.
-__host__ __device__ constexpr uint32_t idesc_f16_f32(int M, int N, bool bf16)
+// (bits 7-9 = 1, 10-12 = 1), both K-major (bits 15, 16 = 0), N >> 3 at 17, M >> 4 at 24.
+__host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N)
 {
-    return (1u << 4) | ((bf16 ? 1u : 0u) << 7) | ((bf16 ? 1u : 0u) << 10) |
-           ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) |
+           ((uint32_t)(M >> 4) << 24);
 }
-__host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N) { return idesc_f16_f32(M, N, true); }
 
 __device__ __forceinline__ void tmem_alloc(uint32_t dst_smem, uint32_t ncols)
 {
