@@ -2,22 +2,28 @@
 // activations never leaving the SM; with TRAIN also the loss and the input gradients of the
 // same rows, followed by one launch for the weight gradients of all layers.
 //
-// Inference.  What bounds it: the split-precision products cost 48 MMAs (128 x 256 x 16, ~135 cycles each)
-// per hidden layer and tile, and SiLU two MUFU operations per element, 4,100 cycles of an SM's
+// Inference.  What bounds it: the split-precision products cost 48 MMAs (128 x 256 x 16, ~135
+// cycles each) per hidden layer and tile, and SiLU two MUFU operations per element, 4,100 cycles of an SM's
 // 16 a clock; layer-by-layer GEMMs added 3 KB of activations per row and layer through HBM and
 // L2, a pass for the features and one for the outputs.  Here a persistent CTA per SM keeps the
 // activations of its 128 rows in shared memory as the two bf16 halves (128 KB, the K-major
 // 128-byte-swizzled operand layout) and streams the weights from L2 in 64 x 256 boxes through
 // a ring of three (96 KB; the last layer's 24 KB in one slot).  Two accumulators in TMEM
-// alternate, and the epilogue hands over its output in K-chunks of 64 columns, so the next
-// layer's x_hi w_hi pass follows it chunk by chunk.  The MMAs run in the order x_hi w_hi
-// (K = 0..255), x_lo w_hi, x_hi w_lo of the split GEMM of the training path: same bits.
+// alternate, and the epilogue hands over its output in K-chunks of 64 columns, which the next
+// layer's MMAs follow: all three products of a chunk at once, so that only the last chunk's
+// 12 MMAs remain when the epilogue is done, and w_hi is fetched once (256 KB a layer).
+// Training, whose parameters after many steps carry any change of rounding, and images, whose
+// end angles are stored in FP64 and whose gates are decided by the logits' last bits, keep the
+// order of the split GEMM, x_hi w_hi (K = 0..255), x_lo w_hi, x_hi w_lo: its first third follows
+// the chunks and 32 MMAs remain.
 //
-// Measured on one GB300: 2^20 rows 3.19 -> 1.37 ms, 300 rows 105 -> 59 us (49 us with the error flag in host memory) (the GEMM per
-// layer: 0.9 ms of MMAs at 0.47 of the bf16 peak, the rest traffic and SiLU passes).  Tried and
-// not kept: two halves of 128 columns per layer with w_hi held for both passes, 256 instead
-// of 384 KB of weights a layer (1.87 ms: an MMA takes ~105 cycles at N = 128 against ~135 at
-// N = 256); the accumulator handed over whole (1.60 ms).
+// Measured on one GB300: 2^20 rows 3.19 ms with a GEMM per layer (0.9 ms of MMAs at 0.47 of
+// the bf16 peak, the rest traffic and SiLU passes), 1.37 in one kernel, 1.13 with a chunk's
+// products together; 300 rows 103 us, 49 and 43.  Error against FP64 over 128 to 4,096 rows:
+// 4.9e-7 rms (5.1e-7 in the order of the split GEMM).  Tried and not kept: two halves of 128 columns per layer with
+// w_hi held for both passes (1.87 ms: an MMA takes ~105 cycles at N = 128 against ~135 at
+// N = 256); the accumulator handed over whole (1.60 ms); the TMEM load of the next chunk
+// started before this one's SiLU (1.23 against 1.13 ms: spills at 80 registers).
 //
 // Training.  A step of 8,192 rows was 37 launches and 467 us on the device: four SiLU-backward
 // passes that read row-major FP32 matrices down their columns (46 us each), five column sums
@@ -27,11 +33,11 @@
 // thread stored (512 KB per CTA, in L2), the transposed bf16 copies for the weight gradients
 // and the column sums; MMA order and elementwise formulas are those of the separate kernels.  A
 // step is four launches: clear, fused, weight gradients, AdamW with both weight copies.
-// Measured: 8 steps of 8,192 rows 3.88 -> 0.91 ms; loss and gradients of 16,384 rows with
-// their copy to the host 743 -> 156 us.
+// Measured: 8 steps of 8,192 rows 3.88 -> 0.87 ms; loss and gradients of 16,384 rows with
+// their copy to the host 743 -> 152 us.
 //
-// Warps: 0 loads, 1 issues the MMAs, 2-5 compute the next tile's features while the
-// current one runs (and its labels), 6-21 drain the accumulator: bias, SiLU, split, back into the operand
+// Warps: 0 loads, 1 issues the MMAs, 2-5 compute the next tile's features (and labels) while
+// the current one runs, 6-21 drain the accumulator: bias, SiLU, split, back into the operand
 // buffer.  All hand-offs are mbarriers with bounded waits; a wait that runs out sets the
 // error flag and every role leaves its loop.
 #include <cuda.h>
@@ -165,6 +171,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     __syncthreads();
     tc::fence_after_sync();
     const uint32_t tmem = *tmem_slot;
+    const bool by_chunk = !TRAIN && g.cam == nullptr; // order of a hidden layer's MMAs
     bool ok = true;
 
     if (warp == 0) {
@@ -184,8 +191,16 @@ __global__ void __launch_bounds__(THREADS, 1)
             };
             for (int64_t t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
                 load(0, 0, 1, WBOX);
-                for (int l = 1; l < N_LAYERS - 1; l++)
-                    for (int k = 0; k < 12; k++) load(l, k, 1, WBOX); // w_hi, w_hi, w_lo
+                for (int l = 1; l < N_LAYERS - 1; l++) {
+                    if (by_chunk) {
+                        for (int k = 0; k < 4; k++) {
+                            load(l, k, 1, WBOX);     // w_hi
+                            load(l, 8 + k, 1, WBOX); // w_lo
+                        }
+                    } else {
+                        for (int k = 0; k < 12; k++) load(l, k, 1, WBOX); // w_hi, w_hi, w_lo
+                    }
+                }
                 load(N_LAYERS - 1, 0, 12, OBOX); // the last layer's 24 KB in one slot
                 if (TRAIN) {
                     load(-(N_LAYERS - 1), 0, 1, WBOX);
@@ -238,7 +253,16 @@ __global__ void __launch_bounds__(THREADS, 1)
                 ++acc;
                 for (int l = 1; l < N_LAYERS - 1 && ok; l++, hid++, acc++) {
                     const uint32_t d = tmem + 256 * (acc & 1);
-                    for (uint32_t k = 0; k < 12 && ok; k++, q++) { // x_hi w_hi, x_lo w_hi, x_hi w_lo
+                    for (uint32_t k = 0; k < 4 && ok && by_chunk; k++, q += 2) {
+                        if (!input(k) || !full(q)) break;
+                        mma4(d, k, slot(q), id_h, k == 0); // x_hi w_hi
+                        mma4(d, 4 + k, slot(q), id_h, false); // x_lo w_hi
+                        tc::mma_commit(EMPTY(q % RING));
+                        if (!full(q + 1)) break;
+                        mma4(d, k, slot(q + 1), id_h, false); // x_hi w_lo
+                        tc::mma_commit(EMPTY((q + 1) % RING));
+                    }
+                    for (uint32_t k = 0; k < 12 && ok && !by_chunk; k++, q++) { // x_hi w_hi, x_lo w_hi, x_hi w_lo
                         if (k < 4 && !input(k)) break;
                         if (!full(q)) break;
                         mma4(d, k < 8 ? k : k - 8, slot(q), id_h, k == 0);
