@@ -59,7 +59,10 @@ extern "C" {
 #define GT_RAY_DISK 5 /* entered the ring volume (gt_trace_disk) */
 
 /* arithmetic modes */
-#define GT_MODE_FP64 0       /* FP64 end to end */
+#define GT_MODE_FP64 0       /* FP64 accuracy: FP64 end to end, or, for camera rays in ordinary
+                              * units (M in [1e-3, 1e3], r0 <= 1e5, step in [1e-9, 1]) with exact
+                              * derivatives, double-float steps on a state of three floats per
+                              * coordinate whose end states are as close to the exact flow */
 #define GT_MODE_FP32_MIXED 1 /* FP32 RK4 with compensated state; a zone r < r_switch stepped with
                               * an FP64 state (its field and stage arithmetic in double-float
                               * where the evaluation's range allows, else FP64) and H = 0
@@ -228,9 +231,9 @@ int gt_trace_states(gt_ctx *ctx, int64_t n, double *t, double *r, double *theta,
 /* ---------------------------------------------------------------------------------
  * Surrogate: an MLP (alpha, beta, spin a/M, q, theta0) -> (escape logit, unit end
  * direction) with layers 16(10 used) -> 256 -> 256 -> 256 -> 256 -> 16(4 used), SiLU,
- * on tcgen05 tensor cores with FP32 accumulation: FP16 weights and activations in the
- * forward products, BF16 in the backward products, FP32 master weights and AdamW.  Trained on rays traced by the integrator; the integrator
- * is its fallback.  Not part of the paper's method. */
+ * on tcgen05 tensor cores with FP32 accumulation: weights and activations as BF16 pairs in
+ * the forward products, BF16 in the backward products, FP32 master weights and AdamW.
+ * Trained on rays traced by the integrator; the integrator is its fallback.  Not part of the paper's method. */
 typedef struct gt_surrogate gt_surrogate;
 
 /* Input ranges the features are normalised over: camera distance r0 and field of view

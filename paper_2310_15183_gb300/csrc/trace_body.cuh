@@ -1115,14 +1115,16 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A, int one_shot)
                 }
             }
         } else { // MODE 2: FP32 steps only, exit tests in FP32
-            // What bounds it: issue slots with four warps a scheduler (the FP32 pipe is busy 70 to
-            // 73 % of the cycles, a slot used in 82 to 84 %), the dependent chain of a step with
-            // fewer -- and a terminating image ends on its longest rays, 450,000 steps of a lone
-            // warp where the mean is 250,000.  Votes, refills and exit tests per step, three
-            // branches around the stage rotations and the spacetime's constants in registers
-            // cost both: a step is 417 instructions (Kerr; 482 before) and 1,261 (Manko-
-            // Novikov; 1,318), a lone Kerr warp takes 764 cycles a step (1,284), a full chip 505 a
-            // warp (641); Manko-Novikov 1,880 (2,550) and 1,470 (1,676).
+            // What bounds it: issue slots with four warps a scheduler (the FP32 pipe is busy 73 % of
+            // the cycles, a slot used in 83 %), the dependent chain of a step with fewer -- and a
+            // terminating image ends on its longest rays, 450,000 steps of a lone warp where the
+            // mean is 250,000.  Votes, refills and exit tests per step, three branches around the
+            // stage rotations and the spacetime's constants in registers cost both.  In the
+            // flush-to-zero build a step is 396 instructions (Kerr) and 1,127 (Manko-Novikov), 482
+            // and 1,318 with all of these; a lone Kerr warp takes 686 cycles a step (1,284), a full
+            // chip 481 a warp (641); Manko-Novikov 1,611 (2,550) and 1,331 (1,676).  Two steps per
+            // iteration spare the copy of the state but not the instruction cache: a lone Kerr
+            // warp 665 cycles, a full chip 530, Manko-Novikov 2,630 and 1,500.
             // Steps back to back until some lane of the warp has something to do: an exit, the
             // zone, a re-projection, a stage angle the fast step does not take.  One test covers
             // them all (the sum is finite only if every coordinate is; r within [r_switch,
