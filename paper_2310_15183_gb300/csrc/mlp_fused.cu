@@ -33,8 +33,10 @@
 // thread stored (512 KB per CTA, in L2), the transposed bf16 copies for the weight gradients
 // and the column sums; MMA order and elementwise formulas are those of the separate kernels.  A
 // step is four launches: clear, fused, weight gradients, AdamW with both weight copies.
-// Measured: 8 steps of 8,192 rows 3.88 -> 0.87 ms; loss and gradients of 16,384 rows with
-// their copy to the host 743 -> 152 us.
+// A step of 8,192 rows is one tile a CTA, run once: four copies of the epilogue's chunk loop
+// cost 15,000 of the kernel's 155,000 cycles in instruction fetches, so training rolls it.
+// Measured: 8 steps of 8,192 rows 3.88 -> 0.85 ms; loss and gradients of 16,384 rows with
+// their copy to the host 743 -> 142 us.
 //
 // Warps: 0 loads, 1 issues the MMAs, 2-5 compute the next tile's features (and labels) while
 // the current one runs, 6-21 drain the accumulator: bias, SiLU, split, back into the operand
@@ -368,7 +370,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                 tc::fence_after_sync();
                 const uint32_t src = t_row + 256 * (acc & 1) + 16 * group;
                 const float4 *b4 = reinterpret_cast<const float4 *>(g.bias[l] + 16 * group);
-#pragma unroll
+#pragma unroll (TRAIN ? 1 : 4)
                 for (int k = 0; k < 4; k++) {
                     float v[16];
                     tc::tmem_ld16(src + 64 * k, v);
@@ -488,7 +490,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                 if (!ok) break;
                 tc::fence_after_sync();
                 const uint32_t src = t_row + 256 * (acc & 1) + 16 * group;
-#pragma unroll
+#pragma unroll 1
                 for (int k = 0; k < 4; k++) {
                     float v[16];
                     tc::tmem_ld16(src + 64 * k, v);
