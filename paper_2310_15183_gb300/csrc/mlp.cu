@@ -167,7 +167,7 @@ __global__ void __launch_bounds__(128) tc_gemm_kernel(GemmArgs g)
     if (tid == 0) {
         tc::mbar_init(tc::smem_u32(&mbar[0]), 1);
         tc::mbar_init(tc::smem_u32(&mbar[1]), 1);
-        asm volatile("fence.mbarrier_init.release.cluster;");
+        tc::fence_mbarrier_init();
     }
     tc::fence_before_sync();
     __syncthreads();
@@ -233,11 +233,15 @@ __global__ void __launch_bounds__(128) tc_gemm_kernel(GemmArgs g)
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, uint32_t src_bytes)
 {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src),
-                 "r"(src_bytes));
+                 "r"(src_bytes)
+                 : "memory");
 }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;"); }
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N)); }
+__device__ __forceinline__ void cp_async_wait()
+{
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
 
 __device__ __forceinline__ void issue_tile(uint32_t s_base, const __nv_bfloat16 *__restrict__ src,
                                            int rows_total, int k_total, int64_t s_row, int row0,
@@ -276,7 +280,7 @@ __global__ void __launch_bounds__(128) tc_gemm_pipe_kernel(GemmArgs g)
     if (warp == 0) tc::tmem_alloc(tc::smem_u32(tmem_slot), NCOLS);
     if (tid == 0) {
         for (int st = 0; st < STAGES; st++) tc::mbar_init(tc::smem_u32(&mbar[st]), 1);
-        asm volatile("fence.mbarrier_init.release.cluster;");
+        tc::fence_mbarrier_init();
     }
     tc::fence_before_sync();
     __syncthreads();
@@ -421,7 +425,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
             tc::mbar_init(ACCE(b), EPI_WARPS);
         }
         tc::mbar_init(DONE, 1);
-        asm volatile("fence.mbarrier_init.release.cluster;");
+        tc::fence_mbarrier_init();
         asm volatile("prefetch.tensormap [%0];" ::"l"(&tmA) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(&tmB) : "memory");
     }

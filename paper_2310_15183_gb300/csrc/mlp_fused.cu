@@ -176,7 +176,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         tc::mbar_init(TAIL, 1);
         tc::mbar_init(FEAT, FEAT_WARPS);
         tc::mbar_init(DONE, 1);
-        asm volatile("fence.mbarrier_init.release.cluster;");
+        tc::fence_mbarrier_init();
     }
     tc::fence_before_sync();
     __syncthreads();
@@ -586,7 +586,7 @@ __global__ void __launch_bounds__(64 + 32 * WG_EPI, 1)
             tc::mbar_init(EMPTY(s), 1);
         }
         tc::mbar_init(ACC, 1);
-        asm volatile("fence.mbarrier_init.release.cluster;");
+        tc::fence_mbarrier_init();
     }
     tc::fence_before_sync();
     __syncthreads();

@@ -1,0 +1,40 @@
+"""Ordering in the hand-written kernels, read from their source: what a build may reorder shows
+on a GPU only as a rare wrong result, so the statements that forbid it are checked as text."""
+import glob
+import os
+import re
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
+                    "paper_2310_15183_gb300", "csrc")
+SOURCES = sorted(glob.glob(os.path.join(CSRC, "*.cu")) + glob.glob(os.path.join(CSRC, "*.cuh")))
+# instructions that order, publish or wait for memory accesses of other instructions
+ORDERING = re.compile(r"fence\.|mbarrier\.|cp\.async|cp\.reduce|red\.|bar\.|barrier\.|"
+                      r"tcgen05\.(alloc|dealloc|relinquish|commit|fence|wait|st|cp)")
+
+
+def _code(path):
+    """The file without comments."""
+    with open(path) as f:
+        return re.sub(r"//[^\n]*|/\*.*?\*/", "", f.read(), flags=re.S)
+
+
+def _asm_statements(path):
+    text = _code(path)
+    for m in re.finditer(r"\basm\b", text):
+        depth, i = 0, text.index("(", m.start())
+        for j in range(i, len(text)):
+            depth += {"(": 1, ")": -1}.get(text[j], 0)
+            if depth == 0:
+                yield text[m.start():j + 1]
+                break
+
+
+@pytest.mark.parametrize("path", SOURCES, ids=os.path.basename)
+def test_ordering_instructions_hold_memory_accesses(path):
+    """Each such statement is volatile and clobbers memory: a compiler may otherwise move an
+    ordinary shared-memory store of an operand past the fence its reader relies on."""
+    for s in _asm_statements(path):
+        if ORDERING.search(s):
+            assert re.match(r"asm\s+volatile", s) and '"memory"' in s, s
