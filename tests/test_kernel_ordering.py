@@ -38,3 +38,12 @@ def test_ordering_instructions_hold_memory_accesses(path):
     for s in _asm_statements(path):
         if ORDERING.search(s):
             assert re.match(r"asm\s+volatile", s) and '"memory"' in s, s
+
+
+@pytest.mark.parametrize("path", SOURCES, ids=os.path.basename)
+def test_tensor_memory_loads_wait_in_their_own_statement(path):
+    """tcgen05.ld returns before its registers hold the data; a wait in a statement of its own
+    says nothing about those registers to the compiler."""
+    for s in _asm_statements(path):
+        if "tcgen05.ld" in s:
+            assert s.find("tcgen05.wait::ld") > s.find("tcgen05.ld."), s
