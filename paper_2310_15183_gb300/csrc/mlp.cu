@@ -512,7 +512,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
                 const int col = n0 + 32 * half + 64 * j + lane;
                 bl[j] = (has_bias && 32 * half + 64 * j < BN && col < g.N) ? __ldg(g.bias + col) : 0.f;
             }
-            ok = tc::mbar_wait(ACCF(b), (tl >> 1) & 1, WAIT_LIMIT);
+            ok = tc::mbar_wait_warp(ACCF(b), (tl >> 1) & 1, WAIT_LIMIT);
             if (!ok) break;
             tc::fence_after_sync();
 #pragma unroll
@@ -568,7 +568,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
         for (int t = blockIdx.x; t < total && ok; t += gridDim.x, ++tl) {
             const int nt = t % n_tiles, mt = (t / n_tiles) % m_tiles, ks = t / (m_tiles * n_tiles);
             const int b = tl & 1;
-            ok = tc::mbar_wait(ACCF(b), (tl >> 1) & 1, WAIT_LIMIT);
+            ok = tc::mbar_wait_warp(ACCF(b), (tl >> 1) & 1, WAIT_LIMIT);
             if (!ok) break;
             tc::fence_after_sync();
             const int m0 = mt * BM + quarter * 32, n0 = nt * BN;

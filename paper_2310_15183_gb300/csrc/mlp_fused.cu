@@ -342,7 +342,7 @@ __global__ void __launch_bounds__(THREADS, 1)
             split8(f, hi[0], lo[0]);
             split8(f + 8, hi[1], lo[1]);
             // the previous tile's last layer has read the operand buffer
-            if (tl > 0) ok = tc::mbar_wait(TAIL, (tl - 1) & 1, WAIT_LIMIT);
+            if (tl > 0) ok = tc::mbar_wait_warp(TAIL, (tl - 1) & 1, WAIT_LIMIT);
             if (!ok) break;
             // row [hi 0..15 | lo 0..15 | hi 0..15 | 0] of one 64-wide chunk
             uint8_t *base = smem + row * 128;
@@ -374,7 +374,7 @@ __global__ void __launch_bounds__(THREADS, 1)
             const int64_t r = t * TILE + row;
             for (int l = 0; l < N_LAYERS - 1 && ok; l++, acc++) {
                 // two barriers in turn: one flips again only after every warp has passed it
-                ok = tc::mbar_wait(ACC(acc & 1), (acc >> 1) & 1, WAIT_LIMIT);
+                ok = tc::mbar_wait_warp(ACC(acc & 1), (acc >> 1) & 1, WAIT_LIMIT);
                 if (!ok) break;
                 tc::fence_after_sync();
                 const uint32_t src = t_row + 256 * (acc & 1) + 16 * group;
@@ -416,7 +416,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                 }
             }
             if (!ok) break;
-            ok = tc::mbar_wait(ACC(acc & 1), (acc >> 1) & 1, WAIT_LIMIT);
+            ok = tc::mbar_wait_warp(ACC(acc & 1), (acc >> 1) & 1, WAIT_LIMIT);
             if (!ok) break;
             if (!TRAIN && group == 0) {
                 tc::fence_after_sync();
@@ -439,7 +439,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                 }
             }
             if (TRAIN && group == 0) { // ---- loss and its gradient, one row a thread
-                ok = tc::mbar_wait(FEAT, tl & 1, WAIT_LIMIT); // the labels, written with the features
+                ok = tc::mbar_wait_warp(FEAT, tl & 1, WAIT_LIMIT); // the labels, written with the features
                 if (!ok) break;
                 tc::fence_after_sync();
                 float v[16];
@@ -495,7 +495,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                 const float *zl = zrow + (int64_t)l * 256 * TILE;
 #pragma unroll
                 for (int j = 0; j < 16; j++) z[j] = zl[j * TILE];
-                ok = tc::mbar_wait(ACC(acc & 1), (acc >> 1) & 1, WAIT_LIMIT);
+                ok = tc::mbar_wait_warp(ACC(acc & 1), (acc >> 1) & 1, WAIT_LIMIT);
                 if (!ok) break;
                 tc::fence_after_sync();
                 const uint32_t src = t_row + 256 * (acc & 1) + 16 * group;
@@ -635,7 +635,7 @@ __global__ void __launch_bounds__(64 + 32 * WG_EPI, 1)
         }
     } else if (c1 > c0) {
         const int quarter = warp & 3, half = (warp - 2) >> 2, n = m0 + quarter * 32 + lane;
-        ok = tc::mbar_wait(ACC, 0, WAIT_LIMIT);
+        ok = tc::mbar_wait_warp(ACC, 0, WAIT_LIMIT);
         tc::fence_after_sync();
         for (int col = 32 * half; col < n_cols && ok; col += 64) {
             float v[32];

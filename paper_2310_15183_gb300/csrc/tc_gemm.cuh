@@ -123,6 +123,13 @@ __device__ __forceinline__ bool mbar_wait(uint32_t mbar_smem, uint32_t parity, u
     return false;
 }
 
+// The same for a whole warp, with one outcome: where a wait runs out for some lanes and not for
+// others, those that left would be missed by the warp's next collective instruction.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t mbar_smem, uint32_t parity, uint32_t limit)
+{
+    return __all_sync(0xffffffffu, mbar_wait(mbar_smem, parity, limit)) != 0;
+}
+
 // 32 lanes x 32 consecutive FP32 columns: thread t of warp w receives TMEM lane
 // 32 (w % 4) + t, columns [col, col + 32).  The load and its wait are one statement: the
 // registers are defined only after the wait, and as two the compiler might use them between.

@@ -47,3 +47,39 @@ def test_tensor_memory_loads_wait_in_their_own_statement(path):
     for s in _asm_statements(path):
         if "tcgen05.ld" in s:
             assert s.find("tcgen05.wait::ld") > s.find("tcgen05.ld."), s
+
+
+def _kernels(text):
+    """Bodies of the __global__ functions."""
+    for m in re.finditer(r"__global__", text):
+        i = text.index("{", text.index(")\n{", m.start()))
+        depth = 0
+        for j in range(i, len(text)):
+            depth += {"{": 1, "}": -1}.get(text[j], 0)
+            if depth == 0:
+                yield text[i:j + 1]
+                break
+
+
+def _enclosing(body, pos):
+    """Heads (the text since the statement before) of the blocks around a position."""
+    stack = []
+    for j in range(pos):
+        if body[j] == "{":
+            stack.append(body[max(body.rfind(c, 0, j) for c in ";{}") + 1:j])
+        elif body[j] == "}":
+            stack.pop()
+    return stack
+
+
+@pytest.mark.parametrize("path", SOURCES, ids=os.path.basename)
+def test_a_bounded_wait_has_one_outcome_per_warp(path):
+    """A wait that may run out is taken by one lane, by the warp as one (mbar_wait_warp), or its
+    outcome is joined over the CTA (__syncthreads_and): lanes that left a loop on their own would
+    be missed by the next warp-wide instruction of the others, which then waits without a limit."""
+    for body in _kernels(_code(path)):
+        if "__syncthreads_and" in body:
+            continue
+        for m in re.finditer(r"mbar_wait\(", body):
+            assert any("lane == 0" in head for head in _enclosing(body, m.start())), \
+                body[m.start() - 80:m.start() + 80]
