@@ -565,6 +565,103 @@ GT_HD void mn_rates_pair(const PairSpacetime &c, DF rp, DF s, DF cs, DF pr, DF p
     o.dpth = p_mul(s, p_fma(DF(0.5f, 0.0f), y_b, p_neg(p_mul(cs, s2_b))));
 }
 
+// ------------------------------------------------------------------ the step
+// Ray state of the double-float kernels: three floats per coordinate.
+struct RayTF {
+    TF t, r, th, ph, pr, pth, pt, pph;
+};
+
+// Largest |exponent| of a Manko-Novikov evaluation taken in double-float: |2 beta Ea|,
+// |2 beta Eb| <= 24 and |2 psi|, |2 psi - 2 gamma''| <= 48.  Beyond, products of the metric
+// functions overflow the float range (an infinite high part turns the low part into NaN, so
+// the rates come out non-finite) or, silently, low parts fall below the normal floats.
+constexpr float PAIR_MAX_EF = 24.0f;
+constexpr float PAIR_MAX_EPSI = 48.0f;
+
+struct PairExp {
+    const PairTables *tab;
+    GT_HD DF operator()(DF a) const { return p_exp(a, tab); }
+};
+
+GT_HD bool finite_rates(const Rates<DF> &o)
+{
+    return isfinite(o.dt.hi) && isfinite(o.dr.hi) && isfinite(o.dth.hi) && isfinite(o.dph.hi) &&
+           isfinite(o.dpr.hi) && isfinite(o.dpth.hi);
+}
+
+// One RK4 step of x in double-float: the stages of rk4_step64 (stage points x + h/2 k1,
+// x + h/2 k2, x + h k3; weights 1, 2, 2, 1 times h w6; h = |sp / k1.dt|) in a rolled loop, so
+// one copy of the field is compiled.  Returns false, x untouched, where an evaluation leaves
+// the double-float range (exponents, the axis, |theta| beyond the table reduction, a rate
+// that is not finite): the caller repeats the step in FP64.
+template <int KIND>
+GT_HD bool pair_step(const PairSpacetime &c, const PairTables *tab, RayTF &x, TF sp, TF w6,
+                     DF &h_out)
+{
+    const DF rp0 = tf_diff(x.r, c.r_plus);
+    DF rp = rp0, pr = tf_pair(x.pr), pth = tf_pair(x.pth), s1, c1;
+    p_sincos(tf_pair(x.th), x.th.c, tab, &s1, &c1);
+    DF s = s1, cs = c1;
+    Rates<DF> k, acc;
+    DF h(0.0f, 0.0f);
+    bool ok = fabsf(x.th.a) <= 128.0f && fabsf(s1.hi) >= 1e-6f;
+#pragma unroll 1
+    for (int stage = 0; stage < 4; stage++) {
+        if (KIND == KIND_MN || (KIND != KIND_KERR && c.kind == KIND_MN)) {
+            float ex[4];
+            mn_rates_pair(c, rp, s, cs, pr, pth, x.pt, x.pph, PairExp{tab}, k, ex);
+            ok = ok && fmaxf(fabsf(ex[0]), fabsf(ex[1])) <= PAIR_MAX_EF &&
+                 fmaxf(fabsf(ex[2]), fabsf(ex[3])) <= PAIR_MAX_EPSI;
+        } else {
+            kerr_rates_pair(c, rp, s, cs, pr, pth, x.pt, x.pph, k);
+        }
+        if (stage == 0) {
+            h = p_norm(p_mul3(p_rcp(k.dt), sp));
+            if (h.hi < 0.0f) h = p_neg(h);
+            acc = k;
+        } else {
+            const float w = stage < 3 ? 2.0f : 1.0f;
+            acc.dt = p_add(acc.dt, p_scale(k.dt, w));
+            acc.dr = p_add(acc.dr, p_scale(k.dr, w));
+            acc.dth = p_add(acc.dth, p_scale(k.dth, w));
+            acc.dph = p_add(acc.dph, p_scale(k.dph, w));
+            acc.dpr = p_add(acc.dpr, p_scale(k.dpr, w));
+            acc.dpth = p_add(acc.dpth, p_scale(k.dpth, w));
+        }
+        if (stage < 3) {
+            const DF d = p_scale(h, stage < 2 ? 0.5f : 1.0f);
+            rp = p_norm(p_fma(d, k.dr, rp0));
+            pr = p_fma(d, k.dpr, tf_pair(x.pr));
+            pth = p_fma(d, k.dpth, tf_pair(x.pth));
+            const DF dth = p_norm(p_mul(d, k.dth));
+            if (fabsf(dth.hi) <= 0.001953125f) {
+                p_rotate(s1, c1, dth, &s, &cs);
+            } else { // a step of a radian's order
+                const DF th = p_norm(p_add(tf_pair(x.th), dth));
+                ok = ok && fabsf(th.hi) <= 128.0f;
+                p_sincos(th, x.th.c, tab, &s, &cs);
+            }
+            ok = ok && fabsf(s.hi) >= 1e-6f;
+        }
+    }
+    // the sums of the stages are finite only if every rate was
+    if (!ok || !finite_rates(acc) || !isfinite(h.hi)) return false;
+    const DF hw = p_norm(p_mul3(h, w6));
+    x.t = tf_add(x.t, p_norm(p_mul(hw, acc.dt)));
+    x.r = tf_add(x.r, p_norm(p_mul(hw, acc.dr)));
+    x.th = tf_add(x.th, p_norm(p_mul(hw, acc.dth)));
+    x.ph = tf_add(x.ph, p_norm(p_mul(hw, acc.dph)));
+    x.pr = tf_add(x.pr, p_norm(p_mul(hw, acc.dpr)));
+    x.pth = tf_add(x.pth, p_norm(p_mul(hw, acc.dpth)));
+    h_out = h;
+    return true;
+}
+
+GT_HD bool tf_greater(TF x, TF y)
+{
+    return x.a > y.a || (x.a == y.a && (x.b > y.b || (x.b == y.b && x.c > y.c)));
+}
+
 #undef GT_P_ADD
 #undef GT_P_MUL
 
