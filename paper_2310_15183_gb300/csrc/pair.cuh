@@ -583,17 +583,11 @@ struct PairExp {
     GT_HD DF operator()(DF a) const { return p_exp(a, tab); }
 };
 
-GT_HD bool finite_rates(const Rates<DF> &o)
-{
-    return isfinite(o.dt.hi) && isfinite(o.dr.hi) && isfinite(o.dth.hi) && isfinite(o.dph.hi) &&
-           isfinite(o.dpr.hi) && isfinite(o.dpth.hi);
-}
-
 // One RK4 step of x in double-float: the stages of rk4_step64 (stage points x + h/2 k1,
 // x + h/2 k2, x + h k3; weights 1, 2, 2, 1 times h w6; h = |sp / k1.dt|) in a rolled loop, so
 // one copy of the field is compiled.  Returns false, x untouched, where an evaluation leaves
-// the double-float range (exponents, the axis, |theta| beyond the table reduction, a rate
-// that is not finite): the caller repeats the step in FP64.
+// the double-float range (exponents, the axis, |theta| beyond the table reduction, a rate or a
+// new coordinate that is not finite): the caller repeats the step in FP64.
 template <int KIND>
 GT_HD bool pair_step(const PairSpacetime &c, const PairTables *tab, RayTF &x, TF sp, TF w6,
                      DF &h_out)
@@ -644,15 +638,22 @@ GT_HD bool pair_step(const PairSpacetime &c, const PairTables *tab, RayTF &x, TF
             ok = ok && fabsf(s.hi) >= 1e-6f;
         }
     }
-    // the sums of the stages are finite only if every rate was
-    if (!ok || !finite_rates(acc) || !isfinite(h.hi)) return false;
     const DF hw = p_norm(p_mul3(h, w6));
-    x.t = tf_add(x.t, p_norm(p_mul(hw, acc.dt)));
-    x.r = tf_add(x.r, p_norm(p_mul(hw, acc.dr)));
-    x.th = tf_add(x.th, p_norm(p_mul(hw, acc.dth)));
-    x.ph = tf_add(x.ph, p_norm(p_mul(hw, acc.dph)));
-    x.pr = tf_add(x.pr, p_norm(p_mul(hw, acc.dpr)));
-    x.pth = tf_add(x.pth, p_norm(p_mul(hw, acc.dpth)));
+    const DF dt = p_norm(p_mul(hw, acc.dt)), dr = p_norm(p_mul(hw, acc.dr));
+    const DF dth = p_norm(p_mul(hw, acc.dth)), dph = p_norm(p_mul(hw, acc.dph));
+    const DF dpr = p_norm(p_mul(hw, acc.dpr)), dpth = p_norm(p_mul(hw, acc.dpth));
+    // one test of the new state: an increment is finite only if h and every stage's rate were,
+    // and a bound on the sum of all magnitudes holds for each new coordinate
+    const float m = ((fabsf(x.t.a) + fabsf(dt.hi)) + (fabsf(x.r.a) + fabsf(dr.hi))) +
+                    ((fabsf(x.th.a) + fabsf(dth.hi)) + (fabsf(x.ph.a) + fabsf(dph.hi))) +
+                    ((fabsf(x.pr.a) + fabsf(dpr.hi)) + (fabsf(x.pth.a) + fabsf(dpth.hi)));
+    if (!ok || !(m <= 1e38f)) return false;
+    x.t = tf_add(x.t, dt);
+    x.r = tf_add(x.r, dr);
+    x.th = tf_add(x.th, dth);
+    x.ph = tf_add(x.ph, dph);
+    x.pr = tf_add(x.pr, dpr);
+    x.pth = tf_add(x.pth, dpth);
     h_out = h;
     return true;
 }
