@@ -59,10 +59,16 @@ extern "C" {
 #define GT_RAY_DISK 5 /* entered the ring volume (gt_trace_disk) */
 
 /* arithmetic modes */
-#define GT_MODE_FP64 0       /* FP64 accuracy: FP64 end to end, or, for camera rays in ordinary
-                              * units (M in [1e-3, 1e3], r0 <= 1e5, step in [1e-9, 1]) with exact
+#define GT_MODE_FP64 0       /* FP64 accuracy: FP64 end to end, or, for camera rays with exact
                               * derivatives, double-float steps on a state of three floats per
-                              * coordinate whose end states are as close to the exact flow */
+                              * coordinate, where their end states are as close to the exact
+                              * flow: M in [1e-3, 1e3], r0 <= 1e5, step >= 1e-9; n_steps >= 1000
+                              * steps of at most 2e-3 M that make at least 0.15 M together, and
+                              * r0 <= 1000 M and 0.03 M n_steps.  Their steps that start within
+                              * 1000 step lengths of the axis, or below r = 4M in
+                              * Manko-Novikov, are FP64's.  Rings, states and per-ray
+                              * spacetimes take FP64 throughout: the same ray by gt_trace and
+                              * by one of those agrees to rounding, not to the bit. */
 #define GT_MODE_FP32_MIXED 1 /* FP32 RK4 with compensated state; a zone r < r_switch stepped with
                               * an FP64 state (its field and stage arithmetic in double-float
                               * where the evaluation's range allows, else FP64) and H = 0

@@ -147,6 +147,16 @@ int kind_for(int flags, int kind)
     return (flags & GT_FLAG_FD_DERIVS) ? (int)gt::KIND_FD : kind;
 }
 
+// What the cameras of a launch allow, all of them (internal.cuh).
+struct Routes {
+    bool range = false, pair = false;
+};
+
+Routes routes_of(double M, double r0, double sp, int64_t n_steps)
+{
+    return {gt::pair_range(M, r0), gt::pair_camera(M, r0, sp, n_steps)};
+}
+
 // Ring, redshift output and state arrays of a launch (all optional).
 struct Extra {
     gt::DiskArgs disk = {};
@@ -380,7 +390,7 @@ int run_trace(gt_ctx *c, const CamDesc *d_cams, int n_cams, int kind_hint, int64
               int64_t n_rays, int64_t n_steps, double sp, int mode, double *t, double *r,
               double *th, double *ph, uint8_t *status, uint32_t *nsteps,
               const int64_t *fresh_ids = nullptr, const gt::RayParams *d_rays = nullptr,
-              bool compact_out = false, const Extra &x = Extra(), bool range_ok = false,
+              bool compact_out = false, const Extra &x = Extra(), const Routes &routes = Routes(),
               const CamDesc *one = nullptr)
 {
     const gt_options e = effective(c->opts);
@@ -416,7 +426,8 @@ int run_trace(gt_ctx *c, const CamDesc *d_cams, int n_cams, int kind_hint, int64
     a.disk = x.disk;
     a.z = x.z;
     a.states = x.states;
-    a.range_ok = range_ok ? 1 : 0;
+    a.range_ok = routes.range ? 1 : 0;
+    a.pair_ok = routes.pair ? 1 : 0;
     if (one) {
         a.pair = one->pair;
         a.stf = gt::to_float(one->st);
@@ -663,7 +674,7 @@ int gt_trace_range(gt_ctx *c, int64_t first, int64_t count, int64_t n_steps, dou
         return GT_ERR_INVALID_ARG;
     const int kind = (c->Q != 0.0) ? gt::KIND_MN : gt::KIND_KERR;
     return run_trace(c, c->d_cam, 1, kind, first, count, n_steps, sp, mode, t, r, th, ph, status,
-                     nsteps, nullptr, nullptr, false, Extra(), gt::pair_range(c->M, c->r0),
+                     nsteps, nullptr, nullptr, false, Extra(), routes_of(c->M, c->r0, sp, n_steps),
                      &c->cam);
 }
 
@@ -684,7 +695,7 @@ int gt_trace_pixels(gt_ctx *c, const int64_t *pixels, int64_t n, int64_t n_steps
     if (!c->cam_valid) return GT_ERR_INVALID_ARG;
     const int kind = (c->Q != 0.0) ? gt::KIND_MN : gt::KIND_KERR;
     return run_trace(c, c->d_cam, 1, kind, 0, n, n_steps, sp, mode, t, r, th, ph, status, nsteps,
-                     pixels, nullptr, true, Extra(), gt::pair_range(c->M, c->r0),
+                     pixels, nullptr, true, Extra(), routes_of(c->M, c->r0, sp, n_steps),
                      &c->cam);
 }
 
@@ -714,7 +725,7 @@ int gt_trace_disk(gt_ctx *c, double r_in, double r_out, double half_thickness, i
     const int kind = (c->Q != 0.0) ? gt::KIND_MN : gt::KIND_KERR;
     return run_trace(c, c->d_cam, 1, kind, 0, (int64_t)c->res_x * c->res_y, n_steps, sp, mode, t,
                      r, th, ph, status, nsteps, nullptr, nullptr, false, x,
-                     gt::pair_range(c->M, c->r0), &c->cam);
+                     routes_of(c->M, c->r0, sp, n_steps), &c->cam);
 }
 
 int gt_trace_states(gt_ctx *c, int64_t n, double *t, double *r, double *th, double *ph,
@@ -807,10 +818,12 @@ int gt_trace_batch(gt_ctx *c, const gt_camera_desc *cams, int n_cams, int64_t n_
         return GT_ERR_INVALID_ARG;
     std::vector<CamDesc> h(n_cams);
     int64_t off = 0;
-    bool any_mn = false, any_kerr = false, range_ok = true;
+    bool any_mn = false, any_kerr = false;
+    Routes routes = {true, true};
     for (int i = 0; i < n_cams; i++) {
         const gt_camera_desc &d = cams[i];
-        range_ok = range_ok && gt::pair_range(d.M, d.r0);
+        const Routes rt = routes_of(d.M, d.r0, sp, n_steps);
+        routes = {routes.range && rt.range, routes.pair && rt.pair};
         if (!valid_spacetime(d.M, d.S, d.Q) ||
             !valid_camera(d.r0, d.theta0, d.fov_deg, d.res_x, d.res_y))
             return GT_ERR_INVALID_ARG;
@@ -847,7 +860,7 @@ int gt_trace_batch(gt_ctx *c, const gt_camera_desc *cams, int n_cams, int64_t n_
         if (!h[i].valid) return GT_ERR_INVALID_ARG;
     const int kind = any_mn && any_kerr ? 2 : (any_mn ? gt::KIND_MN : gt::KIND_KERR);
     return run_trace(c, c->d_batch, n_cams, kind, 0, off, n_steps, sp, mode, t, r, th, ph, status,
-                     nsteps, nullptr, nullptr, false, Extra(), range_ok,
+                     nsteps, nullptr, nullptr, false, Extra(), routes,
                      n_cams == 1 ? &h[0] : nullptr);
 }
 
@@ -883,7 +896,7 @@ int gt_trace_rays(gt_ctx *c, int64_t n, const double *alpha, const double *beta,
     if (err != cudaSuccess) return cuda_code(err);
     // the kernel reads descriptor 0 before the per-ray set-up replaces it
     return run_trace(c, c->d_cam, 1, 2, 0, n, n_steps, sp, mode, t, r, th, ph, status, nsteps,
-                     nullptr, c->d_rays, false, Extra(), gt::pair_range(M, r0));
+                     nullptr, c->d_rays, false, Extra(), routes_of(M, r0, sp, n_steps));
 }
 
 int gt_surrogate_infer(gt_ctx *c, gt_surrogate *s, const gt_gate_cfg *gate, int64_t n_steps,
@@ -961,7 +974,7 @@ int gt_surrogate_infer(gt_ctx *c, gt_surrogate *s, const gt_gate_cfg *gate, int6
     if (rc == GT_OK) rc = list_count(&n1);
     if (rc == GT_OK && n1 > 0)
         rc = run_trace(c, c->d_cam, 1, kind, 0, n1, n_steps, sp, mode, t, r, th, ph, status,
-                       nsteps, list, nullptr, false, Extra(), gt::pair_range(c->M, c->r0),
+                       nsteps, list, nullptr, false, Extra(), routes_of(c->M, c->r0, sp, n_steps),
                      &c->cam);
     if (rc != GT_OK) return rc;
     // 3. probe records from the traced probes
@@ -979,7 +992,7 @@ int gt_surrogate_infer(gt_ctx *c, gt_surrogate *s, const gt_gate_cfg *gate, int6
     if (rc == GT_OK) rc = list_count(&n2);
     if (rc == GT_OK && n2 > 0)
         rc = run_trace(c, c->d_cam, 1, kind, 0, n2, n_steps, sp, mode, t, r, th, ph, status,
-                       nsteps, list, nullptr, false, Extra(), gt::pair_range(c->M, c->r0),
+                       nsteps, list, nullptr, false, Extra(), routes_of(c->M, c->r0, sp, n_steps),
                      &c->cam);
     if (rc != GT_OK) return rc;
     if (n_fallback) *n_fallback = n1 - np + n2;

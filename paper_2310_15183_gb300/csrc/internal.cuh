@@ -136,6 +136,7 @@ struct TraceArgs {
     SpacetimeF stf;
     int single;
     int range_ok; // pair_range() of every camera of the launch
+    int pair_ok;  // pair_camera() of every camera of the launch
 };
 
 // Host-side validation shared by every entry point that takes a spacetime or a camera
@@ -174,16 +175,22 @@ inline void fill_desc(CamDesc &d, double M, double S, double Q, double r0, doubl
     d.offset = offset;
 }
 
-// Kernel mode of a GT_MODE_FP64 launch: the double-float step for camera rays with exact
-// derivatives under RK4, whose scales stay well inside the float range; FP64 arithmetic for
-// the listing's numerics, the ring, caller states, per-ray spacetimes (a set-up per ray) and
-// other scales.
+// Scales that stay well inside the float range.
 inline bool pair_range(double M, double r0) { return M >= 1e-3 && M <= 1e3 && r0 <= 1e5; }
 
+// The double-float step for a camera's GT_MODE_FP64 rays: its end states are as close as FP64's.
+inline bool pair_camera(double M, double r0, double sp, int64_t n_steps)
+{
+    return pair_range(M, r0) && sp >= 1e-9 && pair_accurate(M, r0, sp, n_steps);
+}
+
+// Kernel mode of a GT_MODE_FP64 launch: the double-float step for camera rays with exact
+// derivatives under RK4 (pair_camera); FP64 arithmetic for the listing's numerics, the ring,
+// caller states, per-ray spacetimes (a set-up per ray) and other cameras and steps.
 inline int fp64_kmode(const TraceArgs &a, int kind_hint)
 {
-    return a.range_ok && a.sp >= 1e-9 && a.sp <= 1.0 && kind_hint != KIND_FD && !a.euler &&
-                   !a.f32_io && !a.disk.on && !a.states.t && !a.rays
+    return a.pair_ok && kind_hint != KIND_FD && !a.euler && !a.f32_io && !a.disk.on &&
+                   !a.states.t && !a.rays
                ? KMODE_FP64_PAIR
                : KMODE_FP64;
 }

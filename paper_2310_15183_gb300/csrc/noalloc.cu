@@ -72,10 +72,11 @@ extern "C" int gt_trace_batch_noalloc(int device, void *cuda_stream, const gt_ca
 
     gt::CamDesc h[GT_NOALLOC_MAX_CAMS]; // host staging on the stack, not the heap
     int64_t total = 0;
-    bool any_mn = false, any_kerr = false, range_ok = true;
+    bool any_mn = false, any_kerr = false, range_ok = true, pair_ok = true;
     for (int i = 0; i < n_cams; i++) {
         const gt_camera_desc &d = cams[i];
         range_ok = range_ok && gt::pair_range(d.M, d.r0);
+        pair_ok = pair_ok && gt::pair_camera(d.M, d.r0, step_precision, n_steps);
         if (!gt::valid_spacetime(d.M, d.S, d.Q) ||
             !gt::valid_camera(d.r0, d.theta0, d.fov_deg, d.res_x, d.res_y))
             return GT_ERR_INVALID_ARG;
@@ -143,6 +144,7 @@ extern "C" int gt_trace_batch_noalloc(int device, void *cuda_stream, const gt_ca
     a.nsteps = nsteps;
     a.scratch = words;
     a.range_ok = range_ok ? 1 : 0;
+    a.pair_ok = pair_ok ? 1 : 0;
     a.zone_df = 1; // the context's default zone (double-float Manko-Novikov field)
     if (n_cams == 1) {
         a.pair = h[0].pair;

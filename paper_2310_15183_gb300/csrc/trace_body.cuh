@@ -909,9 +909,11 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A, int one_shot)
             const PairSpacetime &pc = SINGLE ? A.pair : rays ? pr_ray : cams[cam].pair;
             const bool hard = MODE == 5 && KIND != KIND_KERR &&
                               T.r.a - pc.r_plus.a < pc.r_hard;
+            // the zone's precision is the mixed mode's: steps up to the axis itself
+            const float rho_min = MODE == 5 ? PAIR_RHO_STEPS * A.sp_tf.a : 0.0f;
             DF h;
             ++n;
-            if (!hard && pair_step<KIND>(pc, tab, T, A.sp_tf, A.w6_tf, h)) {
+            if (!hard && pair_step<KIND>(pc, tab, T, A.sp_tf, A.w6_tf, rho_min, h)) {
                 if (tf_greater(T.r, r_esc_t))
                     status = GT_RAY_ESCAPED;
                 else if (h.hi < A.h_thr_df.hi || (h.hi == A.h_thr_df.hi && h.lo < A.h_thr_df.lo))
@@ -980,7 +982,7 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A, int one_shot)
                 mixed_to64(m, x);
                 tf_state(x, T);
                 if (A.zone_df && pair_step<KIND>(rays ? pr_ray : cams[cam].pair, tab, T, A.sp_tf,
-                                                 A.w6_tf, hd)) {
+                                                 A.w6_tf, 0.0f, hd)) {
                     h = df_to(hd);
                     tf_unstate(T, x);
                     mixed_from64(x, m);

@@ -206,8 +206,8 @@ static void new_state()
             const RayTF z0 = z;
             DF h;
             auto step = [&](double w) {
-                return Q == 0 ? pair_step<KIND_KERR>(k.p, &TAB, z, tf_from(1.0), tf_from(w), h)
-                              : pair_step<KIND_MN>(k.p, &TAB, z, tf_from(1.0), tf_from(w), h);
+                return Q == 0 ? pair_step<KIND_KERR>(k.p, &TAB, z, tf_from(1.0), tf_from(w), 0.0f, h)
+                              : pair_step<KIND_MN>(k.p, &TAB, z, tf_from(1.0), tf_from(w), 0.0f, h);
             };
             refused += !step(1e38);
             untouched += memcmp(&z, &z0, sizeof z) == 0;
@@ -217,9 +217,85 @@ static void new_state()
     printf("{\"n\": %d, \"refused\": %d, \"untouched\": %d, \"taken\": %d}\n", n, refused, untouched, taken);
 }
 
+// Kernel's choice for a GT_MODE_FP64 camera ray: the pair step where pair_accurate, above 4M in
+// Manko-Novikov and away from the axis, FP64 elsewhere.
+static void route_step(const Constants &k, State<double> &x, RayTF &z, double sp)
+{
+    DF h;
+    const TF t = tf_from(sp), w = tf_from(1.0 / 6.0);
+    const float rho = PAIR_RHO_STEPS * t.a;
+    const bool mn = k.c.kind == KIND_MN;
+    if (!(mn && z.r.a < (float)(4 * k.c.M)) &&
+        (mn ? pair_step<KIND_MN>(k.p, &TAB, z, t, w, rho, h) : pair_step<KIND_KERR>(k.p, &TAB, z, t, w, rho, h)))
+        return;
+    x.t = tf_to(z.t);
+    x.r = tf_to(z.r);
+    x.th = tf_to(z.th);
+    x.ph = tf_to(z.ph);
+    x.pr = tf_to(z.pr);
+    x.pth = tf_to(z.pth);
+    rk4<double>(k.c, x, sp);
+    z = ray(x);
+}
+
+// End positions of `frames` seeded camera frames of both kinds against long double: the 2-norm
+// error over a frame's 20 rays relative to the truth's, root mean square over the frames, of t,
+// r, theta, phi, for the kernel's choice and for FP64; the geometric mean over the frames of the
+// ratio of the two; and how many frames took pairs.
+static void accuracy(int argc, char **argv)
+{
+    if (argc < 9) return;
+    const long n = atol(argv[2]);
+    const double spM = atof(argv[3]), lo = atof(argv[4]), hi = atof(argv[5]);
+    const double th_lo = atof(argv[6]), th_hi = atof(argv[7]);
+    const int frames = atoi(argv[8]);
+    const double M = 0.5, sp = spM * M;
+    double rms[2][4] = {}, lg[4] = {};
+    int pairs = 0;
+    for (int f = 0; f < frames; f++) {
+        const bool mn = f % 2;
+        const double spin = mn ? uni(0.1, 0.98) : (f % 4 ? 0.999 : 0.2) * uni(0, 1);
+        const Constants k = constants(M, spin * M * M, mn ? (f % 4 == 1 ? 2.0 : -2.0) : 0.0);
+        const double r0 = M * exp(uni(log(lo), log(hi))), th0 = exp(uni(log(th_lo), log(th_hi)));
+        const double V = tan(uni(10, 60) * M_PI / 180) / r0;
+        const bool pair = pair_accurate(M, r0, sp, n);
+        pairs += pair;
+        LD nn[4] = {}, e[2][4] = {};
+        for (int id = 0; id < 20; id++) {
+            State<double> x = camera_ray(k, r0, th0, V * (2.0 * (id % 5) - 4) / 4, V * (2.0 * (id / 5) - 3) / 3);
+            State<LD> y = {x.t, x.r, x.th, x.ph, x.pr, x.pth, x.pt, x.pph};
+            State<double> w = x;
+            RayTF z = ray(x);
+            long i = 0;
+            for (; i < n && y.r <= 1.5 * r0 && y.r > 1.02 * k.c.r_plus; i++) {
+                rk4<double>(k.c, x, sp);
+                rk4<LD>(k.l, y, (LD)sp);
+                if (pair) route_step(k, w, z, sp);
+            }
+            const LD v[4] = {y.t, y.r, y.th, y.ph};
+            const double d[4] = {x.t, x.r, x.th, x.ph};
+            const double q[4] = {tf_to(z.t), tf_to(z.r), tf_to(z.th), tf_to(z.ph)};
+            for (int j = 0; j < 4; j++) {
+                nn[j] += v[j] * v[j];
+                const LD a = (pair ? q[j] : d[j]) - v[j], b = d[j] - v[j];
+                e[0][j] += a * a;
+                e[1][j] += b * b;
+            }
+        }
+        for (int j = 0; j < 4; j++) {
+            for (int m = 0; m < 2; m++) rms[m][j] += (double)(e[m][j] / nn[j]) / frames;
+            lg[j] += 0.5 * log((double)(e[0][j] / e[1][j])) / frames;
+        }
+    }
+    printf("{\"pairs\": %d, \"route\": [%.3e, %.3e, %.3e, %.3e], \"f64\": [%.3e, %.3e, %.3e, %.3e], \"ratio\": [%.3f, %.3f, %.3f, %.3f]}\n", pairs,
+           sqrt(rms[0][0]), sqrt(rms[0][1]), sqrt(rms[0][2]), sqrt(rms[0][3]), sqrt(rms[1][0]),
+           sqrt(rms[1][1]), sqrt(rms[1][2]), sqrt(rms[1][3]), exp(lg[0]), exp(lg[1]), exp(lg[2]), exp(lg[3]));
+}
+
 int main(int argc, char **argv)
 {
     const char *part = argc > 1 ? argv[1] : "";
+    if (!strcmp(part, "accuracy")) accuracy(argc, argv);
     if (!strcmp(part, "new_state")) new_state();
     return 0;
 }

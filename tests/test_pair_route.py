@@ -1,14 +1,37 @@
 """The double-float step at the limits of what it accepts (csrc/pair.cuh): on the host the
 kernels' own step, on the GPU the routes that lead to it."""
+import concurrent.futures
 import json
+import math
 import os
 import subprocess
 
+import numpy as np
 import pytest
 
 from paper_2310_15183_gb300 import build
 
+from .parity import to_numpy
+
 HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+# steps, step / M, r0 / M from and to, theta0 from and to, frames, whether pairs are taken
+ACCURACY = {
+    "a few steps": (10, 3e-4, 15, 50, 0.3, 1.5, 24, False),
+    "hundreds of steps": (500, 3e-4, 15, 50, 0.3, 1.5, 24, False),
+    "fewest steps": (1000, 3e-4, 8.5, 30, 0.3, 1.5, 24, True),
+    "the workloads' step": (2000, 3e-4, 15, 60, 0.3, 1.5, 24, True),
+    "shortest path": (2000, 7.5e-5, 8.5, 60, 0.3, 1.5, 24, True),
+    "too short a path": (2000, 1e-6, 8.5, 60, 0.3, 1.5, 24, False),
+    "coarsest steps": (1000, 2e-3, 8.5, 30, 0.3, 1.5, 24, True),
+    "coarse steps": (100, 0.2, 10, 30, 0.3, 1.5, 24, False),
+    "coarse steps, long paths": (6000, 8e-3, 8.5, 25, 0.9, 1.5, 24, False),
+    "far camera": (6000, 3e-4, 60, 180, 0.3, 1.5, 12, True),
+    "too far a camera": (1000, 1e-4, 200, 2000, 0.3, 1.5, 24, False),
+    "near the axis": (2000, 3e-4, 8.5, 60, 1e-3, 0.3, 24, True),
+    "near the axis, coarsest": (1500, 2e-3, 5, 45, 1e-3, 0.3, 24, True),
+}
 
 
 @pytest.fixture(scope="module")
@@ -29,3 +52,96 @@ def test_a_step_whose_new_state_is_not_finite_is_refused(host):
     the FP64 step, also where every rate was finite and only the increments overflow."""
     r = host("new_state")
     assert r["n"] == 64 and r["refused"] == r["untouched"] == r["taken"] == r["n"], r
+
+
+WHOLE_PATHS = (22000, 2e-3, 8.5, 25, 0.9, 1.5, 12)
+
+
+@pytest.fixture(scope="module")
+def accuracy(host):
+    rows = {**{k: v[:-1] for k, v in ACCURACY.items()}, "whole paths": WHOLE_PATHS}
+    with concurrent.futures.ThreadPoolExecutor(os.cpu_count()) as ex:
+        jobs = {k: ex.submit(host, "accuracy", *v) for k, v in rows.items()}
+        return {k: j.result() for k, j in jobs.items()}
+
+
+@pytest.mark.parametrize("name", sorted(ACCURACY))
+def test_fp64_mode_is_as_accurate_as_fp64_arithmetic(accuracy, name):
+    """GT_MODE_FP64's end positions against long double, by the step the kernels would take
+    there, are no further off than FP64 steps', t, r, theta and phi each: both are random sums,
+    so a quarter is left for the sample, and a ulp of the outputs for their own rounding."""
+    r = accuracy[name]
+    assert r["pairs"] == (ACCURACY[name][-2] if ACCURACY[name][-1] else 0), r
+    for got, f64 in zip(r["route"], r["f64"]):
+        assert got <= 1.25 * f64 + 2.0 ** -53, r
+
+
+def test_fp64_mode_is_as_accurate_as_fp64_arithmetic_over_whole_paths(accuracy):
+    """To the escape or the horizon some rays pass the photon orbits, which amplify either
+    arithmetic's rounding a millionfold: the mean over frames is the geometric one, of the
+    ratio of the two errors."""
+    r = accuracy["whole paths"]
+    assert r["pairs"] == WHOLE_PATHS[-1] and max(r["ratio"]) <= 1.25, r
+
+
+# ------------------------------------------------------------------ on the GPU
+# M, S, Q, r0, theta0, nx, ny, steps, step: calls that take FP64 steps
+FP64_CALLS = {
+    "one step": (0.5, 0.2, 0.0, 10.0, 1.2, 9, 7, 1, 1.5e-4),
+    "999 steps": (0.5, 0.24, 2.0, 15.0, 1.2, 9, 7, 999, 1.5e-4),
+    "step above 2e-3 M": (0.5, 0.2, 0.0, 10.0, 1.2, 9, 7, 2000, 1.001e-3),
+    "coarse steps": (0.5, 0.24, 2.0, 10.0, 1.2, 9, 7, 200, 0.3),
+    "short path": (0.5, 0.2, 0.0, 10.0, 1.2, 9, 7, 1000, 7e-5),
+    "far camera": (0.5, 0.2, 0.0, 16.0, 1.2, 9, 7, 1000, 1.5e-4),
+    "large unit of length": (500.0, 1e5, 0.0, 10000.0, 1.2, 9, 7, 1000, 1.01),
+}
+
+
+@pytest.fixture(scope="module")
+def tracer():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    build.build()
+    from paper_2310_15183_gb300 import geotrace
+    t = geotrace.Tracer(0)
+    yield t
+    t.close()
+
+
+def _both(tracer, M, S, Q, r0, th0, nx, ny, steps, sp):
+    """gt_trace, and the FP64 kernel: gt_trace_disk with a ring that no ray meets."""
+    tracer.set_spacetime(M, S, Q)
+    tracer.set_camera(r0, th0, 75.0, nx, ny)
+    tracer.set_options()
+    return (to_numpy(tracer.trace(steps, sp, 0)),
+            to_numpy(tracer.trace_disk(1e12, 2e12, 1e-9, steps, sp, 0)))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("name", sorted(FP64_CALLS))
+def test_calls_outside_the_rule_take_fp64_steps(tracer, name):
+    got, ref = _both(tracer, *FP64_CALLS[name])
+    for k in ("t", "r", "th", "ph", "status", "nsteps"):
+        assert np.array_equal(got[k], ref[k]), k
+
+
+@pytest.mark.gpu
+def test_calls_at_the_edge_of_the_rule_take_pairs(tracer):
+    """1000 steps, of 2e-3 M: bits of their own, the end position within 1e-13 of FP64's."""
+    got, ref = _both(tracer, 0.5, 0.2, 0.0, 10.0, 1.2, 9, 7, 1000, 1e-3)
+    assert not np.array_equal(got["ph"], ref["ph"])
+    for k in ("t", "r", "th", "ph"):
+        assert np.max(np.abs(got[k] - ref[k])) <= 1e-13 * np.max(np.abs(ref[k])), k
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("Q", [0.0, 2.0])
+def test_steps_near_the_axis_are_fp64(tracer, Q):
+    """A camera on the axis whose rays stay within 1000 step lengths of it (rho <= 0.01 + 0.8 in
+    1000 steps of 1e-3): FP64's steps one for one, up to the rounding of two builds of one
+    formula, 1e-15 a step, times what the axis amplifies (1 / theta of the closest, 1e2)."""
+    got, ref = _both(tracer, 0.5, 0.2, Q, 10.0, 1e-3, 9, 7, 1000, 1e-3)
+    assert np.array_equal(got["status"], ref["status"])
+    for k in ("t", "r", "th"):
+        assert np.max(np.abs(got[k] - ref[k])) <= 1e-12 * np.max(np.abs(ref[k])), k
