@@ -186,8 +186,10 @@ int gt_trace_pixels(gt_ctx *ctx, const int64_t *pixels, int64_t n, int64_t n_ste
 int gt_trace_host(gt_ctx *ctx, int64_t n_steps, double step_precision, int mode, double *t,
                   double *r, double *theta, double *phi, uint8_t *status, uint32_t *nsteps);
 
-/* Trace n_cams cameras (host array of descriptors) in one persistent launch.  Outputs
- * are device arrays over the flattened id space (sum of res_x*res_y).  Errors as gt_trace. */
+/* Trace n_cams cameras (host array of descriptors) in one persistent launch -- two where
+ * some cameras take another kernel than the rest (GT_MODE_FP64's double-float steps, the
+ * FP32 steps' flush-to-zero build): a camera's results do not depend on which kernel the
+ * others take.  Outputs are device arrays over the flattened id space (sum of res_x*res_y).  Errors as gt_trace. */
 int gt_trace_batch(gt_ctx *ctx, const gt_camera_desc *cams, int n_cams, int64_t n_steps,
                    double step_precision, int mode, double *t, double *r, double *theta,
                    double *phi, uint8_t *status, uint32_t *nsteps);

@@ -124,11 +124,26 @@ bool use_two(const gt_options &e, const gt::TraceArgs &a, int kind_hint, bool on
            gt::two_rays_supported(a, gt::KMODE_MIXED_FP32, kind_hint);
 }
 
+// The queue from its start again, for the second launch of a split one.
+cudaError_t restart_queue(const gt::TraceArgs &a, cudaStream_t s)
+{
+    return cudaMemsetAsync(a.scratch + gt::SCR_NEXT_RAY, 0, sizeof(unsigned long long), s);
+}
+
 cudaError_t launch_fp32(const gt_options &e, const gt::TraceArgs &a, int kind_hint, int block,
                         int grid, bool one_shot, cudaStream_t s)
 {
     if (use_two(e, a, kind_hint, one_shot)) return gt::launch_trace_two(a, kind_hint, block, grid, s);
-    return gt::launch_trace(a, gt::KMODE_MIXED_FP32, kind_hint, block, grid, one_shot, s);
+    if (!a.pick_mask) return gt::launch_trace(a, gt::KMODE_MIXED_FP32, kind_hint, block, grid, one_shot, s);
+    gt::TraceArgs b = a;
+    b.ftz = 0;
+    b.pick = 0;
+    cudaError_t err = gt::launch_trace(b, gt::KMODE_MIXED_FP32, kind_hint, block, grid, one_shot, s);
+    if (err == cudaSuccess) err = restart_queue(a, s);
+    b.ftz = 1;
+    b.pick = a.pick_mask;
+    if (err != cudaSuccess) return err;
+    return gt::launch_trace(b, gt::KMODE_MIXED_FP32, kind_hint, block, grid, one_shot, s);
 }
 
 // The listing passes the spacetime parameters to its kernels as float32.
@@ -147,14 +162,9 @@ int kind_for(int flags, int kind)
     return (flags & GT_FLAG_FD_DERIVS) ? (int)gt::KIND_FD : kind;
 }
 
-// What the cameras of a launch allow, all of them (internal.cuh).
-struct Routes {
-    bool range = false, pair = false;
-};
-
-Routes routes_of(double M, double r0, double sp, int64_t n_steps)
+gt::Routes camera_routes(const gt_ctx *c, double sp, int64_t n_steps)
 {
-    return {gt::pair_range(M, r0), gt::pair_camera(M, r0, sp, n_steps)};
+    return gt::Routes(gt::routes_of(c->M, c->r0, sp, n_steps));
 }
 
 // Ring, redshift output and state arrays of a launch (all optional).
@@ -211,6 +221,25 @@ int launch_shape(gt_ctx *c, const gt_options &e, int kmode, int kind_hint, int64
     const int most = e.blocks_per_sm > 0 ? e.blocks_per_sm : chosen ? 4 : 16;
     const int64_t full = (int64_t)(most < fit ? most : fit) * c->sm_count;
     *grid = (int)(need < full ? need : full);
+    return GT_OK;
+}
+
+// The FP64 launch: the double-float kernel, the FP64 one, or both in turn over their cameras.
+int launch_fp64(gt_ctx *c, const gt_options &e, const gt::TraceArgs &a, int kind_hint, bool pair,
+                bool one_shot, cudaStream_t s)
+{
+    gt::TraceArgs b = a;
+    for (int second = 0; second < (a.pick_mask ? 2 : 1); second++) {
+        const bool p = a.pick_mask ? second != 0 : pair;
+        const int kmode = p ? gt::KMODE_FP64_PAIR : gt::KMODE_FP64;
+        b.pick = p ? a.pick_mask : 0;
+        int block, grid;
+        const int rc = launch_shape(c, e, kmode, kind_hint, a.n_rays, one_shot, &block, &grid);
+        if (rc != GT_OK) return rc;
+        cudaError_t err = second ? restart_queue(a, s) : cudaSuccess;
+        if (err == cudaSuccess) err = gt::launch_trace(b, kmode, kind_hint, block, grid, one_shot, s);
+        if (err != cudaSuccess) return cuda_code(err);
+    }
     return GT_OK;
 }
 
@@ -302,8 +331,10 @@ int build_mixed_graph(gt_ctx *c, const gt::TraceArgs &base, int kind_hint, const
         a.in_count = w + gt::SCR_TO64;
         a.out_items = listB;
         a.out_count = w + gt::SCR_TO32;
+        gt::TraceArgs z = a; // the zone takes every camera's rays
+        z.pick_mask = 0;
         if (e1 == cudaSuccess)
-            e1 = gt::launch_trace(a, zone, kind_hint, block64, grid64, false, cs);
+            e1 = gt::launch_trace(z, zone, kind_hint, block64, grid64, false, cs);
         if (e1 == cudaSuccess) e1 = cudaMemsetAsync(w + gt::SCR_NEXT_RAY, 0, W8, cs);
         if (e1 == cudaSuccess) e1 = cudaMemsetAsync(w + gt::SCR_TO64, 0, W8, cs);
         a.in_items = listB;
@@ -366,7 +397,9 @@ int run_mixed_rounds(gt_ctx *c, gt::TraceArgs &a, int kind_hint, const gt_option
         const int zone = a.zone_df ? gt::KMODE_ZONE_PAIR : gt::KMODE_ZONE_FP64;
         rc = launch_shape(c, e, zone, kind_hint, (int64_t)parked, one_shot, &block, &grid);
         if (rc != GT_OK) return rc;
-        err = gt::launch_trace(a, zone, kind_hint, block, grid, one_shot, c->stream);
+        gt::TraceArgs z = a; // the zone takes every camera's rays
+        z.pick_mask = 0;
+        err = gt::launch_trace(z, zone, kind_hint, block, grid, one_shot, c->stream);
         if (err != cudaSuccess) return cuda_code(err);
         // FP32 continuation: B -> (A, finished)
         a.in_items = listB;
@@ -390,8 +423,8 @@ int run_trace(gt_ctx *c, const CamDesc *d_cams, int n_cams, int kind_hint, int64
               int64_t n_rays, int64_t n_steps, double sp, int mode, double *t, double *r,
               double *th, double *ph, uint8_t *status, uint32_t *nsteps,
               const int64_t *fresh_ids = nullptr, const gt::RayParams *d_rays = nullptr,
-              bool compact_out = false, const Extra &x = Extra(), const Routes &routes = Routes(),
-              const CamDesc *one = nullptr)
+              bool compact_out = false, const Extra &x = Extra(),
+              const gt::Routes &routes = gt::Routes(), const CamDesc *one = nullptr)
 {
     const gt_options e = effective(c->opts);
     if ((e.flags & PAPER_FLAGS) && mode != GT_MODE_FP64) return GT_ERR_INVALID_ARG;
@@ -426,24 +459,29 @@ int run_trace(gt_ctx *c, const CamDesc *d_cams, int n_cams, int kind_hint, int64
     a.disk = x.disk;
     a.z = x.z;
     a.states = x.states;
-    a.range_ok = routes.range ? 1 : 0;
-    a.pair_ok = routes.pair ? 1 : 0;
     if (one) {
         a.pair = one->pair;
         a.stf = gt::to_float(one->st);
         a.single = 1;
     }
+    // the kernel that each camera's scales and the call's steps allow
+    const bool pair_call = mode == GT_MODE_FP64 && gt::pair_launch(a, kind_hint);
+    const bool pair = pair_call && (routes.all & gt::ROUTE_PAIR);
+    a.ftz = (routes.all & gt::ROUTE_FTZ) ? 1 : 0;
+    if (pair_call && routes.split(gt::ROUTE_PAIR)) a.pick_mask = gt::ROUTE_PAIR;
+    if (mode != GT_MODE_FP64 && routes.split(gt::ROUTE_FTZ)) a.pick_mask = gt::ROUTE_FTZ;
     cudaError_t err =
         cudaMemsetAsync(c->d_scratch, 0, gt::SCR_WORDS * sizeof(unsigned long long), c->stream);
     if (err != cudaSuccess) return cuda_code(err);
     const bool one_shot = (e.flags & GT_FLAG_ONE_SHOT) != 0;
-    const int kmode64 = gt::fp64_kmode(a, kind_hint);
     int rc;
     if (e.flags & GT_FLAG_GRAPH) {
         // the launch replayed from a CUDA graph, captured once per distinct launch and
         // cached: FP64 is one persistent launch; FP32-mixed is its rounds under a WHILE
         // node whose condition the device sets from the park count
-        const int kmode = mode == GT_MODE_FP64 ? kmode64 : gt::KMODE_MIXED_FP32;
+        const int kmode = mode != GT_MODE_FP64 ? gt::KMODE_MIXED_FP32
+                          : pair               ? gt::KMODE_FP64_PAIR
+                                               : gt::KMODE_FP64;
         if (one_shot) return GT_ERR_INVALID_ARG; // graphs replay the persistent launch
         int block, grid;
         rc = launch_shape(c, e, kmode, kind_hint, n_rays, one_shot, &block, &grid);
@@ -468,10 +506,9 @@ int run_trace(gt_ctx *c, const CamDesc *d_cams, int n_cams, int kind_hint, int64
                 cudaError_t e1 = cudaMemsetAsync(c->d_scratch, 0,
                                                  gt::SCR_WORDS * sizeof(unsigned long long),
                                                  c->cap_stream);
-                cudaError_t e2 = gt::launch_trace(a, kmode, kind_hint, block, grid, one_shot,
-                                                  c->cap_stream);
+                const int rc2 = launch_fp64(c, e, a, kind_hint, pair, one_shot, c->cap_stream);
                 err = cudaStreamEndCapture(c->cap_stream, &graph);
-                if (e1 != cudaSuccess || e2 != cudaSuccess || err != cudaSuccess) {
+                if (e1 != cudaSuccess || rc2 != GT_OK || err != cudaSuccess) {
                     if (graph) cudaGraphDestroy(graph);
                     return GT_ERR_CUDA;
                 }
@@ -497,11 +534,7 @@ int run_trace(gt_ctx *c, const CamDesc *d_cams, int n_cams, int kind_hint, int64
         }
         rc = cuda_code(cudaGraphLaunch(c->graph_exec, c->stream));
     } else if (mode == GT_MODE_FP64) {
-        int block, grid;
-        rc = launch_shape(c, e, kmode64, kind_hint, n_rays, one_shot, &block, &grid);
-        if (rc != GT_OK) return rc;
-        err = gt::launch_trace(a, kmode64, kind_hint, block, grid, one_shot, c->stream);
-        rc = cuda_code(err);
+        rc = launch_fp64(c, e, a, kind_hint, pair, one_shot, c->stream);
     } else {
         rc = run_mixed_rounds(c, a, kind_hint, e, one_shot);
     }
@@ -674,8 +707,7 @@ int gt_trace_range(gt_ctx *c, int64_t first, int64_t count, int64_t n_steps, dou
         return GT_ERR_INVALID_ARG;
     const int kind = (c->Q != 0.0) ? gt::KIND_MN : gt::KIND_KERR;
     return run_trace(c, c->d_cam, 1, kind, first, count, n_steps, sp, mode, t, r, th, ph, status,
-                     nsteps, nullptr, nullptr, false, Extra(), routes_of(c->M, c->r0, sp, n_steps),
-                     &c->cam);
+                     nsteps, nullptr, nullptr, false, Extra(), camera_routes(c, sp, n_steps), &c->cam);
 }
 
 int gt_trace_pixels(gt_ctx *c, const int64_t *pixels, int64_t n, int64_t n_steps, double sp,
@@ -695,8 +727,7 @@ int gt_trace_pixels(gt_ctx *c, const int64_t *pixels, int64_t n, int64_t n_steps
     if (!c->cam_valid) return GT_ERR_INVALID_ARG;
     const int kind = (c->Q != 0.0) ? gt::KIND_MN : gt::KIND_KERR;
     return run_trace(c, c->d_cam, 1, kind, 0, n, n_steps, sp, mode, t, r, th, ph, status, nsteps,
-                     pixels, nullptr, true, Extra(), routes_of(c->M, c->r0, sp, n_steps),
-                     &c->cam);
+                     pixels, nullptr, true, Extra(), camera_routes(c, sp, n_steps), &c->cam);
 }
 
 int gt_trace_disk(gt_ctx *c, double r_in, double r_out, double half_thickness, int64_t n_steps,
@@ -725,7 +756,7 @@ int gt_trace_disk(gt_ctx *c, double r_in, double r_out, double half_thickness, i
     const int kind = (c->Q != 0.0) ? gt::KIND_MN : gt::KIND_KERR;
     return run_trace(c, c->d_cam, 1, kind, 0, (int64_t)c->res_x * c->res_y, n_steps, sp, mode, t,
                      r, th, ph, status, nsteps, nullptr, nullptr, false, x,
-                     routes_of(c->M, c->r0, sp, n_steps), &c->cam);
+                     camera_routes(c, sp, n_steps), &c->cam);
 }
 
 int gt_trace_states(gt_ctx *c, int64_t n, double *t, double *r, double *th, double *ph,
@@ -819,15 +850,16 @@ int gt_trace_batch(gt_ctx *c, const gt_camera_desc *cams, int n_cams, int64_t n_
     std::vector<CamDesc> h(n_cams);
     int64_t off = 0;
     bool any_mn = false, any_kerr = false;
-    Routes routes = {true, true};
+    gt::Routes routes;
     for (int i = 0; i < n_cams; i++) {
         const gt_camera_desc &d = cams[i];
-        const Routes rt = routes_of(d.M, d.r0, sp, n_steps);
-        routes = {routes.range && rt.range, routes.pair && rt.pair};
         if (!valid_spacetime(d.M, d.S, d.Q) ||
             !valid_camera(d.r0, d.theta0, d.fov_deg, d.res_x, d.res_y))
             return GT_ERR_INVALID_ARG;
         fill_desc(h[i], d.M, d.S, d.Q, d.r0, d.theta0, d.fov_deg, d.res_x, d.res_y, off);
+        h[i].route = gt::routes_of(d.M, d.r0, sp, n_steps);
+        if (i == 0) routes = gt::Routes(h[i].route);
+        routes.add(h[i].route);
         if (c->opts.flags & GT_FLAG_F32_IO) round_params_f32(h[i]);
         off += (int64_t)d.res_x * d.res_y;
         if (d.Q != 0.0)
@@ -860,8 +892,7 @@ int gt_trace_batch(gt_ctx *c, const gt_camera_desc *cams, int n_cams, int64_t n_
         if (!h[i].valid) return GT_ERR_INVALID_ARG;
     const int kind = any_mn && any_kerr ? 2 : (any_mn ? gt::KIND_MN : gt::KIND_KERR);
     return run_trace(c, c->d_batch, n_cams, kind, 0, off, n_steps, sp, mode, t, r, th, ph, status,
-                     nsteps, nullptr, nullptr, false, Extra(), routes,
-                     n_cams == 1 ? &h[0] : nullptr);
+                     nsteps, nullptr, nullptr, false, Extra(), routes, n_cams == 1 ? &h[0] : nullptr);
 }
 
 int gt_trace_rays(gt_ctx *c, int64_t n, const double *alpha, const double *beta,
@@ -896,7 +927,8 @@ int gt_trace_rays(gt_ctx *c, int64_t n, const double *alpha, const double *beta,
     if (err != cudaSuccess) return cuda_code(err);
     // the kernel reads descriptor 0 before the per-ray set-up replaces it
     return run_trace(c, c->d_cam, 1, 2, 0, n, n_steps, sp, mode, t, r, th, ph, status, nsteps,
-                     nullptr, c->d_rays, false, Extra(), routes_of(M, r0, sp, n_steps));
+                     nullptr, c->d_rays, false, Extra(),
+                     gt::Routes(gt::routes_of(M, r0, sp, n_steps)));
 }
 
 int gt_surrogate_infer(gt_ctx *c, gt_surrogate *s, const gt_gate_cfg *gate, int64_t n_steps,
@@ -974,8 +1006,7 @@ int gt_surrogate_infer(gt_ctx *c, gt_surrogate *s, const gt_gate_cfg *gate, int6
     if (rc == GT_OK) rc = list_count(&n1);
     if (rc == GT_OK && n1 > 0)
         rc = run_trace(c, c->d_cam, 1, kind, 0, n1, n_steps, sp, mode, t, r, th, ph, status,
-                       nsteps, list, nullptr, false, Extra(), routes_of(c->M, c->r0, sp, n_steps),
-                     &c->cam);
+                       nsteps, list, nullptr, false, Extra(), camera_routes(c, sp, n_steps), &c->cam);
     if (rc != GT_OK) return rc;
     // 3. probe records from the traced probes
     if (pg.stride > 0) {
@@ -992,8 +1023,7 @@ int gt_surrogate_infer(gt_ctx *c, gt_surrogate *s, const gt_gate_cfg *gate, int6
     if (rc == GT_OK) rc = list_count(&n2);
     if (rc == GT_OK && n2 > 0)
         rc = run_trace(c, c->d_cam, 1, kind, 0, n2, n_steps, sp, mode, t, r, th, ph, status,
-                       nsteps, list, nullptr, false, Extra(), routes_of(c->M, c->r0, sp, n_steps),
-                     &c->cam);
+                       nsteps, list, nullptr, false, Extra(), camera_routes(c, sp, n_steps), &c->cam);
     if (rc != GT_OK) return rc;
     if (n_fallback) *n_fallback = n1 - np + n2;
     if (n_probes) *n_probes = np;

@@ -33,8 +33,12 @@ struct CamDesc {
     double r_switch;        // FP32-mixed: zone radius
     PairSpacetime pair;     // the spacetime constants of the double-float step
     int32_t valid;          // 1 when the camera sits where g_tt < 0
-    int32_t pad_;
+    int32_t route;          // ROUTE_* (set by the host for cameras of a batch)
 };
+
+// Kernels a camera's rays may take, by its scales and the call's steps (routes_of): the
+// double-float step in GT_MODE_FP64, the flush-to-zero build of the FP32 steps.
+enum : int { ROUTE_PAIR = 1, ROUTE_FTZ = 2 };
 
 // Scratch words of one launch (device memory owned by the context).
 enum : int {
@@ -54,7 +58,7 @@ enum : int {
     KMODE_MIXED_FP32 = 2,
     KMODE_ZONE_FP64 = 3,  // zone steps in FP64 (GT_FLAG_ZONE_FP64)
     KMODE_ZONE_PAIR = 4,  // zone steps in double-float (the default)
-    KMODE_FP64_PAIR = 5   // GT_MODE_FP64 with the double-float step (fp64_kmode)
+    KMODE_FP64_PAIR = 5   // GT_MODE_FP64 with the double-float step (ROUTE_PAIR)
 };
 
 // Kind of a launch: one spacetime kind for every camera (KIND_KERR, KIND_MN), per camera
@@ -135,8 +139,11 @@ struct TraceArgs {
     PairSpacetime pair;
     SpacetimeF stf;
     int single;
-    int range_ok; // pair_range() of every camera of the launch
-    int pair_ok;  // pair_camera() of every camera of the launch
+    int ftz; // FP32 steps: the flush-to-zero build
+    // with pick_mask only the rays of cameras whose (route & pick_mask) is pick: the cameras of a
+    // batch that take different kernels are traced in one launch each, every launch passing over
+    // the others' rays.  (In a launch's base arguments pick_mask says that it is split so.)
+    int pick_mask, pick;
 };
 
 // Host-side validation shared by every entry point that takes a spacetime or a camera
@@ -184,15 +191,31 @@ inline bool pair_camera(double M, double r0, double sp, int64_t n_steps)
     return pair_range(M, r0) && sp >= 1e-9 && pair_accurate(M, r0, sp, n_steps);
 }
 
-// Kernel mode of a GT_MODE_FP64 launch: the double-float step for camera rays with exact
-// derivatives under RK4 (pair_camera); FP64 arithmetic for the listing's numerics, the ring,
-// caller states, per-ray spacetimes (a set-up per ray) and other cameras and steps.
-inline int fp64_kmode(const TraceArgs &a, int kind_hint)
+// ROUTE_* of a camera.
+inline int routes_of(double M, double r0, double sp, int64_t n_steps)
 {
-    return a.pair_ok && kind_hint != KIND_FD && !a.euler && !a.f32_io && !a.disk.on &&
-                   !a.states.t && !a.rays
-               ? KMODE_FP64_PAIR
-               : KMODE_FP64;
+    return (pair_camera(M, r0, sp, n_steps) ? ROUTE_PAIR : 0) | (pair_range(M, r0) ? ROUTE_FTZ : 0);
+}
+
+// ROUTE_* that all cameras of a launch have, and that any has.
+struct Routes {
+    int all = 0, any = 0;
+    Routes() = default;
+    explicit Routes(int r) : all(r), any(r) {}
+    void add(int r)
+    {
+        all &= r;
+        any |= r;
+    }
+    bool split(int route) const { return (any & route) && !(all & route); }
+};
+
+// Whether a GT_MODE_FP64 launch may take the double-float step at all: camera rays with exact
+// derivatives under RK4; FP64 arithmetic for the listing's numerics, the ring, caller states and
+// per-ray spacetimes (a set-up per ray).
+inline bool pair_launch(const TraceArgs &a, int kind_hint)
+{
+    return kind_hint != KIND_FD && !a.euler && !a.f32_io && !a.disk.on && !a.states.t && !a.rays;
 }
 
 // Launchers (trace.cu).  Return a cudaError_t from the launch.
@@ -205,7 +228,7 @@ cudaError_t launch_set_condition(cudaGraphConditionalHandle h, const unsigned lo
 int max_blocks_per_sm(int kmode, int kind_hint, int block);
 cudaError_t launch_trace(const TraceArgs &a, int kmode, int kind_hint, int block, int grid,
                          bool one_shot, cudaStream_t s);
-// The FP32 rounds kernel (trace_fp32.cu), for launches with a.range_ok.
+// The FP32 rounds kernel (trace_fp32.cu), for launches with a.ftz.
 cudaError_t launch_trace_fp32(const TraceArgs &a, int kind_hint, int block, int grid, bool one_shot,
                               cudaStream_t s);
 int max_blocks_per_sm_fp32(int kind_hint, int block);

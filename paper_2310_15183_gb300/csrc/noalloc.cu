@@ -72,15 +72,17 @@ extern "C" int gt_trace_batch_noalloc(int device, void *cuda_stream, const gt_ca
 
     gt::CamDesc h[GT_NOALLOC_MAX_CAMS]; // host staging on the stack, not the heap
     int64_t total = 0;
-    bool any_mn = false, any_kerr = false, range_ok = true, pair_ok = true;
+    bool any_mn = false, any_kerr = false;
+    gt::Routes routes;
     for (int i = 0; i < n_cams; i++) {
         const gt_camera_desc &d = cams[i];
-        range_ok = range_ok && gt::pair_range(d.M, d.r0);
-        pair_ok = pair_ok && gt::pair_camera(d.M, d.r0, step_precision, n_steps);
         if (!gt::valid_spacetime(d.M, d.S, d.Q) ||
             !gt::valid_camera(d.r0, d.theta0, d.fov_deg, d.res_x, d.res_y))
             return GT_ERR_INVALID_ARG;
         gt::fill_desc(h[i], d.M, d.S, d.Q, d.r0, d.theta0, d.fov_deg, d.res_x, d.res_y, total);
+        h[i].route = gt::routes_of(d.M, d.r0, step_precision, n_steps);
+        if (i == 0) routes = gt::Routes(h[i].route);
+        routes.add(h[i].route);
         total += (int64_t)d.res_x * d.res_y;
         if (d.Q != 0.0)
             any_mn = true;
@@ -143,8 +145,6 @@ extern "C" int gt_trace_batch_noalloc(int device, void *cuda_stream, const gt_ca
     a.status = status;
     a.nsteps = nsteps;
     a.scratch = words;
-    a.range_ok = range_ok ? 1 : 0;
-    a.pair_ok = pair_ok ? 1 : 0;
     a.zone_df = 1; // the context's default zone (double-float Manko-Novikov field)
     if (n_cams == 1) {
         a.pair = h[0].pair;
@@ -153,12 +153,20 @@ extern "C" int gt_trace_batch_noalloc(int device, void *cuda_stream, const gt_ca
     }
     const int kind = any_mn && any_kerr ? 2 : (any_mn ? gt::KIND_MN : gt::KIND_KERR);
     const int block = 128;
-    const int kmode =
-        mode == GT_MODE_FP64 ? gt::fp64_kmode(a, kind) : gt::KMODE_MIXED_INLINE;
-    const int fit = gt::max_blocks_per_sm(kmode, kind, block);
-    const int grid = (fit < 4 ? fit : 4) * sms;
     // FP32-mixed runs its zone inline here: the park lists of the context path
     // would need allocated memory
-    e = gt::launch_trace(a, kmode, kind, block, grid, false, s);
+    const int kmodes[2] = {mode != GT_MODE_FP64                ? gt::KMODE_MIXED_INLINE
+                     : (routes.all & gt::ROUTE_PAIR) ? gt::KMODE_FP64_PAIR
+                                                     : gt::KMODE_FP64,
+                     gt::KMODE_FP64_PAIR};
+    const bool split = mode == GT_MODE_FP64 && routes.split(gt::ROUTE_PAIR);
+    if (split) a.pick_mask = gt::ROUTE_PAIR; // each camera's kernel in turn
+    for (int k = 0; k < (split ? 2 : 1) && e == cudaSuccess; k++) {
+        a.pick = k == 0 ? 0 : gt::ROUTE_PAIR;
+        const int fit = gt::max_blocks_per_sm(kmodes[k], kind, block);
+        const int grid = (fit < 4 ? fit : 4) * sms;
+        if (k > 0) e = cudaMemsetAsync(words, 0, WORDS_BYTES, s);
+        if (e == cudaSuccess) e = gt::launch_trace(a, kmodes[k], kind, block, grid, false, s);
+    }
     return e == cudaSuccess ? GT_OK : GT_ERR_CUDA;
 }

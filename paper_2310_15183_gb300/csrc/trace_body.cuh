@@ -740,7 +740,10 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A, int one_shot)
         return d.valid != 0;
     };
 
-    // Start work item `w`; returns false when the ray is already finished and stored.
+    auto picked = [&](int c) { return !A.pick_mask || (cams[c].route & A.pick_mask) == A.pick; };
+
+    // Start work item `w`; returns false when the ray is already finished and stored, or another
+    // launch's.
     auto start = [&](int64_t w) -> bool {
         if (w < A.n_fresh) { // a fresh ray: initial data from the camera
             const int64_t pix = A.fresh_ids ? A.fresh_ids[w] : w;
@@ -768,6 +771,7 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A, int one_shot)
                 }
             } else {
                 if (KIND >= KIND_ANY || A.n_cams > 1) load_camera(find_camera(cams, A.n_cams, pix));
+                if (!picked(cam)) return false;
                 camera_init(cams[cam], A.first + pix - cams[cam].offset, x);
                 if (A.f32_io) { // the listing's kernels take the initial state as float32
                     x.t = round_f32(x.t);
@@ -793,6 +797,7 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A, int one_shot)
                 load_rayparams(id, false);
             else if (KIND >= KIND_ANY || A.n_cams > 1)
                 load_camera(it.cam);
+            if (!picked(cam)) return false;
             x.t = it.t;
             x.r = it.r;
             x.th = it.th;
@@ -876,12 +881,14 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A, int one_shot)
                             } else if (w < A.n_fresh) {
                                 const int64_t pix = A.fresh_ids ? A.fresh_ids[w] : w;
                                 const int c = A.n_cams > 1 ? find_camera(cams, A.n_cams, pix) : 0;
+                                if (!picked(c)) continue;
                                 const double r0 = rays ? rays->r0 : cams[c].r0;
                                 const double th0 = rays ? rays->theta0[pix] : cams[c].th0;
                                 store_ray(A, (A.fresh_ids && A.compact_out) ? w : pix, 0.0, r0,
                                           th0, 0.0, GT_RAY_TIMEOUT, 0);
                             } else {
                                 const ParkItem &p = A.in_items[w - A.n_fresh];
+                                if (!picked(p.cam)) continue;
                                 Ray64 y;
                                 y.t = p.t;
                                 y.r = p.r;

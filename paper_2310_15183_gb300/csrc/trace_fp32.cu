@@ -187,7 +187,7 @@ static cudaError_t launch_two(const TraceArgs &a, int block, int grid, cudaStrea
 bool two_rays_supported(const TraceArgs &a, int kmode, int kind_hint)
 {
     return kmode == KMODE_MIXED_FP32 && (kind_hint == KIND_KERR || kind_hint == KIND_MN) &&
-           a.range_ok && a.n_cams == 1 && !a.rays && !a.states.t && !a.disk.on && a.timeout_ns == 0;
+           a.ftz && a.n_cams == 1 && !a.rays && !a.states.t && !a.disk.on && a.timeout_ns == 0;
 }
 
 cudaError_t launch_trace_two(const TraceArgs &args, int kind_hint, int block, int grid,

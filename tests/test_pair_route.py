@@ -145,3 +145,82 @@ def test_steps_near_the_axis_are_fp64(tracer, Q):
     assert np.array_equal(got["status"], ref["status"])
     for k in ("t", "r", "th"):
         assert np.max(np.abs(got[k] - ref[k])) <= 1e-12 * np.max(np.abs(ref[k])), k
+
+
+def _cameras():
+    from paper_2310_15183_gb300 import workloads as W
+    near = W.Camera(0.5, 0.2, 0.0, 10.0, 1.2, 75.0, 9, 7)
+    return {"distant": [near, W.Camera(0.5, 0.1, 0.0, 2e5, 1.2, 1.0, 5, 3), near],
+            "heavy first": [W.Camera(2e3, 1e6, 0.0, 6e4, 1.2, 75.0, 5, 3), near],
+            "both kinds": [near, W.Camera(0.5, 0.24, 2.0, 15.0, 1.3, 75.0, 7, 6),
+                           W.Camera(0.5, 0.24, 2.0, 2e5, 1.3, 1.0, 3, 3),
+                           W.Camera(0.5, 0.1, 0.0, 2e5, 1.2, 1.0, 5, 3)]}
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("mode,flags", [(0, 0), (0, 4), (0, 8), (1, 0), (1, 4), (1, 8)])
+@pytest.mark.parametrize("name", sorted(_cameras()))
+def test_a_cameras_bits_do_not_depend_on_its_batch_mates(tracer, name, mode, flags):
+    """Cameras of a batch that take different kernels -- one beyond the double-float and
+    flush-to-zero ranges among others inside -- give the bits of a batch of their own route,
+    through the direct launch, one ray per thread, and a graph replayed twice."""
+    cams = _cameras()[name]
+    steps, sp = 1500, 1e-3
+    inside = [c.M <= 1e3 and c.r0 <= 1e5 for c in cams]
+    tracer.set_options(flags=flags)
+    out = tracer.alloc_outputs(sum(c.n_rays for c in cams))
+    for _ in range(2):
+        for v in out.values():
+            v.fill_(77)
+        tracer.trace_batch(cams, steps, sp, mode, out)
+    got = to_numpy(out)
+    off = np.cumsum([0] + [c.n_rays for c in cams])
+    for part in (True, False):
+        mine = [i for i, v in enumerate(inside) if v == part]
+        # a camera of each kind in the group, so that it runs the same per-camera kernel
+        alone = to_numpy(tracer.trace_batch([cams[i] for i in mine], steps, sp, mode))
+        at = np.concatenate([np.arange(off[i], off[i + 1]) for i in mine])
+        for k in ("t", "r", "th", "ph", "status", "nsteps"):
+            assert np.array_equal(got[k][at], alone[k], equal_nan=k in ("t", "r", "th", "ph")), (part, k)
+    tracer.set_options()
+
+
+@pytest.mark.gpu
+def test_watchdog_reaches_every_ray_of_a_split_batch(tracer):
+    """A batch traced in two launches under a limit that runs out in the first: the timeout code,
+    every ray's status written once, the context usable."""
+    from paper_2310_15183_gb300 import geotrace as g
+    from paper_2310_15183_gb300 import workloads as W
+    cams = [W.Camera(0.5, 0.2, 0.0, 1e4, 1.2, 75.0, 64, 48),
+            W.Camera(0.5, 0.2, 0.0, 2e5, 1.2, 1.0, 64, 48)]
+    out = tracer.alloc_outputs(sum(c.n_rays for c in cams))
+    for mode in (0, 1):
+        out["status"].fill_(77)
+        tracer.set_options(timeout_seconds=0.2)
+        with pytest.raises(g.GeotraceError) as e:
+            tracer.trace_batch(cams, 1 << 31, 1e-5, mode, out)
+        assert e.value.code == -5
+        assert np.all(to_numpy(out)["status"] == g.TIMEOUT)
+    tracer.set_options()
+    assert np.all(to_numpy(tracer.trace_batch(cams, 100, 1e-3, 0))["nsteps"] == 100)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("name", sorted(_cameras()))
+def test_noalloc_takes_each_cameras_route(tracer, name):
+    """gt_trace_batch_noalloc in GT_MODE_FP64 gives gt_trace_batch's bits, split or not."""
+    import ctypes
+    torch = pytest.importorskip("torch")
+    from paper_2310_15183_gb300 import geotrace as g
+    cams = _cameras()[name]
+    descs = (g.CameraDesc * len(cams))(*[g.CameraDesc(c.M, c.S, c.Q, c.r0, c.theta0, c.fov_deg, c.res_x,
+                                                      c.res_y) for c in cams])
+    out = tracer.alloc_outputs(sum(c.n_rays for c in cams))
+    rc = g.load_library().gt_trace_batch_noalloc(
+        0, ctypes.c_void_p(torch.cuda.current_stream().cuda_stream), descs, len(cams), 1500, 1e-3, 0,
+        *[ctypes.c_void_p(out[k].data_ptr()) for k in ("t", "r", "th", "ph", "status", "nsteps")])
+    assert rc == 0
+    tracer.set_options()
+    got, want = to_numpy(out), to_numpy(tracer.trace_batch(cams, 1500, 1e-3, 0))
+    for k in got:
+        assert np.array_equal(got[k], want[k], equal_nan=k in ("t", "r", "th", "ph")), k
