@@ -191,10 +191,12 @@ inline bool pair_camera(double M, double r0, double sp, int64_t n_steps)
     return pair_range(M, r0) && sp >= 1e-9 && pair_accurate(M, r0, sp, n_steps);
 }
 
-// ROUTE_* of a camera.
+// ROUTE_* of a camera.  Flush-to-zero: scales as above, and a step whose increments stay normal
+// floats (below 4e-34 the horizon's step is a denormal, below 7e-38 the increments of t are).
 inline int routes_of(double M, double r0, double sp, int64_t n_steps)
 {
-    return (pair_camera(M, r0, sp, n_steps) ? ROUTE_PAIR : 0) | (pair_range(M, r0) ? ROUTE_FTZ : 0);
+    return (pair_camera(M, r0, sp, n_steps) ? ROUTE_PAIR : 0) |
+           (pair_range(M, r0) && sp >= 1e-9 ? ROUTE_FTZ : 0);
 }
 
 // ROUTE_* that all cameras of a launch have, and that any has.

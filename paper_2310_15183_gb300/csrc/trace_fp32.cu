@@ -3,9 +3,12 @@
 // With denormals a reciprocal, an exponential and an inverse square root each carry two to four
 // instructions of scaling around the hardware's approximation and an IEEE division its slow
 // path: 100 of a Manko-Novikov step's 1,261 instructions and a tenth of a lone Kerr warp's
-// step latency.  No denormal reaches a result for spacetimes and cameras of ordinary scale
-// (pair_range: every intermediate stays above 1e-31 away from the axis itself), where both
-// compilations give the same bits; other scales run trace.cu's kernel.  One GB300: 500x400
+// step latency.  In spacetimes and cameras of ordinary scale (pair_range, steps of 1e-9 and
+// more) the two compilations give the same bits: Manko-Novikov's sixth power of k / r does leave
+// the normal floats far out (1e-49 at r = 1e8 M), in terms that are then below the last bit of
+// the sums they enter -- except for spins within 1e-6 of extremal, where the FP32 field is wrong
+// by hundreds of times itself either way.  Other scales and steps run
+// trace.cu's kernel.  One GB300: 500x400
 // Manko-Novikov frame of 20,000 steps 157 -> 142 ms, 301x211 Kerr shadow 306 -> 294 ms
 // (264 on some views), 24 Kerr cameras 332 -> 310, labels 281 -> 267, gated image 460 -> 424; a lone
 // Kerr warp 764 -> 686 cycles a step, Manko-Novikov on a full chip 1,470 -> 1,333.

@@ -224,3 +224,16 @@ def test_noalloc_takes_each_cameras_route(tracer, name):
     got, want = to_numpy(out), to_numpy(tracer.trace_batch(cams, 1500, 1e-3, 0))
     for k in got:
         assert np.array_equal(got[k], want[k], equal_nan=k in ("t", "r", "th", "ph")), k
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("sp", [1e-9, 1e-10, 1e-30, 2e-38])
+def test_mixed_mode_takes_steps_down_to_the_smallest_floats(tracer, sp):
+    """Ten steps of any length make ten of them in -t, to the precision of FP32 (and of the
+    denormals of 1e-38: 2^-149): a build that flushes them would leave t at zero."""
+    tracer.set_spacetime(0.5, 0.2, 0.0)
+    tracer.set_camera(10.0, 1.2, 75.0, 9, 7)
+    tracer.set_options()
+    got = to_numpy(tracer.trace(10, sp, 1))
+    assert np.all(got["status"] == 2)
+    assert np.max(np.abs(got["t"] + 10 * sp)) <= 1e-5 * 10 * sp + 100 * 2.0 ** -149
