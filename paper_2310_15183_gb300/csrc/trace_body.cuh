@@ -314,6 +314,42 @@ __device__ __noinline__ double rk4_step64_call(const SpacetimeC &st, const Ray64
     return rk4_step64<KIND>(st, x, sp, w6, y);
 }
 
+// A double-float step of an FP64 state, for the FP32 kernel with its zone inline (MODE 1).
+template <int KIND>
+__device__ __forceinline__ bool pair_step64(const PairSpacetime &c, const PairTables *tab, Ray64 &x,
+                                            TF sp, TF w6, double &h)
+{
+    RayTF T;
+    DF hd;
+    tf_state(x, T);
+    if (!pair_step<KIND>(c, tab, T, sp, w6, 0.0f, hd)) return false;
+    h = df_to(hd);
+    tf_unstate(T, x);
+    return true;
+}
+
+template <int KIND>
+__device__ __noinline__ bool pair_step64_call(const PairSpacetime &c, const PairTables *tab, Ray64 &x,
+                                              TF sp, TF w6, double &h)
+{
+    return pair_step64<KIND>(c, tab, x, sp, w6, h);
+}
+
+// What MODE 1 compiles of it, by its effect on the FP32 steps beside it: Kerr nothing (it has no
+// zone by default, MODE 1's only form; a ray at r < 0 takes FP64), cameras of both kinds a call,
+// Manko-Novikov the step itself.  gt_trace_batch_noalloc, FP32 steps alone: 40,000 Kerr rays x
+// 4,000 steps 5.41 ms (the step inline 9.09, a call 9.43), 16,000 of both kinds x 2,000 4.93 to
+// 5.26 (inline 5.23 to 5.36), 40,000 Manko-Novikov x 2,000 8.77 to 9.19 (a call 9.88); in the
+// zone, 12,000 Manko-Novikov rays x 1,000 steps 25 ms (a call 21).
+template <int KIND>
+__device__ __forceinline__ bool inline_zone_step(const PairSpacetime &c, const PairTables *tab, Ray64 &x,
+                                                 TF sp, TF w6, double &h)
+{
+    if constexpr (KIND == KIND_KERR) return false;
+    else if constexpr (KIND == KIND_ANY) return pair_step64_call<KIND>(c, tab, x, sp, w6, h);
+    else return pair_step64<KIND>(c, tab, x, sp, w6, h);
+}
+
 // ------------------------------------------------------------------ ring and redshift
 __device__ __forceinline__ bool in_disk(const DiskArgs &dk, double r, double th)
 {
@@ -650,7 +686,7 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A, int one_shot)
 {
     constexpr bool ZONE = MODE == 3 || MODE == 4;  // zone rays, parked when they leave
     constexpr bool PAIR = MODE == 4 || MODE == 5;  // three-float state, double-float step
-    constexpr bool TABLES = PAIR || MODE == 1;
+    constexpr bool TABLES = PAIR || (MODE == 1 && KIND != KIND_KERR);
     // per-ray spacetimes come with KIND_ANY only, and never to the double-float MODE 5
     const RayParams *const rays = KIND == KIND_ANY && MODE != 5 ? A.rays : nullptr;
     __shared__ PairTables tab_s[1];
@@ -985,13 +1021,9 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A, int one_shot)
             double h;
             bool ok = true;
             if ((double)m.r.hi < r_sw) { // the zone inline
-                DF hd;
                 mixed_to64(m, x);
-                tf_state(x, T);
-                if (A.zone_df && pair_step<KIND>(rays ? pr_ray : cams[cam].pair, tab, T, A.sp_tf,
-                                                 A.w6_tf, 0.0f, hd)) {
-                    h = df_to(hd);
-                    tf_unstate(T, x);
+                if (A.zone_df && inline_zone_step<KIND>(rays ? pr_ray : cams[cam].pair, tab, x, A.sp_tf,
+                                                        A.w6_tf, h)) {
                     mixed_from64(x, m);
                 } else {
                     Ray64 y;

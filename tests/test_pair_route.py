@@ -237,3 +237,33 @@ def test_mixed_mode_takes_steps_down_to_the_smallest_floats(tracer, sp):
     got = to_numpy(tracer.trace(10, sp, 1))
     assert np.all(got["status"] == 2)
     assert np.max(np.abs(got["t"] + 10 * sp)) <= 1e-5 * 10 * sp + 100 * 2.0 ** -149
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("kinds", ["kerr", "mn", "both"])
+def test_noalloc_mixed_steps_are_the_rounds_kernels_bits(tracer, kinds):
+    """The FP32 steps of gt_trace_batch_noalloc (a branch between stages, denormals kept) and of
+    gt_trace_batch (straight-line steps, denormals flushed, for cameras of both kinds the form
+    with the kind as the ray's own): one arithmetic, the same bits -- up to escape and horizon for
+    Kerr, outside the zone for Manko-Novikov (2000 steps of 1.5e-4 from r0 = 15)."""
+    import ctypes
+    torch = pytest.importorskip("torch")
+    from paper_2310_15183_gb300 import geotrace as g
+    from paper_2310_15183_gb300 import workloads as W
+    mn = [W.Camera(0.5, 0.24, 2.0, 15.0, 1.3, 75.0, 17, 9), W.Camera(0.5, 0.1, -1.0, 12.0, 0.8, 60.0, 8, 9)]
+    kerr = [W.Camera(0.5, 0.2, 0.0, 8.0, 1.2, 60.0, 17, 11), W.Camera(0.5, -0.24, 0.0, 12.0, 0.5, 75.0, 9, 8)]
+    cams = {"kerr": kerr, "mn": mn, "both": kerr + mn}[kinds]
+    steps, sp = (20000, 2e-3) if kinds == "kerr" else (2000, 1.5e-4)
+    descs = (g.CameraDesc * len(cams))(*[g.CameraDesc(c.M, c.S, c.Q, c.r0, c.theta0, c.fov_deg, c.res_x,
+                                                      c.res_y) for c in cams])
+    out = tracer.alloc_outputs(sum(c.n_rays for c in cams))
+    rc = g.load_library().gt_trace_batch_noalloc(
+        0, ctypes.c_void_p(torch.cuda.current_stream().cuda_stream), descs, len(cams), steps, sp, 1,
+        *[ctypes.c_void_p(out[k].data_ptr()) for k in ("t", "r", "th", "ph", "status", "nsteps")])
+    assert rc == 0
+    tracer.set_options()
+    got, want = to_numpy(out), to_numpy(tracer.trace_batch(cams, steps, sp, 1))
+    if kinds == "kerr":
+        assert set(got["status"]) >= {0, 1}
+    for k in got:
+        assert np.array_equal(got[k], want[k], equal_nan=k in ("t", "r", "th", "ph")), k
