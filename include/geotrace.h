@@ -107,7 +107,8 @@ typedef struct gt_ctx gt_ctx;
 typedef struct gt_options {
     int block_size;          /* threads per block, multiple of 32 in [32, 256] */
     int blocks_per_sm;       /* persistent grid = min(blocks_per_sm, resident limit) * SMs */
-                             /* (one of the two 0: 128 or 4; both 0: chosen by the launch) */
+                             /* (one of the two 0: 128 or 4; both 0: one-warp blocks, as many
+                              * as there are rays for, at most 16 per SM) */
     int flags;               /* GT_FLAG_* */
     int reproject_every;     /* FP32-mixed: steps between H = 0 re-projections; 0 = 4096 */
     double r_switch;         /* FP32-mixed: zone r < r_switch; < 0 = none; 0 = automatic:
@@ -370,12 +371,15 @@ int gt_trace_batch_noalloc(int device, void *cuda_stream, const gt_camera_desc *
                            double *theta, double *phi, uint8_t *status, uint32_t *nsteps);
 
 /* Autotuner: time gt_trace_range over `trial_rays` central pixels of the configured
- * camera for `trial_steps` steps with every candidate launch shape (block size in
- * {64, 128, 192, 256} x resident blocks per SM in {1, 2, 3, 4, 6, 8}, within the
- * kernel's occupancy limit, x rays per thread in {1, 2} for GT_MODE_FP32_MIXED), keep the
- * fastest in the context's options, and report it (best_rays_per_thread may be NULL).
+ * camera for `trial_steps` steps, by the kernel that calls of many steps take, with every
+ * candidate launch shape (block size in {64, 128, 192, 256} x resident blocks per SM in
+ * {1, 2, 3, 4, 6, 8}, within the kernel's occupancy limit, x rays per thread in {1, 2} for
+ * GT_MODE_FP32_MIXED) and with the default shape.  The fastest candidate is reported
+ * (best_rays_per_thread may be NULL) and kept in the context's options; where the default
+ * shape is faster than every candidate the options go back to it (zeros).
+ * best_steps_per_s is the rate of the shape kept.
  * With cache_path != NULL the result is looked up first and appended after tuning,
- * keyed by mode, spacetime kind, SM count and device name (plain text lines).
+ * keyed by mode, kernel, spacetime kind, SM count and device name (plain text lines).
  * Synchronous.  Errors: GT_ERR_NOT_CONFIGURED, GT_ERR_INVALID_ARG, GT_ERR_CUDA. */
 int gt_autotune(gt_ctx *ctx, int mode, int64_t trial_rays, int64_t trial_steps,
                 double step_precision, const char *cache_path, int *best_block,

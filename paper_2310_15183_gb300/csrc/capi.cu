@@ -34,6 +34,8 @@ struct gt_ctx {
     int cam_flags = -1;
     double cam_rsw = -2.0;
     CamDesc cam = {}; // the descriptor as set up on the device
+    // while gt_autotune runs its trials: the step count whose kernel they take (0: their own)
+    int64_t route_steps = 0;
     // batch descriptors (device)
     CamDesc *d_batch = nullptr;
     int batch_cap = 0;
@@ -164,8 +166,12 @@ int kind_for(int flags, int kind)
 
 gt::Routes camera_routes(const gt_ctx *c, double sp, int64_t n_steps)
 {
+    if (c->route_steps > n_steps) n_steps = c->route_steps;
     return gt::Routes(gt::routes_of(c->M, c->r0, sp, n_steps));
 }
+
+// Steps of a call long enough for every route that the camera and the step allow.
+constexpr int64_t ROUTE_OF_LONG_CALLS = (int64_t)1 << 40;
 
 // Ring, redshift output and state arrays of a launch (all optional).
 struct Extra {
@@ -1039,15 +1045,26 @@ int gt_autotune(gt_ctx *c, int mode, int64_t trial_rays, int64_t trial_steps, do
     if (!c->st_set || !c->cam_set) return GT_ERR_NOT_CONFIGURED;
     DeviceGuard g(c->device);
     if (!g.ok) return GT_ERR_CUDA;
-    const int kind = (c->Q != 0.0) ? gt::KIND_MN : gt::KIND_KERR;
+    const gt_options saved = c->opts;
+    // the kernel that long calls of this camera take, in the key and in the trials
+    const int kind =
+        kind_for(saved.flags, (c->Q != 0.0) ? gt::KIND_MN : gt::KIND_KERR);
+    const bool pair = !(saved.flags & PAPER_FLAGS) &&
+                      (gt::routes_of(c->M, c->r0, sp, ROUTE_OF_LONG_CALLS) & gt::ROUTE_PAIR);
+    const int kmode = mode != GT_MODE_FP64 ? gt::KMODE_MIXED_FP32
+                      : pair               ? gt::KMODE_FP64_PAIR
+                                           : gt::KMODE_FP64;
     cudaDeviceProp prop;
     if (cudaGetDeviceProperties(&prop, c->device) != cudaSuccess) return GT_ERR_CUDA;
     char key[256];
-    snprintf(key, sizeof key, "mode=%d kind=%d sms=%d dev=%s", mode, kind, c->sm_count, prop.name);
-    auto report = [&](int b, int k, int rpt, double v) {
-        c->opts.block_size = b;
-        c->opts.blocks_per_sm = k;
-        c->opts.rays_per_thread = rpt;
+    snprintf(key, sizeof key, "mode=%d kernel=%d kind=%d sms=%d dev=%s", mode, kmode, kind,
+             c->sm_count, prop.name);
+    // the fastest candidate is reported; `fixed` tells whether it is faster than the default
+    // shape too and so becomes the context's
+    auto report = [&](int b, int k, int rpt, double v, bool fixed) {
+        c->opts.block_size = fixed ? b : 0;
+        c->opts.blocks_per_sm = fixed ? k : 0;
+        c->opts.rays_per_thread = fixed ? rpt : 0;
         if (best_block) *best_block = b;
         if (best_blocks_per_sm) *best_blocks_per_sm = k;
         if (best_rays_per_thread) *best_rays_per_thread = rpt;
@@ -1059,15 +1076,16 @@ int gt_autotune(gt_ctx *c, int mode, int64_t trial_rays, int64_t trial_steps, do
         if (f) {
             char line[512];
             while (fgets(line, sizeof line, f)) {
-                int b = 0, k = 0, rpt = 1;
+                int b = 0, k = 0, rpt = 1, fixed = 1;
                 double v = 0;
                 char *bar = strchr(line, '|');
                 if (!bar) continue;
                 *bar = 0;
-                if (strcmp(line, key) == 0 && sscanf(bar + 1, "%d %d %d %lf", &b, &k, &rpt, &v) == 4 &&
-                    b >= 32 && b <= 256 && b % 32 == 0 && k >= 1 && k <= 64 && (rpt == 1 || rpt == 2)) {
+                if (strcmp(line, key) == 0 &&
+                    sscanf(bar + 1, "%d %d %d %lf %d", &b, &k, &rpt, &v, &fixed) == 5 && b >= 32 &&
+                    b <= 256 && b % 32 == 0 && k >= 1 && k <= 64 && (rpt == 1 || rpt == 2)) {
                     fclose(f);
-                    report(b, k, rpt, v);
+                    report(b, k, rpt, v, fixed != 0);
                     return GT_OK;
                 }
             }
@@ -1088,39 +1106,40 @@ int gt_autotune(gt_ctx *c, int mode, int64_t trial_rays, int64_t trial_steps, do
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
-    const gt_options saved = c->opts;
     const int blocks[] = {64, 128, 192, 256};
     const int per_sm[] = {1, 2, 3, 4, 6, 8};
     const int n_rpt = mode == GT_MODE_FP32_MIXED ? 2 : 1;
     int bb = 128, bk = 4, br = 1;
     double bv = -1.0;
     int rc = GT_OK;
+    c->route_steps = ROUTE_OF_LONG_CALLS;
+    auto trial = [&](int block, int blocks_per_sm, int rpt) { // steps per second
+        c->opts = saved;
+        c->opts.block_size = block;
+        c->opts.blocks_per_sm = blocks_per_sm;
+        c->opts.rays_per_thread = rpt;
+        c->opts.timeout_seconds = 0.0;
+        double best_ms = 1e300;
+        for (int rep = 0; rep < 2 && rc == GT_OK; rep++) {
+            cudaEventRecord(e0, c->stream);
+            rc = gt_trace_range(c, first, count, trial_steps, sp, mode, buf, buf + count,
+                                buf + 2 * count, buf + 3 * count, nullptr, ns);
+            cudaEventRecord(e1, c->stream);
+            if (cudaEventSynchronize(e1) != cudaSuccess) rc = GT_ERR_CUDA;
+            float ms = 0.f;
+            cudaEventElapsedTime(&ms, e0, e1);
+            if (rep > 0 && ms < best_ms) best_ms = ms; // first run warms up
+        }
+        return (double)count * (double)trial_steps / (best_ms * 1e-3);
+    };
     for (int rpt = 1; rpt <= n_rpt && rc == GT_OK; rpt++) {
         for (int bi = 0; bi < 4 && rc == GT_OK; bi++) {
-            const int kmode = mode == GT_MODE_FP64 ? gt::KMODE_FP64_PAIR : gt::KMODE_MIXED_FP32;
             const int fit = rpt == 2 ? gt::max_blocks_per_sm_two(kind, blocks[bi])
                                      : gt::max_blocks_per_sm(kmode, kind, blocks[bi]);
             for (int ki = 0; ki < 6 && rc == GT_OK; ki++) {
                 if (per_sm[ki] > fit) continue;
-                c->opts = saved;
-                c->opts.block_size = blocks[bi];
-                c->opts.blocks_per_sm = per_sm[ki];
-                c->opts.rays_per_thread = rpt;
-                c->opts.timeout_seconds = 0.0;
-                double best_ms = 1e300;
-                for (int rep = 0; rep < 2 && rc == GT_OK; rep++) {
-                    cudaEventRecord(e0, c->stream);
-                    rc = gt_trace_range(c, first, count, trial_steps, sp, mode, buf, buf + count,
-                                        buf + 2 * count, buf + 3 * count, nullptr, ns);
-                    cudaEventRecord(e1, c->stream);
-                    if (cudaEventSynchronize(e1) != cudaSuccess) rc = GT_ERR_CUDA;
-                    float ms = 0.f;
-                    cudaEventElapsedTime(&ms, e0, e1);
-                    if (rep > 0 && ms < best_ms) best_ms = ms; // first run warms up
-                }
-                if (rc != GT_OK) break;
-                const double v = (double)count * (double)trial_steps / (best_ms * 1e-3);
-                if (v > bv) {
+                const double v = trial(blocks[bi], per_sm[ki], rpt);
+                if (rc == GT_OK && v > bv) {
                     bv = v;
                     bb = blocks[bi];
                     bk = per_sm[ki];
@@ -1129,17 +1148,21 @@ int gt_autotune(gt_ctx *c, int mode, int64_t trial_rays, int64_t trial_steps, do
             }
         }
     }
+    const double v_default = rc == GT_OK ? trial(0, 0, 0) : 0.0;
+    c->route_steps = 0;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     cudaFree(buf);
     cudaFree(ns);
     c->opts = saved;
     if (rc != GT_OK) return rc;
-    report(bb, bk, br, bv);
+    const bool fixed = bv >= v_default;
+    const double v_kept = fixed ? bv : v_default;
+    report(bb, bk, br, v_kept, fixed);
     if (cache_path) {
         FILE *f = fopen(cache_path, "a");
         if (f) {
-            fprintf(f, "%s|%d %d %d %.6g\n", key, bb, bk, br, bv);
+            fprintf(f, "%s|%d %d %d %.6g %d\n", key, bb, bk, br, v_kept, fixed ? 1 : 0);
             fclose(f);
         }
     }

@@ -267,3 +267,40 @@ def test_noalloc_mixed_steps_are_the_rounds_kernels_bits(tracer, kinds):
         assert set(got["status"]) >= {0, 1}
     for k in got:
         assert np.array_equal(got[k], want[k], equal_nan=k in ("t", "r", "th", "ph")), k
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("mode", [0, 1])
+def test_autotuner_tunes_the_kernel_of_long_calls_and_compares_the_default(tracer, tmp_path, mode):
+    """Trials of few steps time the kernel that calls of many steps take, the cache's key names
+    it, and the line says whether the candidate beats the default shape; a shape cached for
+    another kernel is not taken; the tuned context is no slower than the default one."""
+    import time
+    torch = pytest.importorskip("torch")
+    tracer.set_options()
+    tracer.set_spacetime(0.5, 0.2, 0.0)
+    tracer.set_camera(10.0, 1.2, 75.0, 64, 64)
+
+    def pass_ms():
+        tracer.trace(2000, 1.5e-4, mode)
+        best = 1e9
+        for _ in range(5):
+            torch.cuda.synchronize()
+            t = time.perf_counter()
+            tracer.trace(2000, 1.5e-4, mode)
+            torch.cuda.synchronize()
+            best = min(best, time.perf_counter() - t)
+        return best
+
+    plain = pass_ms()
+    name = torch.cuda.get_device_name(0)
+    path = tmp_path / "tune.txt"
+    path.write_text("mode=%d kind=0 sms=%d dev=%s|256 1 1 1e30\n" % (mode, tracer.sm_count(), name))
+    shape = tracer.autotune(mode, trial_rays=4096, trial_steps=300, cache_path=str(path))
+    assert shape[3] < 1e20
+    lines = path.read_text().splitlines()
+    assert len(lines) == 2 and "kernel=%d" % (2 if mode else 5) in lines[1]
+    assert lines[1].split("|")[1].split()[4] in ("0", "1")
+    assert tracer.autotune(mode, trial_rays=4096, trial_steps=300, cache_path=str(path))[:3] == shape[:3]
+    assert pass_ms() <= 1.1 * plain
+    tracer.set_options()
