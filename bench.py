@@ -126,6 +126,28 @@ def measured_traffic(kernel: str, rays: int):
     return rec["dram_bytes_per_ray"] * rays
 
 
+# Warp instructions of one double-float RK4 step (profiles/kernels_short_counters.md).
+PAIR_STEP_INSTR = {"kerr": 2657, "mn": 9197}
+
+
+def fp64_takes_pairs(cam, wl) -> bool:
+    """Whether GT_MODE_FP64 traces this workload in double-float steps (geotrace.h, GT_MODE_FP64)."""
+    n, sp = wl.n_steps, wl.step_precision
+    return (1e-3 <= cam.M <= 1e3 and cam.r0 <= 1e5 and sp >= 1e-9 and n >= 1000
+            and sp <= 2e-3 * cam.M and sp * n >= 0.15 * cam.M
+            and cam.r0 <= min(0.03 * n, 1000.0) * cam.M)
+
+
+def trace_kernel_name(cam, wl, mixed: bool, rays_per_thread: int) -> str:
+    """The kernel that traces this workload's camera (trace.cu, trace_fp32.cu)."""
+    kind = 1 if cam.Q != 0 else 0
+    if not mixed:
+        return f"pair_kernel<5,{kind},1>" if fp64_takes_pairs(cam, wl) else f"trace_kernel<0,{kind},0>"
+    if rays_per_thread == 2:
+        return f"trace2_kernel<{kind},0>"
+    return f"trace_kernel<2,{kind},0,{kind}>"  # Manko-Novikov's constants as kernel parameters
+
+
 # ------------------------------------------------------------------ CPU oracle
 def oracle_rate(wl: W.Workload, target_s: float = 12.0, seed: int = 3) -> dict:
     """Time the FP64 oracle, as it stands, on a bounded pixel sample of the workload."""
@@ -903,25 +925,32 @@ def main():
     flops_per_step = counts[f"{kind}_step_flops_mixed" if mode else f"{kind}_step_flops"]
     kernel_s = t_dev / args.steps
     achieved = flops_per_step * steps_per_pass / kernel_s
-    if mode == geotrace.MODE_FP32_MIXED:
-        sms = tr.sm_count()
-        peak = sms * FP32_LANES_PER_SM * 2 * MAX_SM_MHZ * 1e6
-        peak_note = f"FP32 FMA: {sms} SMs x 128 lanes x 2 flop x 2070 MHz (derived)"
-        measured_peak = geotrace.measure_fma_peak(local, fp64=False)
-        kname = f"trace_kernel<2,{1 if cam.Q != 0 else 0},0,1>"
+    kname = trace_kernel_name(cam, wl, mode == geotrace.MODE_FP32_MIXED, launch["rays_per_thread"])
+    fp32_lanes = tr.sm_count() * FP32_LANES_PER_SM * MAX_SM_MHZ * 1e6  # lane instructions a second
+    if kname.startswith("pair_kernel"):
+        # the steps run on the FP32 pipes: their bound is the issue of their own instructions
+        achieved = PAIR_STEP_INSTR[kind] * steps_per_pass / kernel_s
+        roofline = {"bound": "alu", "achieved": achieved / 1e12, "peak": fp32_lanes / 1e12,
+                    "unit": "T lane instructions/s", "frac": achieved / fp32_lanes,
+                    "traffic": measured_traffic(kname, n), "kernel": kname,
+                    "peak_source": f"FP32 issue: {tr.sm_count()} SMs x 128 lanes x 2070 MHz (derived)",
+                    "instructions_per_rk4_step": PAIR_STEP_INSTR[kind],
+                    "fp64_flops_per_rk4_step": flops_per_step,
+                    "fp64_flops_over_nominal_fp64": flops_per_step * steps_per_pass / kernel_s / FP64_NOMINAL}
     else:
-        peak = FP64_NOMINAL
-        peak_note = ("FP64 dense 1.25 TFLOP/s (nominal); the steps run in double-float pairs on the "
-                     "FP32 pipes, so the fraction may exceed 1")
-        measured_peak = geotrace.measure_fma_peak(local, fp64=True, iters=200)
-        kname = f"pair_kernel<5,{1 if cam.Q != 0 else 0},1>"
-    roofline = {"bound": "alu", "achieved": achieved / 1e12, "peak": peak / 1e12,
-                "unit": "TFLOP/s", "frac": achieved / peak,
-                "traffic": measured_traffic(kname, n), "kernel": kname,
-                "peak_source": peak_note, "measured_fma_peak": measured_peak / 1e12,
-                "frac_of_measured_fma_peak": achieved / measured_peak,
-                "flops_per_rk4_step": flops_per_step,
-                "flop_convention": "add/mul 1, fma 2, div/rsqrt/exp 1, sincos 2 (opcount.cpp)"}
+        achieved = flops_per_step * steps_per_pass / kernel_s
+        fp64 = mode != geotrace.MODE_FP32_MIXED
+        peak = FP64_NOMINAL if fp64 else 2 * fp32_lanes
+        measured_peak = geotrace.measure_fma_peak(local, fp64=fp64, **({"iters": 200} if fp64 else {}))
+        roofline = {"bound": "alu", "achieved": achieved / 1e12, "peak": peak / 1e12,
+                    "unit": "TFLOP/s", "frac": achieved / peak,
+                    "traffic": measured_traffic(kname, n), "kernel": kname,
+                    "peak_source": "FP64 dense 1.25 TFLOP/s (nominal)" if fp64 else
+                    f"FP32 FMA: {tr.sm_count()} SMs x 128 lanes x 2 flop x 2070 MHz (derived)",
+                    "measured_fma_peak": measured_peak / 1e12,
+                    "frac_of_measured_fma_peak": achieved / measured_peak,
+                    "flops_per_rk4_step": flops_per_step,
+                    "flop_convention": "add/mul 1, fma 2, div/rsqrt/exp 1, sincos 2 (opcount.cpp)"}
 
     # ---------------- the CPU oracle on a bounded sample (rank 0, N = 1): the CPU baseline,
     # and the FP64 reference every GPU result of this workload is judged against
@@ -958,9 +987,13 @@ def main():
             "steps_per_s": s64 / t64, "rays_per_s": cnt / t64, "seconds": t64,
             "sample": "the whole image" if rows == cam.res_y else
                       f"{rows} central rows ({cnt} rays) of the same camera",
-            "arithmetic": "double-float pairs on the FP32 pipes, FP64 where their range ends",
-            "achieved_tflops": f64 * s64 / t64 / 1e12, "frac_of_fp64_nominal": f64 * s64 / t64 / FP64_NOMINAL,
-            "flops_per_rk4_step": f64}
+            "arithmetic": "double-float pairs on the FP32 pipes, FP64 where their precision ends"
+            if fp64_takes_pairs(cam, wl) else "FP64",
+            "fp64_flops_per_rk4_step": f64,
+            # work of FP64 steps over what the FP64 pipes could do: no roofline of pair steps
+            "fp64_flops_over_nominal_fp64": f64 * s64 / t64 / FP64_NOMINAL}
+        if fp64_takes_pairs(cam, wl):
+            modes["fp64_plain"]["frac_of_fp32_issue"] = PAIR_STEP_INSTR[kind] * s64 / t64 / fp32_lanes
         if acc_ref is not None and rows == cam.res_y:
             modes["fp64_plain"]["accuracy_vs_oracle"] = accuracy(host_sample(o64, acc_pix), acc_ref)
         modes.setdefault("fp32_mixed", {}).update(

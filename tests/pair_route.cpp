@@ -296,6 +296,8 @@ int main(int argc, char **argv)
 {
     const char *part = argc > 1 ? argv[1] : "";
     if (!strcmp(part, "accuracy")) accuracy(argc, argv);
+    if (!strcmp(part, "rule") && argc > 5)
+        printf("%d\n", pair_accurate(atof(argv[2]), atof(argv[3]), atof(argv[4]), atol(argv[5])));
     if (!strcmp(part, "new_state")) new_state();
     return 0;
 }

@@ -84,6 +84,24 @@ def test_fp64_mode_is_as_accurate_as_fp64_arithmetic_over_whole_paths(accuracy):
     assert r["pairs"] == WHOLE_PATHS[-1] and max(r["ratio"]) <= 1.25, r
 
 
+def test_benchmark_names_the_kernel_that_runs(host):
+    """bench.py's roofline is of the launched kernel: Manko-Novikov alone has its constants as
+    kernel parameters, two rays a thread are a kernel of their own, and GT_MODE_FP64 takes pairs
+    by the kernels' rule."""
+    import bench
+    from paper_2310_15183_gb300 import workloads as W
+    mn = W.WORKLOADS["mn1000"]
+    kerr = W.Camera(0.5, 0.2, 0.0, 15.0, 1.2, 75.0, 8, 8)
+    assert bench.trace_kernel_name(mn.camera, mn, True, 1) == "trace_kernel<2,1,0,1>"
+    assert bench.trace_kernel_name(kerr, mn, True, 1) == "trace_kernel<2,0,0,0>"
+    assert bench.trace_kernel_name(kerr, mn, True, 2) == "trace2_kernel<0,0>"
+    assert bench.trace_kernel_name(mn.camera, mn, False, 1) == "pair_kernel<5,1,1>"
+    for M, r0, sp, n in ((0.5, 15, 1.5e-4, 1000), (0.5, 15, 1.5e-4, 999), (0.5, 15.1, 1.5e-4, 1000),
+                         (0.5, 15, 1.01e-3, 20000), (0.5, 15, 1e-5, 5000), (0.5, 501, 1e-4, 10 ** 6)):
+        cam, wl = W.Camera(M, 0.0, 0.0, r0, 1.2, 75.0, 8, 8), W.Workload("x", None, n, sp)
+        assert bench.fp64_takes_pairs(cam, wl) == bool(host("rule", M, r0, sp, n)), (M, r0, sp, n)
+
+
 # ------------------------------------------------------------------ on the GPU
 # M, S, Q, r0, theta0, nx, ny, steps, step: calls that take FP64 steps
 FP64_CALLS = {
