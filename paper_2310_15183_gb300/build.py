@@ -50,7 +50,7 @@ def _stale() -> bool:
 
 def _compile(src: str) -> tuple:
     obj = os.path.join(BUILD, os.path.basename(src)[:-3] + ".o")
-    extra = os.environ.get("GT_NVCC_EXTRA", "").split()  # e.g. -DGT_FIELD_NOINLINE
+    extra = os.environ.get("GT_NVCC_EXTRA", "").split()
     extra = FILE_FLAGS.get(os.path.basename(src), []) + extra
     cmd = [nvcc()] + ARCH + FLAGS + extra + ["-c", src, "-o", obj]
     p = subprocess.run(cmd, capture_output=True, text=True)

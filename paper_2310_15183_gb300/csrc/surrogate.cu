@@ -15,7 +15,6 @@
 // backward products take plain BF16, whose range holds gradients scaled by 1/batch.
 // Accumulation is FP32 throughout.
 #include <cuda_bf16.h>
-#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>

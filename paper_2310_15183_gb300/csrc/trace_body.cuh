@@ -512,16 +512,8 @@ __device__ __forceinline__ void mixed_to64(const RayMixed &m, Ray64 &x)
     x.pph = m.pph;
 }
 
-// The FP32 field is evaluated 4 times per step; GT_FIELD_NOINLINE keeps one out-of-line
-// copy instead of four inlined ones (smaller code, fewer instruction-cache misses).
-#ifdef GT_FIELD_NOINLINE
-#define GT_FIELD_ATTR __noinline__
-#else
-#define GT_FIELD_ATTR __forceinline__
-#endif
-
 template <int KIND, bool PRECISE, bool OWN = false>
-__device__ GT_FIELD_ATTR void rates_f32(const SpacetimeF &st, float r, float s, float cs,
+__device__ __forceinline__ void rates_f32(const SpacetimeF &st, float r, float s, float cs,
                                           float pr, float pth, float pt, float pph,
                                           Rates<float> &o)
 {
