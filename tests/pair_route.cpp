@@ -292,9 +292,31 @@ static void accuracy(int argc, char **argv)
            sqrt(rms[1][1]), sqrt(rms[1][2]), sqrt(rms[1][3]), exp(lg[0]), exp(lg[1]), exp(lg[2]), exp(lg[3]));
 }
 
+// The operations over all that the step gives them: exp to the exponent bounds, in units of
+// 2^-45 + |x| 2^-47; sin/cos to the reduction's limit and the rotation by whole pairs, absolute.
+static void operations()
+{
+    LD w[3] = {};
+    for (int i = 0; i < 400000; i++) {
+        const DF x = df((LD)uni(-48, 48) + uni(-1, 1) * 1e-9L);
+        const LD want = expl(ld(x)), unit = ldexpl(1, -45) + fabsl(ld(x)) * ldexpl(1, -47);
+        w[0] = fmaxl(w[0], fabsl(ld(p_exp(x, &TAB)) - want) / want / unit);
+        const TF th = tf((LD)uni(-128, 128) + uni(-1, 1) * 1e-17L);
+        DF s, c, s2, c2;
+        p_sincos(tf_pair(th), th.c, &TAB, &s, &c);
+        w[1] = fmaxl(w[1], fmaxl(fabsl(ld(s) - sinl(ld(th))), fabsl(ld(c) - cosl(ld(th)))));
+        const DF d = df((LD)uni(-1, 1) * ldexpl(1, -9 - (int)uni(0, 30)) * (1 + uni(-1, 1) * 1e-8L));
+        p_rotate(s, c, d, &s2, &c2);
+        const LD a = atan2l(ld(s), ld(c)) + ld(d);
+        w[2] = fmaxl(w[2], fmaxl(fabsl(ld(s2) - sinl(a)), fabsl(ld(c2) - cosl(a))));
+    }
+    printf("{\"exp\": %.3e, \"sincos\": %.3e, \"rotate\": %.3e}\n", (double)w[0], (double)w[1], (double)w[2]);
+}
+
 int main(int argc, char **argv)
 {
     const char *part = argc > 1 ? argv[1] : "";
+    if (!strcmp(part, "operations")) operations();
     if (!strcmp(part, "accuracy")) accuracy(argc, argv);
     if (!strcmp(part, "rule") && argc > 5)
         printf("%d\n", pair_accurate(atof(argv[2]), atof(argv[3]), atof(argv[4]), atol(argv[5])));

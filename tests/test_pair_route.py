@@ -54,6 +54,13 @@ def test_a_step_whose_new_state_is_not_finite_is_refused(host):
     assert r["n"] == 64 and r["refused"] == r["untouched"] == r["taken"] == r["n"], r
 
 
+def test_operations_over_the_range_the_step_gives_them(host):
+    """exp: the argument's low part, at most 2^-24 |x|, is rounded three times (3 |x| 2^-49), the
+    series and the table cost 2^-45; sin/cos and the rotation as on their inner ranges, 2^-46."""
+    r = host("operations")
+    assert r["exp"] <= 1.0 and r["sincos"] <= 2.0 ** -46 and r["rotate"] <= 2.0 ** -46, r
+
+
 WHOLE_PATHS = (22000, 2e-3, 8.5, 25, 0.9, 1.5, 12)
 
 
