@@ -69,9 +69,9 @@ extern "C" {
                               * Manko-Novikov, are FP64's.  Rings, states and per-ray
                               * spacetimes take FP64 throughout: the same ray by gt_trace and
                               * by one of those agrees to rounding, not to the bit. */
-#define GT_MODE_FP32_MIXED 1 /* FP32 RK4 with compensated state; a zone r < r_switch stepped with
-                              * an FP64 state (its field and stage arithmetic in double-float
-                              * where the evaluation's range allows, else FP64) and H = 0
+#define GT_MODE_FP32_MIXED 1 /* FP32 RK4 with compensated state; a zone r < r_switch stepped in
+                              * double-float on a state of three floats per coordinate where the
+                              * evaluation's range allows, else in FP64; and H = 0
                               * re-projection.
                               * Runs in rounds (FP32 launch, zone launch, ...) and returns
                               * once the work has completed. */
@@ -272,7 +272,10 @@ int gt_surrogate_get_params(gt_surrogate *s, float *host, int64_t n);
 int gt_surrogate_set_params(gt_surrogate *s, const float *host, int64_t n);
 
 /* Network outputs for n samples (device float64 inputs) into `out` (device float32,
- * n x 4: logit, direction x, y, z).  Runs on the context's stream. */
+ * n x 4: logit, direction x, y, z).  Runs on the context's stream.  The products of a layer
+ * are summed in another order than in gt_surrogate_infer and in training: for the same
+ * inputs the two agree to the rounding of FP32 sums (5e-7 rms of the outputs), not to the
+ * bit, so a logit at a gate's threshold may lie on either side of it. */
 int gt_surrogate_eval(gt_ctx *ctx, gt_surrogate *s, int64_t n, const double *alpha,
                       const double *beta, const double *spin, const double *q,
                       const double *theta0, float *out);
@@ -350,7 +353,7 @@ int gt_surrogate_get_grads(gt_surrogate *s, float *host, int64_t n);
  * is not acceptable.  The paper has no counterpart.
  *
  * No context is needed and nothing is allocated: the queue counter and the camera
- * descriptors live in one static device array of the library (about 22 KB for
+ * descriptors live in one static device array of the library (about 28 KB for
  * GT_NOALLOC_MAX_CAMS cameras), which every device that loads the library holds until
  * the process exits.  The caller still owns and passes the device output arrays
  * (layout as gt_trace_batch; default launch options, no watchdog).  In FP32-mixed
@@ -406,8 +409,7 @@ int gt_device_sm_count(gt_ctx *ctx, int *out);
 int gt_measure_fma_peak(int device, int fp64, int iters, double *flops_per_s);
 
 /* BF16 tensor-core GEMM on `device` / `cuda_stream` (tcgen05, FP32 accumulation in
- * tensor memory), the building block of the surrogate network's training and
- * inference (which also runs it on FP16 operands internally):
+ * tensor memory), of the kind the surrogate network's own kernels are built from:
  * C[m, n] (+)= act(sum_k A[m, k] B[n, k] + bias[n]) for m < M, n < N.
  * A (m, k) is read at A[m * a_sm + k * a_sk] and B (n, k) at B[n * b_sn + k * b_sk]
  * (bf16 device arrays, any strides, so transposed views need no copy); bias is an

@@ -202,12 +202,12 @@ int prepare_camera(gt_ctx *c)
     return GT_OK;
 }
 
-// Block and grid of a launch.  A block size or a number of blocks per SM that the caller set
-// is taken as it is (with 128 threads or 4 blocks for the other one); by default a block is one warp, so that a launch of few rays spreads
-// warp by warp over all SMs (a grid of four-warp blocks puts 4,096 rays on 32 SMs: 10.2 ms
-// for 2,000 FP64 Schwarzschild steps against 4.2 ms on 128 SMs), and the persistent grid
-// has as many as the registers let an SM hold -- 16 for the FP32 and FP64 kernels -- but no
-// more than there are rays for.
+// Block and grid of a launch.  A block size or a number of blocks per SM that the caller set is
+// taken as it is (with 128 threads or 4 blocks for the other one).  By default a block is one
+// warp, so that a launch of few rays spreads warp by warp over all SMs (a grid of four-warp
+// blocks puts 4,096 rays on 32 SMs: 10.2 ms for 2,000 FP64 Schwarzschild steps against 4.2 ms on
+// 128 SMs), and the persistent grid has as many as the registers let an SM hold -- 16 for the
+// FP32 and FP64 kernels -- but no more than there are rays for.
 int launch_shape(gt_ctx *c, const gt_options &e, int kmode, int kind_hint, int64_t n_work,
                  bool one_shot, int *block, int *grid)
 {
@@ -1047,8 +1047,7 @@ int gt_autotune(gt_ctx *c, int mode, int64_t trial_rays, int64_t trial_steps, do
     if (!g.ok) return GT_ERR_CUDA;
     const gt_options saved = c->opts;
     // the kernel that long calls of this camera take, in the key and in the trials
-    const int kind =
-        kind_for(saved.flags, (c->Q != 0.0) ? gt::KIND_MN : gt::KIND_KERR);
+    const int kind = kind_for(saved.flags, (c->Q != 0.0) ? gt::KIND_MN : gt::KIND_KERR);
     const bool pair = !(saved.flags & PAPER_FLAGS) &&
                       (gt::routes_of(c->M, c->r0, sp, ROUTE_OF_LONG_CALLS) & gt::ROUTE_PAIR);
     const int kmode = mode != GT_MODE_FP64 ? gt::KMODE_MIXED_FP32

@@ -24,11 +24,12 @@
 // without that rounding.
 //
 // Measured against the FP64 kernel it replaces for GT_MODE_FP64 camera rays (one GB300): 48,000
-// Manko-Novikov rays x 2,000 steps 287 -> 40 ms (200,000 rays: 2.9e9 steps/s), Kerr 1.06e10
+// Manko-Novikov rays x 2,000 steps 287 -> 38.6 ms (200,000 rays: 2.9e9 steps/s), Kerr 1.06e10
 // steps/s; against the renormalised double-float zone step with an FP64 state, 40,000
-// in-zone rays x 4,000 steps 242 -> 80 ms.  Against long double the end positions of 2,000 to
-// 20,000 steps are off by 4e-17 to 1.6e-15 (t, r, theta, phi; relative 2-norm over a frame)
-// where FP64's are off by 1.1e-15 to 7e-15 (tests/pair_arith.cpp).
+// in-zone rays x 4,000 steps 242 -> 77.7 ms.  Against long double the end positions of 2,000 to
+// 20,000 steps of 3e-4 M are off by 4e-17 to 1.6e-15 (t, r, theta, phi; relative 2-norm over a
+// frame) where FP64's are off by 1.1e-15 to 7e-15 (tests/pair_arith.cpp).  That holds for many
+// small steps away from the axis: pair_accurate and PAIR_RHO_STEPS below draw the line.
 #pragma once
 
 #include <stdint.h>

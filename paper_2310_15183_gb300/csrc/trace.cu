@@ -104,7 +104,7 @@ cudaError_t launch_trace(const TraceArgs &args, int kmode, int kind_hint, int bl
     case KMODE_FP64: return launch_mode<0>(a, kind_hint, block, grid, one_shot, s);
     case KMODE_MIXED_INLINE: return launch_mode<1>(a, kind_hint, block, grid, one_shot, s);
     case KMODE_MIXED_FP32:
-        // outside the float range's middle, and for caller states, the build that keeps denormals
+        // for other scales and steps (ROUTE_FTZ), and for caller states, the build that keeps denormals
         return a.ftz ? launch_trace_fp32(a, kind_hint, block, grid, one_shot, s)
                      : launch_mode<2>(a, kind_hint, block, grid, one_shot, s);
     case KMODE_ZONE_FP64: return launch_mode<3>(a, kind_hint, block, grid, one_shot, s);
