@@ -768,7 +768,9 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A, int one_shot)
         return d.valid != 0;
     };
 
-    auto picked = [&](int c) { return !A.pick_mask || (cams[c].route & A.pick_mask) == A.pick; };
+    auto picked = [&](int c) {
+        return SINGLE || !A.pick_mask || (cams[c].route & A.pick_mask) == A.pick;
+    };
 
     // Start work item `w`; returns false when the ray is already finished and stored, or another
     // launch's.
