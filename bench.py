@@ -134,8 +134,8 @@ def fp64_takes_pairs(cam, wl) -> bool:
     """Whether GT_MODE_FP64 traces this workload in double-float steps (geotrace.h, GT_MODE_FP64)."""
     n, sp = wl.n_steps, wl.step_precision
     return (1e-3 <= cam.M <= 1e3 and cam.r0 <= 1e5 and sp >= 1e-9 and n >= 1000
-            and sp <= 2e-3 * cam.M and sp * n >= 0.15 * cam.M
-            and cam.r0 <= min(0.03 * n, 1000.0) * cam.M)
+            and sp <= 2e-3 * cam.M and sp * n >= max(0.15 * cam.M, 0.005 * cam.r0)
+            and cam.r0 <= min(0.05 * n, 1000.0) * cam.M)
 
 
 def trace_kernel_name(cam, wl, mixed: bool, rays_per_thread: int) -> str:

@@ -63,9 +63,9 @@ extern "C" {
                               * derivatives, double-float steps on a state of three floats per
                               * coordinate, where their end states are as close to the exact
                               * flow: M in [1e-3, 1e3], r0 <= 1e5, step >= 1e-9; n_steps >= 1000
-                              * steps of at most 2e-3 M that make at least 0.15 M together, and
-                              * r0 <= 1000 M and 0.03 M n_steps.  Their steps that start within
-                              * 1000 step lengths of the axis, or below r = 4M in
+                              * steps of at most 2e-3 M that make at least 0.15 M and 0.005 r0
+                              * together, and r0 <= 1000 M and 0.05 M n_steps.  Their steps that
+                              * start within 1000 step lengths of the axis, or below r = 4M in
                               * Manko-Novikov, are FP64's.  Rings, states and per-ray
                               * spacetimes take FP64 throughout: the same ray by gt_trace and
                               * by one of those agrees to rounding, not to the bit. */

@@ -587,15 +587,16 @@ constexpr float PAIR_MAX_EPSI = 48.0f;
 // change, and steps enough to average: t and phi start at zero, and after ten steps of any size
 // they are off by 6e-15 where FP64's are off by 1e-16.  Root-mean-square error over camera
 // frames of both kinds, spins 0 to 0.999, pair / FP64, worst of t, r, theta, phi:
-//   steps of 3e-4 M, r0 15-50 M:  500 steps 1.40, 700 1.15, 900 0.99, 1100 0.90, 2000 0.62;
+//   steps of 3e-4 M, r0 15-50 M:  500 steps 1.40, 700 1.15, 900 0.99, 1000 0.87, 2000 0.62;
 //   1000 steps, r0 8.5-60 M: of 1e-3 M 0.81, of 1e-4 M 1.17 (1500 of them: 0.79);
-//   2000 steps of 1e-4 M, r0 30-60 M: 0.55, 60-100 M: 1.17;  5000 steps, 100-400 M: 0.68;
+//   2000 steps of 1e-4 M, r0 30-60 M: 0.55, 60-100 M: 1.17 (5000, 80-100 M: 0.50);
+//   2000 steps of 3e-4 M, r0 60-100 M: 0.77;  8000 of 2.5e-4 M, 200-400 M: 0.38;
 //   whole paths, r0 8.5-30 M: steps of 2e-3 M 0.43, of 5e-3 M 1.34, of 0.2 M up to 25.
 inline bool pair_accurate(double M, double r0, double sp, int64_t n_steps)
 {
-    const double n = (double)n_steps;
-    return n_steps >= 1000 && sp <= 2e-3 * M && sp * n >= 0.15 * M && r0 <= 0.03 * M * n &&
-           r0 <= 1000.0 * M;
+    const double n = (double)n_steps, path = sp * n;
+    return n_steps >= 1000 && sp <= 2e-3 * M && path >= 0.15 * M && path >= 0.005 * r0 &&
+           r0 <= 0.05 * M * n && r0 <= 1000.0 * M;
 }
 
 // The same at the axis, where theta and phi change on the scale rho = r sin theta: steps from

@@ -21,8 +21,10 @@ ACCURACY = {
     "a few steps": (10, 3e-4, 15, 50, 0.3, 1.5, 24, False),
     "hundreds of steps": (500, 3e-4, 15, 50, 0.3, 1.5, 24, False),
     "fewest steps": (1000, 3e-4, 8.5, 30, 0.3, 1.5, 24, True),
+    "fewest steps, farthest camera": (1000, 3e-4, 30, 49, 0.3, 1.5, 24, True),
     "the workloads' step": (2000, 3e-4, 15, 60, 0.3, 1.5, 24, True),
-    "shortest path": (2000, 7.5e-5, 8.5, 60, 0.3, 1.5, 24, True),
+    "shortest path": (2000, 7.6e-5, 8.5, 30, 0.3, 1.5, 24, True),
+    "shortest path, far camera": (4000, 7.6e-5, 40, 60, 0.3, 1.5, 24, True),
     "too short a path": (2000, 1e-6, 8.5, 60, 0.3, 1.5, 24, False),
     "coarsest steps": (1000, 2e-3, 8.5, 30, 0.3, 1.5, 24, True),
     "coarse steps": (100, 0.2, 10, 30, 0.3, 1.5, 24, False),
@@ -103,7 +105,8 @@ def test_benchmark_names_the_kernel_that_runs(host):
     assert bench.trace_kernel_name(kerr, mn, True, 1) == "trace_kernel<2,0,0,0>"
     assert bench.trace_kernel_name(kerr, mn, True, 2) == "trace2_kernel<0,0>"
     assert bench.trace_kernel_name(mn.camera, mn, False, 1) == "pair_kernel<5,1,1>"
-    for M, r0, sp, n in ((0.5, 15, 1.5e-4, 1000), (0.5, 15, 1.5e-4, 999), (0.5, 15.1, 1.5e-4, 1000),
+    for M, r0, sp, n in ((0.5, 15, 1.5e-4, 1000), (0.5, 15, 1.5e-4, 999), (0.5, 25.1, 3e-4, 1000),
+                         (0.5, 25, 3e-4, 1000), (0.5, 20, 9.9e-5, 1000), (0.5, 20, 1.01e-4, 1000),
                          (0.5, 15, 1.01e-3, 20000), (0.5, 15, 1e-5, 5000), (0.5, 501, 1e-4, 10 ** 6)):
         cam, wl = W.Camera(M, 0.0, 0.0, r0, 1.2, 75.0, 8, 8), W.Workload("x", None, n, sp)
         assert bench.fp64_takes_pairs(cam, wl) == bool(host("rule", M, r0, sp, n)), (M, r0, sp, n)
@@ -117,7 +120,8 @@ FP64_CALLS = {
     "step above 2e-3 M": (0.5, 0.2, 0.0, 10.0, 1.2, 9, 7, 2000, 1.001e-3),
     "coarse steps": (0.5, 0.24, 2.0, 10.0, 1.2, 9, 7, 200, 0.3),
     "short path": (0.5, 0.2, 0.0, 10.0, 1.2, 9, 7, 1000, 7e-5),
-    "far camera": (0.5, 0.2, 0.0, 16.0, 1.2, 9, 7, 1000, 1.5e-4),
+    "far camera": (0.5, 0.2, 0.0, 25.1, 1.2, 9, 7, 1000, 3e-4),
+    "short path for the distance": (0.5, 0.2, 0.0, 20.0, 1.2, 9, 7, 1000, 9.9e-5),
     "large unit of length": (500.0, 1e5, 0.0, 10000.0, 1.2, 9, 7, 1000, 1.01),
 }
 
