@@ -306,6 +306,36 @@ __device__ __forceinline__ void tf_unstate(const RayTF &s, Ray64 &x)
 // The tables of pair.cuh, copied by each block into shared memory.
 __device__ const PairTables g_pair_tables = make_pair_tables();
 
+// The evolving coordinates of an FP64 state in the words of a three-float one, and back: a ray that
+// stays in FP64 for a while needs no registers of its own for it.
+__device__ __forceinline__ void hold64(double v, TF &t)
+{
+    t.a = __int_as_float(__double2loint(v));
+    t.b = __int_as_float(__double2hiint(v));
+}
+__device__ __forceinline__ double held64(TF t)
+{
+    return __hiloint2double(__float_as_int(t.b), __float_as_int(t.a));
+}
+__device__ __forceinline__ void hold64(const Ray64 &x, RayTF &s)
+{
+    hold64(x.t, s.t);
+    hold64(x.r, s.r);
+    hold64(x.th, s.th);
+    hold64(x.ph, s.ph);
+    hold64(x.pr, s.pr);
+    hold64(x.pth, s.pth);
+}
+__device__ __forceinline__ void held64(const RayTF &s, Ray64 &x)
+{
+    x.t = held64(s.t);
+    x.r = held64(s.r);
+    x.th = held64(s.th);
+    x.ph = held64(s.ph);
+    x.pr = held64(s.pr);
+    x.pth = held64(s.pth);
+}
+
 // The same step in FP64, out of line: the double-float kernels keep their registers.
 template <int KIND>
 __device__ __noinline__ double rk4_step64_call(const SpacetimeC &st, const Ray64 &x, double sp,
@@ -709,6 +739,14 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A, int one_shot)
     uint32_t n_f64 = 0;             // zone field evaluations of the ray in FP64 (this launch)
     PairSpacetime pr_ray;           // double-float constants of a per-ray spacetime
     RayTF T;                        // state of the double-float kernels
+    // A GT_MODE_FP64 ray that stays where pairs are refused -- below 4M, at the axis -- keeps its
+    // FP64 state: no conversion of twelve values a step (~72 instructions of the FP64 pipe beside
+    // the step's 1,343) and no refused pair step.  48,000 Manko-Novikov rays x 1,000 steps at 3.8M
+    // 138.8 -> 130.3 ms (the FP64 kernel: 143.6), 3,000 across 4M 266 -> 251, on the axis 151 ->
+    // 148.  Kerr refuses only at the axis (43.7 ms; the FP64 kernel 54.2), and the test in front of
+    // every step costs a lone Schwarzschild warp 4 %: left out there.
+    constexpr bool KEEP64 = MODE == 5 && KIND != KIND_KERR;
+    bool in64 = false; // T holds the FP64 state (hold64)
     uint32_t rp_next = 0xFFFFFFFFu; // next step count that is a multiple of reproject_every
     Ray64 x;
     RayMixed m;
@@ -840,6 +878,7 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A, int one_shot)
         n_entry = n;
         n_f64 = 0;
         if (PAIR) tf_state(x, T);
+        in64 = false;
         if (MODE == 1 || MODE == 2) {
             mixed_from64(x, m);
             if (A.reproject_every > 0) {
@@ -894,7 +933,8 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A, int one_shot)
             if (stop) {
                 if (active) {
                     if (MODE == 1 || MODE == 2) mixed_to64(m, x);
-                    if (PAIR) tf_unstate(T, x);
+                    if (PAIR && !in64) tf_unstate(T, x);
+                    if (PAIR && in64) held64(T, x);
                     store_full(A, id, x, GT_RAY_TIMEOUT, n, nan(""));
                 }
                 if (!one_shot) {
@@ -944,10 +984,9 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A, int one_shot)
             // GT_MODE_FP64 takes Manko-Novikov steps below 4M in FP64: next to the ergosurface
             // 1/A^2 amplifies the rounding of the field, where 48 bits show against 53
             const PairSpacetime &pc = SINGLE ? A.pair : rays ? pr_ray : cams[cam].pair;
-            const bool hard = MODE == 5 && KIND != KIND_KERR &&
-                              T.r.a - pc.r_plus.a < pc.r_hard;
-            // the zone's precision is the mixed mode's: steps up to the axis itself
+            // (the zone's precision is the mixed mode's: steps up to the axis itself)
             const float rho_min = MODE == 5 ? PAIR_RHO_STEPS * A.sp_tf.a : 0.0f;
+            const bool hard = KEEP64 && (in64 || T.r.a - pc.r_plus.a < pc.r_hard);
             DF h;
             ++n;
             if (!hard && pair_step<KIND>(pc, tab, T, A.sp_tf, A.w6_tf, rho_min, h)) {
@@ -964,7 +1003,10 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A, int one_shot)
                 if (status >= 0) tf_unstate(T, x);
             } else {
                 Ray64 y;
-                tf_unstate(T, x);
+                if (in64)
+                    held64(T, x);
+                else
+                    tf_unstate(T, x);
                 const double h64 = rk4_step64_call<KIND>(rays ? st : cams[cam].st, x, A.sp, A.w6, y);
                 n_f64 += 4;
                 if (!isfinite(h64) || !finite6(y)) {
@@ -975,7 +1017,13 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A, int one_shot)
                     if (MODE == 4 && A.disk.on && status != GT_RAY_ESCAPED &&
                         in_disk(A.disk, x.r, x.th))
                         status = GT_RAY_DISK;
-                    tf_state(x, T);
+                    const float r = (float)x.r;
+                    in64 = KEEP64 && (r - pc.r_plus.a < pc.r_hard ||
+                                      r * fabsf(__sinf((float)x.th)) < rho_min);
+                    if (in64)
+                        hold64(x, T);
+                    else
+                        tf_state(x, T);
                 }
             }
             if (ZONE && status < 0 && tf_greater(T.r, r_out_t)) { // leave the zone

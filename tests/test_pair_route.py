@@ -333,3 +333,42 @@ def test_autotuner_tunes_the_kernel_of_long_calls_and_compares_the_default(trace
     assert tracer.autotune(mode, trial_rays=4096, trial_steps=300, cache_path=str(path))[:3] == shape[:3]
     assert pass_ms() <= 1.1 * plain
     tracer.set_options()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("Q,r0,th0", [(2.0, 1.9, 1.2), (2.0, 10.0, 0.01), (0.0, 10.0, 0.01)])
+def test_a_ray_stopped_among_fp64_steps_reports_where_it_is(tracer, Q, r0, th0):
+    """Rays below 4M and at the axis keep an FP64 state between steps: stopped there by the
+    watchdog they report it.  A step makes -step of t, to the order of step^2."""
+    from paper_2310_15183_gb300 import geotrace as g
+    tracer.set_spacetime(0.5, 0.24, Q)
+    tracer.set_camera(r0, th0, 60.0, 32, 24)
+    out = tracer.alloc_outputs(32 * 24)
+    tracer.set_options(timeout_seconds=0.1)
+    with pytest.raises(g.GeotraceError) as e:
+        tracer.trace(1 << 31, 1.5e-4, 0, out)
+    assert e.value.code == -5
+    tracer.set_options()
+    got = to_numpy(out)
+    live = got["nsteps"].view(np.uint32) > 0
+    assert np.all(got["status"] == g.TIMEOUT) and live.sum() > 100
+    t = -1.5e-4 * got["nsteps"].view(np.uint32)
+    assert np.max(np.abs(got["t"][live] / t[live] - 1.0)) <= 1e-3
+    assert np.all((got["r"][live] > 1.0) & (got["r"][live] < 1.5 * r0))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("steps", [1000, 3000])
+@pytest.mark.parametrize("Q,r0,th0", [(2.0, 1.9, 1.2), (2.0, 2.05, 1.2), (2.0, 10.0, 0.05)])
+def test_rays_that_change_between_pairs_and_fp64(tracer, Q, r0, th0, steps):
+    """Rays below 4M, across it, and across the axis's line: the FP64 kernel's status, step count
+    and end position (1e-9, the project's parity tolerance), and the same bits for a ray in a
+    warp of its own."""
+    got, ref = _both(tracer, 0.5, 0.24, Q, r0, th0, 9, 7, steps, 3e-4 if r0 < 3 else 1e-3)
+    assert np.array_equal(got["status"], ref["status"]) and np.array_equal(got["nsteps"], ref["nsteps"])
+    for k in ("t", "r", "th"):
+        assert np.max(np.abs(got[k] - ref[k])) <= 1e-9 * np.max(np.abs(ref[k])), k
+    for i in (0, 31, 40):
+        one = to_numpy(tracer.trace_range(i, 1, steps, 3e-4 if r0 < 3 else 1e-3, 0))
+        for k in got:
+            assert np.array_equal(one[k], got[k][i:i + 1]), (k, i)
