@@ -127,7 +127,7 @@ def measured_traffic(kernel: str, rays: int):
 
 
 # Warp instructions of one double-float RK4 step (profiles/kernels_short_counters.md).
-PAIR_STEP_INSTR = {"kerr": 2662, "mn": 9199}
+PAIR_STEP_INSTR = {"kerr": 2662, "mn": 9203}
 
 
 def fp64_takes_pairs(cam, wl) -> bool:
